@@ -66,32 +66,33 @@ extern "C" {
 #define PTT_TIMEOUT (-4)   /* a bounded wait expired                             */
 #define PTT_ENOTSUP (-5)   /* valid request this library does not implement      */
 
-#define PTT_FP64 0         /* every step of the path in FP64                     */
+#define PTT_FP64 0         /* FP64: state, products, solves and sums in FP64; the
+                              Fourier and Chebyshev transforms between FP64
+                              arrays in 64-bit block fixed point (integers on a
+                              scale per line), at least as accurate as in FP64
+                              and several times faster: GB300's FP64 pipe runs
+                              at 1/64 of its FP32 pipe                         */
 #define PTT_MIXED 1        /* FP32 Fourier and Chebyshev transforms (FFTs; the
                               Chebyshev ones as DCT-II/III) and the products'
                               fluctuation parts (means and mean products in
-                              FP64, the mean column through double-single y
+                              FP64, the mean column through the FP64 form's y
                               passes); in 2D the explicit-term history and
                               its SBDF sum in FP32 (the mean mode's in FP64);
                               FP64 state and its SBDF sum, tau
                               solves and diagnostic sums (the energy's
                               transform in FP32, the Tr c and mid-plane
-                              transforms in double-single)                   */
+                              transforms as in the FP64 form)                  */
 #define PTT_MIXED_TC 2     /* as PTT_MIXED, with the Chebyshev transforms as dense
                               contractions on the tensor cores: BF16 slices of a
                               fixed-point split, FP32 accumulation (FP32 FFTs for
                               the shapes that contraction does not cover,
                               ny > 321); same accuracy as PTT_MIXED, slower on
                               this part at the shapes measured               */
-#define PTT_FP64_DS 3      /* FP64-accurate: the Fourier and Chebyshev transforms
-                              and the products in double-single arithmetic
-                              (each value the unevaluated sum of two FP32
-                              numbers, 48 significant bits) on the FP32 pipe;
-                              FP64 state, SBDF sums, tau solves and
-                              diagnostics.  Holds the FP64 path's bars against
-                              the FP64 solution (1e-11 after one step, 1e-9
-                              after 100); GB300's FP64 pipe is 1/64 of its
-                              FP32 pipe per instruction                      */
+#define PTT_FP64_DS 3      /* FP64-accurate: the kernels of PTT_FP64.  (The name is
+                              of an earlier form in pairs of FP32 numbers, which
+                              the fixed-point transforms are faster and more
+                              accurate than.)  A precision of its own: its
+                              members never share a group with PTT_FP64 ones   */
 
 /* Physical and numerical parameters of one member.  Defaults (the paper's
  * single fluid, Sec. 2): lx = lz = 10, re = 1e-2, wi = 150, beta = 0.9,

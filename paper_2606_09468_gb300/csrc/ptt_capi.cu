@@ -63,31 +63,174 @@ struct HostPlan {
   std::vector<int> radix;
 };
 
-// three_first: the padded x and z lengths (3K or more for K kept modes).
-// Their inverse lines are zero in the middle third [n/3, 2n/3), so a first
-// pass of radix 3 has one zero input (8 FP64 operations per butterfly
-// against 12); used where n has no factor 5.
-// wide: the plans of FP32 groups may take radix-8 passes (fewer passes,
-// each a shared-memory round trip; their transforms are bound by
-// instruction issue, not arithmetic); the FP64 plans keep radices up to 5,
-// whose tangent-form twiddles save FP64 operations, and so do the
-// double-single ones (measured slower with radix 8: register pressure).
-HostPlan make_plan(int n, bool three_first = false, bool wide = false) {
+// FP32 plans (mixed groups: the padded lengths and the energy grid), radices
+// 2 to 5 and 8 (few passes: each is a shared-memory round trip, and the
+// transforms are bound by instruction issue).  three_first: the padded x and z
+// lengths (3K or more for K kept modes), whose inverse lines are zero in the
+// middle third [n/3, 2n/3): a first pass of radix 3 has one zero input; used
+// where n has no factor 5.
+HostPlan make_plan(int n, bool three_first = false) {
   HostPlan p;
   p.n = n;
   int r = n;
   if (three_first && n % 3 == 0 && n % 5 != 0) { p.radix.push_back(3); r /= 3; }
-  // radix 5 first: the first pass takes no twiddles, and a twiddled radix-5
-  // butterfly costs the most (44 FP64 operations against 36 untwiddled)
-  // radices 13, 11, 7 (unpadded lengths only) first: their butterflies are
-  // the costliest, and the first pass takes no twiddles
-  for (int f : {13, 11, 7, 5})
-    while (r % f == 0) { p.radix.push_back(f); r /= f; }
-  if (wide)
-    while (r % 8 == 0) { p.radix.push_back(8); r /= 8; }
-  for (int f : {4, 2, 3})
+  // radix 5 first: the first pass takes no twiddles
+  for (int f : {5, 8, 4, 2, 3})
     while (r % f == 0) { p.radix.push_back(f); r /= f; }
   return p;
+}
+
+// Threads of the y and z kernels, which run their passes' butterflies at once
+// per group of lines: a plan's n / radix stays within them (fx_mb).
+constexpr int kFxPassThreads = 256;
+
+// Fixed-point plans: the factorisation of least estimated time per point, from
+// the cycles per warp of a butterfly (additions 2, products with a constant
+// 17, twiddles 55 per complex value) and about 35 per point and pass for the
+// shared-memory round trip and the indexes.  Primes 7, 11 and 13 (unpadded
+// lengths) take one pass each.  The first pass is an odd radix where there is
+// one: its stores are a radix apart, and even strides collide in the
+// shared-memory banks; three_first as above (radix 3 or 6).
+HostPlan make_plan_fx(int n, bool three_first = false) {
+  HostPlan p;
+  p.n = n;
+  int r = n;
+  std::vector<int> odd;
+  for (int f : {13, 11, 7})
+    while (r % f == 0) { odd.push_back(f); r /= f; }
+  const int rad[6] = {8, 6, 5, 4, 3, 2};
+  const double cost[6] = {103, 107, 121, 84, 94, 66};
+  std::vector<int> best, cur;
+  double bc = 1e30;
+  auto search = [&](auto&& self, int m, int from, double c) -> void {
+    if (c >= bc) return;
+    if (m == 1) { bc = c; best = cur; return; }
+    for (int i = from; i < 6; ++i)
+      if (m % rad[i] == 0 && n / rad[i] <= kFxPassThreads * fx_mb(rad[i])) {
+        cur.push_back(rad[i]);
+        self(self, m / rad[i], i, c + cost[i]);
+        cur.pop_back();
+      }
+  };
+  search(search, r, 0, 0.0);
+  auto lead = [&](int f) {
+    auto it = std::find(best.begin(), best.end(), f);
+    if (it == best.end()) return false;
+    best.erase(it);
+    p.radix.push_back(f);
+    return true;
+  };
+  if (three_first) { if (!lead(3)) lead(6); }
+  else if (odd.empty() && !lead(5)) lead(3);
+  p.radix.insert(p.radix.end(), odd.begin(), odd.end());
+  // then by size: the later passes' stores are contiguous
+  for (int f : {5, 3, 6, 4, 2, 8})
+    for (int b : best)
+      if (b == f) p.radix.push_back(f);
+  return p;
+}
+
+// cos and sin of 2 pi k / n in 62 fractional bits.  The first octant's angle
+// 2 pi q / (4n), q <= n/2, from FP64 z_0 and one Newton step of z^(4n) = 1:
+// z = z_0 (1 - (z_0^(4n) - 1)/(4n)), the power by squarings on 62 fractional
+// bits (its error, about 4n units, is divided by 4n again).
+struct FxRoots {
+  int n;
+  std::vector<long long> c, s;
+  std::vector<char> have;
+  explicit FxRoots(int n_) : n(n_), c(n_ / 2 + 1), s(n_ / 2 + 1), have(n_ / 2 + 1, 0) {}
+  static long long mul(long long a, long long b) {
+    return (long long)(((__int128)a * b + ((__int128)1 << 61)) >> 62);
+  }
+  void octant(long long q, long long* co, long long* si) {
+    if (!have[q]) {
+      const double th = 0.5 * kPi * (double)q / (double)n, one = 4611686018427387904.0;   // 2^62
+      const long long c0 = (long long)(std::cos(th) * one), s0 = (long long)(std::sin(th) * one);
+      const unsigned N = 4u * (unsigned)n;
+      long long x = c0, y = s0;
+      int bit = 31;
+      while (!((N >> bit) & 1u)) --bit;
+      for (--bit; bit >= 0; --bit) {
+        const long long x2 = mul(x, x) - mul(y, y), y2 = 2 * mul(x, y);
+        x = x2; y = y2;
+        if ((N >> bit) & 1u) {
+          const long long x3 = mul(x, c0) - mul(y, s0), y3 = mul(x, s0) + mul(y, c0);
+          x = x3; y = y3;
+        }
+      }
+      const long long ex = (x - (1LL << 62)) / (long long)N, ey = y / (long long)N;
+      c[q] = c0 - (mul(c0, ex) - mul(s0, ey));
+      s[q] = s0 - (mul(c0, ey) + mul(s0, ex));
+      have[q] = 1;
+    }
+    *co = c[q];
+    *si = s[q];
+  }
+  void at(long long k, long long* co, long long* si) {   // as cis
+    long long q = (4 * (k % n) + 4LL * n) % (4LL * n);
+    bool ns = false, nc = false, sw = false;
+    if (q > 2LL * n) { q = 4LL * n - q; ns = true; }
+    if (q > n) { q = 2LL * n - q; nc = true; }
+    if (2 * q > n) { q = n - q; sw = true; }
+    long long cc, ss;
+    octant(q, &cc, &ss);
+    if (sw) std::swap(cc, ss);
+    *co = nc ? -cc : cc;
+    *si = ns ? -ss : ss;
+  }
+};
+int4 fx_split(long long c, long long s) {
+  const int cl = (int)(unsigned)(unsigned long long)c, sl = (int)(unsigned)(unsigned long long)s;
+  return make_int4((int)((c - cl) >> 32), cl, (int)((s - sl) >> 32), sl);
+}
+
+// Offsets of the pass tables of a fixed-point plan (FftPlan::xoff); returns
+// the number of entries (at least 1).
+int fx_offsets(const HostPlan& hp, int* xoff) {
+  int off = 0, Ns = 1;
+  for (size_t s = 0; s < hp.radix.size(); ++s) {
+    xoff[s] = off;
+    if (s > 0) off += (hp.radix[s] - 1) * Ns;
+    Ns *= hp.radix[s];
+  }
+  return std::max(off, 1);
+}
+void fx_twiddles(const HostPlan& hp, std::vector<int4>& tab) {
+  int xoff[kMaxStages], Ns = 1;
+  tab.assign((size_t)fx_offsets(hp, xoff), make_int4(0, 0, 0, 0));
+  FxRoots root(hp.n);
+  for (size_t s = 0; s < hp.radix.size(); ++s) {
+    const int R = hp.radix[s];
+    if (s > 0)
+      for (int r = 1; r < R; ++r)
+        for (int jm = 0; jm < Ns; ++jm) {
+          long long cc, ss;
+          root.at((long long)jm * r * (hp.n / (Ns * R)), &cc, &ss);
+          tab[(size_t)xoff[s] + (size_t)(r - 1) * Ns + jm] = fx_split(cc, -ss);
+        }
+    Ns *= R;
+  }
+}
+// Quarter-period tables on M Gauss points (GroupDev::tw4Px, tw4Pix): inverse
+// exp(+i pi k/(2M)); forward h_k (2^e/D) exp(-i pi k/(2M)), h_0 = 1/2, h_k = 1, with
+// 2^e <= D < 2^(e+1).  Returns e.
+int fx_quarter_tables(int M, long long D, std::vector<int4>* fwd, std::vector<int4>* inv) {
+  int e = 0;
+  while ((2LL << e) <= D) ++e;
+  FxRoots root(4 * M);
+  if (fwd) fwd->resize(M);
+  if (inv) inv->resize(M);
+  for (int k = 0; k < M; ++k) {
+    long long c, s;
+    root.at(k, &c, &s);
+    if (inv) (*inv)[k] = fx_split(c, s);
+    if (fwd) {
+      const int sh = (k == 0) ? e - 1 : e;   // D >= M >= 14: e >= 3
+      auto scaled = [&](long long v) { return (long long)((((__int128)v << sh) + (v < 0 ? -D / 2 : D / 2)) / D); };
+      (*fwd)[k] = fx_split(scaled(c), -scaled(s));
+    }
+  }
+  return e;
 }
 
 // Quasi-tridiagonal operator tables of (alpha - beta D^2) a = R on the
@@ -330,13 +473,6 @@ void initial_fields3(const ptt_params& p, uint64_t seed, double amp, std::vector
 // points with each direction's constants folded in: fwd[k] = (s_k/2)
 // exp(-i pi k/(2M)) with s_0 = 1/M, s_k = 2/M (the DCT-II normalisation of
 // the coefficients), inv[k] = (1/2) exp(+i pi k/(2M)).
-// A complex double as double-single parts (re.h, re.l, im.h, im.l): h the FP32
-// rounding, l the FP32 rounding of the remainder (48 significant bits).
-float4 ds_split(double2 v) {
-  const float rh = (float)v.x, ih = (float)v.y;
-  return make_float4(rh, (float)(v.x - (double)rh), ih, (float)(v.y - (double)ih));
-}
-
 void quarter_tables(int M, std::vector<double2>& fwd, std::vector<double2>& inv) {
   fwd.resize(M);
   inv.resize(M);
@@ -346,82 +482,6 @@ void quarter_tables(int M, std::vector<double2>& fwd, std::vector<double2>& inv)
     const double h = (k == 0 ? 0.5 : 1.0) / M;
     fwd[k] = make_double2(h * cc, -h * ss);
     inv[k] = make_double2(0.5 * cc, 0.5 * ss);
-  }
-}
-
-// Record offsets of the tangent tables: toff[s] in records (tk), tto[s] in
-// doubles (tt); *nrec and *ndbl receive the table sizes (one spare entry).
-void tangent_offsets(const HostPlan& hp, int* toff, int* tto, int* nrec, int* ndbl) {
-  int rec = 0, dbl = 0, Ns = 1;
-  for (size_t st = 0; st < hp.radix.size(); ++st) {
-    const int R = hp.radix[st];
-    toff[st] = rec;
-    tto[st] = dbl;
-    if (st > 0 && R <= 5) {   // radices 7, 11, 13 keep plain twiddles
-      rec += Ns;
-      dbl += (R == 5 ? 16 : 6) * Ns;
-    }
-    Ns *= R;
-  }
-  *nrec = rec + 1;
-  *ndbl = dbl + 16;
-}
-
-// Tangent-form twiddle records of an FFT plan (see FftPlan): for each pass
-// s >= 1 (radix 2 to 5) and stride index jm < Ns, the forward twiddles
-// w_r = exp(-2 pi i m_r / n), m_r = jm r st, written as i^k_r c_r (1 + i t_r)
-// with k_r the nearest quarter turn, so that |angle of c_r + i c_r t_r| <=
-// pi/4 (c_r >= 1/sqrt 2, |t_r| <= 1).
-void tangent_tables(const HostPlan& hp, std::vector<double>& tt, std::vector<int>& tk) {
-  const int n = hp.n;
-  int toff[kMaxStages], tto[kMaxStages], nrec = 0, ndbl = 0;
-  tangent_offsets(hp, toff, tto, &nrec, &ndbl);
-  tt.assign((size_t)ndbl, 0.0);
-  tk.assign((size_t)nrec, 0);
-  double C1, S1, C2, S2;  // cos, sin of 2 pi/5 and 4 pi/5
-  cis(1, 5, &C1, &S1);
-  cis(2, 5, &C2, &S2);
-  int Ns = 1;
-  for (size_t st = 0; st < hp.radix.size(); ++st) {
-    const int R = hp.radix[st];
-    if (st > 0 && R <= 5) {
-      const long long stride = n / ((long long)Ns * R);
-      const int RS = (R == 5) ? 16 : 6;
-      for (int jm = 0; jm < Ns; ++jm) {
-        double c[5] = {1, 1, 1, 1, 1}, t[5] = {0, 0, 0, 0, 0};
-        int kp = 0;
-        for (int r = 1; r < R; ++r) {
-          const long long m = ((long long)jm * r * stride) % n;
-          // angle -2 pi m / n = 2 pi (-4 m) / (4 n); quarter turns k = round(-4 m / n)
-          long long k = -(4 * m + n / 2) / n;             // floor((-4 m + n/2) / n) for m >= 0
-          while (-4 * m - k * n > n / 2) ++k;
-          while (-4 * m - k * n < -(n / 2)) --k;
-          const long long e = -4 * m - k * n;             // reduced angle 2 pi e / (4 n)
-          double cc, ss;
-          cis(e, 4LL * n, &cc, &ss);
-          c[r] = cc;
-          t[r] = ss / cc;
-          kp |= (int)(((k % 4) + 4) % 4) << (2 * (r - 1));
-        }
-        double* rec = &tt[(size_t)tto[st] + (size_t)RS * jm];
-        if (R == 5) {
-          rec[0] = t[1]; rec[1] = t[2]; rec[2] = t[3]; rec[3] = t[4];
-          rec[4] = c[4] / c[1]; rec[5] = c[3] / c[2];
-          rec[6] = c[1]; rec[7] = c[2];
-          rec[8] = C1 * c[1]; rec[9] = C2 * c[2]; rec[10] = C2 * c[1]; rec[11] = C1 * c[2];
-          rec[12] = S1 * c[1]; rec[13] = S2 * c[2]; rec[14] = S2 * c[1]; rec[15] = S1 * c[2];
-        } else if (R == 4) {
-          rec[0] = t[1]; rec[1] = t[2]; rec[2] = t[3]; rec[3] = c[1]; rec[4] = c[2]; rec[5] = c[3] / c[1];
-        } else if (R == 3) {
-          rec[0] = t[1]; rec[1] = t[2]; rec[2] = c[1]; rec[3] = c[2] / c[1]; rec[4] = 0.5 * c[1];
-          rec[5] = 0.86602540378443864676 * c[1];
-        } else if (R == 2) {
-          rec[0] = t[1]; rec[1] = c[1];
-        }
-        tk[toff[st] + jm] = kp;
-      }
-    }
-    Ns *= R;
   }
 }
 
@@ -442,8 +502,10 @@ struct Group {
   int nx, ny, nz;
   std::vector<int> members;  // global member ids
   GroupDev d{};
+  int ds = 0;                // PTT_FP64_DS
   HostPlan hp[7];            // M, Mx, nx, Pu, Me, Mz, nz
-  HostPlan hpn;              // M with radices up to 5 (mixed groups: the mean column)
+  bool fx[7];                // fixed-point plan (else FP32)
+  HostPlan hpn;              // M in fixed point (mixed groups: the mean column)
 };
 
 int check_params(const ptt_params& p) {
@@ -483,38 +545,46 @@ void group_sizes(int nx, int ny, int nz, Group& g) {
   int Me = 2 * ny - 1;
   while ((Me & 1) || !smooth235(Me)) ++Me;
   d.Me = Me;
-  const size_t target = 96 * 1024;
-  auto cols = [&](int P) {
-    long long c = (long long)(target / smem_ycols(1, P, 0));
-    if (c < 1) c = 1;
-    if (c > 16) c = 16;
-    return (int)c;
+  // columns per block of the y passes: as many FP32 columns as 48 KB hold in
+  // two buffers, or fixed-point ones as leave three blocks an SM
+  auto cols = [&](bool fx, int P, int Nd) {
+    const long long c = fx ? 72 * 1024 / (long long)smem_ycols_fx(1, P, Nd) : 48 * 1024 / (long long)smem_ycols(1, P);
+    return (int)std::max(1LL, std::min(16LL, c));
   };
-  d.Ccol = cols(d.M);
-  d.CcolE = cols(d.Me);
-  d.CcolU = cols(d.Pu);
+  d.Ccol = cols(!d.f32, d.M, d.N);
+  d.CcolE = cols(!d.f32, d.Me, 0);
+  d.CcolU = cols(true, d.Pu, 0);
   d.xthreads = 512;   // launch-shape defaults (ptt_autotune may change them)
   d.zC = 8;
-  g.hp[0] = make_plan(d.M);
-  g.hp[1] = make_plan(d.Mx, true);
-  g.hp[2] = make_plan(nx);
-  g.hp[3] = make_plan(d.Pu);
-  g.hp[4] = make_plan(d.Me);
-  g.hp[5] = make_plan(d.Mz, true);
-  g.hp[6] = make_plan(nz);
 }
 
-// The plans of an FP32 group with radix-8 passes: those of the padded
-// lengths (M, Mx, Mz) and of the energy grid (Me), which only FP32 kernels
-// use in such groups.  The unpadded lengths (nx, 2 (ny - 1), nz) keep radices
-// up to 5 (and 7, 11, 13): the FP64 state transforms (set and get state, the
-// x synthesis of Tr c) and the double-single Tr c transforms use them.
-void wide_plans(Group& g) {
+// Plans of a group (d.f32 set): an FP32 group's padded lengths (M, Mx, Mz)
+// and energy grid (Me) in FP32, everything else in fixed point.
+void group_plans(Group& g) {
   const int n[7] = {g.d.M, g.d.Mx, g.d.nx, g.d.Pu, g.d.Me, g.d.Mz, g.d.nz};
   const bool three[7] = {false, true, false, false, false, true, false};
-  const bool widen[7] = {true, true, false, false, true, true, false};
-  for (int i = 0; i < 7; ++i)
-    if (widen[i]) g.hp[i] = make_plan(n[i], three[i], true);
+  const bool padded[7] = {true, true, false, false, true, true, false};
+  for (int i = 0; i < 7; ++i) {
+    g.fx[i] = !(g.d.f32 && padded[i]);
+    g.hp[i] = g.fx[i] ? make_plan_fx(n[i], three[i]) : make_plan(n[i], three[i]);
+  }
+  g.hpn = make_plan_fx(g.d.M);
+  if (!g.d.f32) g.d.xthreads = 256;
+}
+
+// Least threads per block of the plan's passes.
+int fx_min_threads(const HostPlan& hp) {
+  int t = 32;
+  for (int R : hp.radix) t = std::max(t, (hp.n / R + fx_mb(R) - 1) / fx_mb(R));
+  return (t + 31) & ~31;
+}
+
+void set_plan(FftPlan& pl, const HostPlan& hp) {
+  pl.n = hp.n;
+  pl.nst = (int)hp.radix.size();
+  for (int s = 0; s < pl.nst; ++s) pl.radix[s] = hp.radix[s];
+  plan_pass_consts(pl);
+  fx_offsets(hp, pl.xoff);
 }
 
 // Carve (or, with base == nullptr, size) all device arrays.
@@ -603,38 +673,21 @@ void carve(std::vector<Group>& groups, Carver& cv) {
     d.stageS = cv.take<double2>((size_t)nf * NK);
     FftPlan* pls[7] = {&d.plP, &d.plMx, &d.plNx, &d.plPu, &d.plPe, &d.plMz, &d.plNz};
     for (int i = 0; i < 7; ++i) {
-      pls[i]->n = g.hp[i].n;
-      pls[i]->nst = (int)g.hp[i].radix.size();
-      for (int s = 0; s < pls[i]->nst; ++s) pls[i]->radix[s] = g.hp[i].radix[s];
-      plan_pass_consts(*pls[i]);
-      pls[i]->tw = cv.take<double2>((size_t)g.hp[i].n);
-      // single-precision tables: the step's padded lengths and the energy grid
-      pls[i]->twf = (d.f32 && (i < 2 || i == 4 || i == 5)) ? cv.take<float2>((size_t)g.hp[i].n) : nullptr;
-      // double-single tables: every length of a double-single group; the
-      // unpadded y and z lengths of a mixed group (its Tr c transforms)
-      pls[i]->twd = (d.ds || (d.f32 && (i == 0 || i == 3 || i == 6))) ? cv.take<float4>((size_t)g.hp[i].n)
-                                                                   : nullptr;
-      int nrec = 0, ndbl = 0;
-      tangent_offsets(g.hp[i], pls[i]->toff, pls[i]->tto, &nrec, &ndbl);
-      pls[i]->tt = cv.take<double>((size_t)ndbl);
-      pls[i]->tk = cv.take<int>((size_t)nrec);
+      set_plan(*pls[i], g.hp[i]);
+      pls[i]->twf = g.fx[i] ? nullptr : cv.take<float2>((size_t)g.hp[i].n);
+      int xoff[kMaxStages];
+      pls[i]->twx = g.fx[i] ? cv.take<int4>((size_t)fx_offsets(g.hp[i], xoff)) : nullptr;
     }
-    d.tw4P = cv.take<double2>((size_t)d.M);
+    set_plan(d.plPn, g.hpn);
+    d.plPn.twf = nullptr;
+    int xoff[kMaxStages];
+    d.plPn.twx = d.f32 ? cv.take<int4>((size_t)fx_offsets(g.hpn, xoff)) : nullptr;
     d.tw4Pf = d.f32 ? cv.take<float2>((size_t)d.M) : nullptr;
-    d.tw4Pi = cv.take<double2>((size_t)d.M);
     d.tw4Pif = d.f32 ? cv.take<float2>((size_t)d.M) : nullptr;
-    d.tw4E = cv.take<double2>((size_t)d.Me);
     d.tw4Ef = d.f32 ? cv.take<float2>((size_t)d.Me) : nullptr;
-    d.tw4Pd = (d.ds || d.f32) ? cv.take<float4>((size_t)d.M) : nullptr;
-    d.tw4Pid = (d.ds || d.f32) ? cv.take<float4>((size_t)d.M) : nullptr;
-    // mixed groups: the narrow plan of M shares plP's tables
-    d.plPn = d.plP;
-    if (d.f32) {
-      d.plPn.nst = (int)g.hpn.radix.size();
-      for (int s = 0; s < d.plPn.nst; ++s) d.plPn.radix[s] = g.hpn.radix[s];
-      plan_pass_consts(d.plPn);
-    }
-    d.tw4Ed = d.ds ? cv.take<float4>((size_t)d.Me) : nullptr;
+    d.tw4Px = cv.take<int4>((size_t)d.M);
+    d.tw4Pix = cv.take<int4>((size_t)d.M);
+    d.tw4Ex = d.f32 ? nullptr : cv.take<int4>((size_t)d.Me);
   }
 }
 
@@ -650,10 +703,10 @@ std::vector<Group> make_groups(const ptt_params* pm, int nmem) {
       g.nx = pm[i].nx;
       g.ny = pm[i].ny;
       g.nz = pm[i].nz;
-      group_sizes(g.nx, g.ny, g.nz, g);
       g.d.f32 = (pm[i].precision == PTT_MIXED || pm[i].precision == PTT_MIXED_TC) ? 1 : 0;
-      g.d.ds = (pm[i].precision == PTT_FP64_DS) ? 1 : 0;
-      if (g.d.f32) { g.hpn = g.hp[0]; wide_plans(g); }
+      group_sizes(g.nx, g.ny, g.nz, g);
+      g.ds = (pm[i].precision == PTT_FP64_DS) ? 1 : 0;
+      group_plans(g);
       g.d.ymma = (pm[i].precision == PTT_MIXED_TC) ? 1 : 0;   // requested; carve() checks the shape
       groups.push_back(std::move(g));
       it = idx.find(key);
@@ -669,7 +722,7 @@ std::vector<Group> make_groups(const ptt_params* pm, int nmem) {
 bool multi_eligible(const std::vector<Group>& groups) {
   if (groups.size() < 2 || (int)groups.size() > multi2d_max_groups()) return false;
   for (const Group& g : groups)
-    if (g.d.nz != 1 || g.d.ymma || g.d.f32 != groups[0].d.f32 || g.d.ds != groups[0].d.ds) return false;
+    if (g.d.nz != 1 || g.d.ymma || g.d.f32 != groups[0].d.f32 || g.ds != groups[0].ds) return false;
   return true;
 }
 
@@ -724,9 +777,8 @@ void set_last_error(const char* msg) {
   std::snprintf(g_last_error, sizeof(g_last_error), "%s", msg);
 }
 
-int shape_plan(const ptt_params& p, GroupDev& d, std::vector<double2>& twP,
-               std::vector<double2>& twMx, std::vector<double2>& tw4, MemberPrm& prm,
-               std::vector<double>* tt, std::vector<int>* tk) {
+int shape_plan(const ptt_params& p, GroupDev& d, std::vector<int4>& tables, size_t (&off)[4],
+               MemberPrm& prm) {
   const int s = check_params(p);
   if (s) return s;
   if (p.precision != PTT_FP64) return PTT_ENOTSUP;
@@ -736,34 +788,22 @@ int shape_plan(const ptt_params& p, GroupDev& d, std::vector<double2>& twP,
   g.ny = p.ny;
   g.nz = 1;
   group_sizes(p.nx, p.ny, 1, g);
+  group_plans(g);
   d = g.d;
   d.nb = 1;
   // columns per block as carve() caps them for one member
   d.Ccol = std::max(1, std::min(d.Ccol, (int)((long long)d.KZ * 9 / 304)));
-  FftPlan* pls[2] = {&d.plP, &d.plMx};
-  std::vector<double2>* tws[2] = {&twP, &twMx};
-  for (int i = 0; i < 2; ++i) {
-    const HostPlan& hp = g.hp[i];
-    pls[i]->n = hp.n;
-    pls[i]->nst = (int)hp.radix.size();
-    for (int k = 0; k < pls[i]->nst; ++k) pls[i]->radix[k] = hp.radix[k];
-    plan_pass_consts(*pls[i]);
-    // tangent-form twiddle records of the FP64 passes (device pointers are
-    // set by the caller once the tables have a home)
-    int nrec = 0, ndbl = 0;
-    tangent_offsets(hp, pls[i]->toff, pls[i]->tto, &nrec, &ndbl);
-    tangent_tables(hp, tt[i], tk[i]);
-    tws[i]->resize(hp.n);
-    for (int k = 0; k < hp.n; ++k) {
-      double cc, ss;
-      cis(k, hp.n, &cc, &ss);
-      (*tws[i])[k] = make_double2(cc, -ss);
-    }
+  set_plan(d.plP, g.hp[0]);
+  set_plan(d.plMx, g.hp[1]);
+  std::vector<int4> part[4];
+  fx_twiddles(g.hp[0], part[0]);
+  fx_twiddles(g.hp[1], part[1]);
+  d.fexpP = fx_quarter_tables(d.M, (long long)d.M * d.Mx, &part[2], &part[3]);
+  tables.clear();
+  for (int i = 0; i < 4; ++i) {
+    off[i] = tables.size();
+    tables.insert(tables.end(), part[i].begin(), part[i].end());
   }
-  // tw4: the forward table of the Gauss-grid transforms, then the inverse one
-  std::vector<double2> inv;
-  quarter_tables(d.M, tw4, inv);
-  tw4.insert(tw4.end(), inv.begin(), inv.end());
   member_prm(p, prm);
   return PTT_OK;
 }
@@ -944,7 +984,7 @@ int ptt_create(const ptt_params* pm, int32_t nmem, void* d_ws, size_t bytes, voi
   for (Group& g : c->groups) {
     if (g.d.nz == 1 && (smem_xfused(g.d.Mx, g.d.f32) > (size_t)optin || smem_spec(g.d.N) > (size_t)optin))
       return PTT_EINVAL;
-    if (g.d.nz > 1 && (smem_xfused3(g.d.Mx, g.d.f32) == 0 || smem_xfused3(g.d.Mx, g.d.f32) > (size_t)optin))
+    if (g.d.nz > 1 && (smem_xfused3(g.d.Mx, g.d.f32) == 0 || smem_xfused3(g.d.Mx, g.d.f32) + 2048 > (size_t)optin))
       return PTT_EINVAL;
   }
   CK(set_kernel_attributes(optin));
@@ -1058,72 +1098,57 @@ int ptt_create(const ptt_params* pm, int32_t nmem, void* d_ws, size_t bytes, voi
       }
       CK(cudaMemcpyAsync((void*)d.ccw, cw.data(), cw.size() * 8, cudaMemcpyHostToDevice, c->stream));
     }
-    // quarter-period twiddles of the Gauss-grid transforms (forward and
-    // inverse on the padded grid, inverse on the diagnostic grid)
-    {
+    // quarter-period twiddles of the Gauss-grid transforms and the FFT plans'
+    // twiddles
+    auto up = [&](const void* dst, const void* src, size_t bytes) {
+      return cudaMemcpyAsync(const_cast<void*>(dst), src, bytes, cudaMemcpyHostToDevice, c->stream);
+    };
+    if (d.f32) {
       std::vector<double2> fwd, inv, fwdE, invE;
       quarter_tables(d.M, fwd, inv);
       quarter_tables(d.Me, fwdE, invE);
       const std::vector<double2>* src[3] = {&fwd, &inv, &invE};
-      const double2* dst[3] = {d.tw4P, d.tw4Pi, d.tw4E};
-      const float2* dstf[3] = {d.tw4Pf, d.tw4Pif, d.tw4Ef};
-      const float4* dstd[3] = {d.tw4Pd, d.tw4Pid, d.tw4Ed};
-      std::vector<float2> twf[3];
-      std::vector<float4> twd[3];
+      const float2* dst[3] = {d.tw4Pf, d.tw4Pif, d.tw4Ef};
       for (int t = 0; t < 3; ++t) {
-        const std::vector<double2>& tw = *src[t];
-        CK(cudaMemcpyAsync((void*)dst[t], tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice,
-                           c->stream));
-        if (dstf[t]) {
-          twf[t].resize(tw.size());
-          for (size_t k = 0; k < tw.size(); ++k) twf[t][k] = make_float2((float)tw[k].x, (float)tw[k].y);
-          CK(cudaMemcpyAsync((void*)dstf[t], twf[t].data(), twf[t].size() * sizeof(float2),
-                             cudaMemcpyHostToDevice, c->stream));
-        }
-        if (dstd[t]) {
-          twd[t].resize(tw.size());
-          for (size_t k = 0; k < tw.size(); ++k) twd[t][k] = ds_split(tw[k]);
-          CK(cudaMemcpyAsync((void*)dstd[t], twd[t].data(), twd[t].size() * sizeof(float4),
-                             cudaMemcpyHostToDevice, c->stream));
-        }
-      }
-      CK(cudaStreamSynchronize(c->stream));
-    }
-    // twiddle tables
-    FftPlan* pls[7] = {&d.plP, &d.plMx, &d.plNx, &d.plPu, &d.plPe, &d.plMz, &d.plNz};
-    for (int t = 0; t < 7; ++t) {
-      const int n = pls[t]->n;
-      std::vector<double2> tw(n);
-      for (int k = 0; k < n; ++k) {
-        double cc, ss;
-        cis(k, n, &cc, &ss);
-        tw[k] = make_double2(cc, -ss);
-      }
-      CK(cudaMemcpyAsync((void*)pls[t]->tw, tw.data(), n * sizeof(double2), cudaMemcpyHostToDevice, c->stream));
-      {
-        std::vector<double> tt;
-        std::vector<int> tk;
-        tangent_tables(g.hp[t], tt, tk);
-        CK(cudaMemcpyAsync((void*)pls[t]->tt, tt.data(), tt.size() * sizeof(double),
-                           cudaMemcpyHostToDevice, c->stream));
-        CK(cudaMemcpyAsync((void*)pls[t]->tk, tk.data(), tk.size() * sizeof(int),
-                           cudaMemcpyHostToDevice, c->stream));
+        std::vector<float2> twf;
+        for (const double2& v : *src[t]) twf.push_back(make_float2((float)v.x, (float)v.y));
+        CK(up(dst[t], twf.data(), twf.size() * sizeof(float2)));
         CK(cudaStreamSynchronize(c->stream));
       }
-      if (pls[t]->twf) {
-        std::vector<float2> twf(n);
-        for (int k = 0; k < n; ++k) twf[k] = make_float2((float)tw[k].x, (float)tw[k].y);
-        CK(cudaMemcpyAsync((void*)pls[t]->twf, twf.data(), n * sizeof(float2), cudaMemcpyHostToDevice,
-                           c->stream));
-      }
-      std::vector<float4> twd;
-      if (pls[t]->twd) {
-        twd.resize(n);
-        for (int k = 0; k < n; ++k) twd[k] = ds_split(tw[k]);
-        CK(cudaMemcpyAsync((void*)pls[t]->twd, twd.data(), n * sizeof(float4), cudaMemcpyHostToDevice,
-                           c->stream));
-      }
+    }
+    {
+      // the FP64 step's x and z passes leave their normalisation to the
+      // forward y table; a mixed group's mean column carries its own
+      std::vector<int4> fwd, inv;
+      d.fexpP = fx_quarter_tables(d.M, d.f32 ? (long long)d.M : (long long)d.M * d.Mx * d.Mz, &fwd, &inv);
+      CK(up(d.tw4Px, fwd.data(), fwd.size() * sizeof(int4)));
+      CK(up(d.tw4Pix, inv.data(), inv.size() * sizeof(int4)));
       CK(cudaStreamSynchronize(c->stream));
+      if (d.tw4Ex) {
+        fx_quarter_tables(d.Me, d.Me, nullptr, &inv);
+        CK(up(d.tw4Ex, inv.data(), inv.size() * sizeof(int4)));
+        CK(cudaStreamSynchronize(c->stream));
+      }
+    }
+    FftPlan* pls[8] = {&d.plP, &d.plMx, &d.plNx, &d.plPu, &d.plPe, &d.plMz, &d.plNz, &d.plPn};
+    const HostPlan* hps[8] = {&g.hp[0], &g.hp[1], &g.hp[2], &g.hp[3], &g.hp[4], &g.hp[5], &g.hp[6], &g.hpn};
+    for (int t = 0; t < 8; ++t) {
+      if (pls[t]->twf) {
+        std::vector<float2> twf(hps[t]->n);
+        for (int k = 0; k < hps[t]->n; ++k) {
+          double cc, ss;
+          cis(k, hps[t]->n, &cc, &ss);
+          twf[k] = make_float2((float)cc, (float)-ss);
+        }
+        CK(up(pls[t]->twf, twf.data(), twf.size() * sizeof(float2)));
+        CK(cudaStreamSynchronize(c->stream));
+      }
+      if (pls[t]->twx) {
+        std::vector<int4> tab;
+        fx_twiddles(*hps[t], tab);
+        CK(up(pls[t]->twx, tab.data(), tab.size() * sizeof(int4)));
+        CK(cudaStreamSynchronize(c->stream));
+      }
     }
     CK(cudaStreamSynchronize(c->stream));
   }
@@ -1418,12 +1443,13 @@ int ptt_autotune(ptt_ctx* c, int32_t* choices, int32_t max_groups) {
   for (size_t gi = 0; gi < c->groups.size(); ++gi) {
     GroupDev& d = c->groups[gi].d;
     const bool d3 = d.nz > 1;
-    // threads per block of the fused x pass (stage 1); the in-place 3D
-    // form runs 512
-    if (!(d3 && xfused3_inplace(d.Mx, d.f32))) {
+    // threads per block of the fused x pass (stage 1)
+    {
       int best = d.xthreads;
       float bt = 1e30f;
-      for (int t = 128; t <= 512; t += 64) {
+      // the fixed-point 2D kernel takes at most 256
+      const int lo = d.f32 ? 128 : std::max(128, fx_min_threads(c->groups[gi].hp[1]));
+      for (int t = lo; t <= (d.f32 || d3 ? 512 : 256); t += 64) {
         d.xthreads = t;
         float ms = 0;
         int s = time_stages_of(c, d, 1, 1, reps, &ms);
@@ -1439,7 +1465,7 @@ int ptt_autotune(ptt_ctx* c, int32_t* choices, int32_t max_groups) {
       int best = d.Ccol;
       float bt = 1e30f;
       for (int C : cand) {
-        if (smem_ycols(C, d.M, d.f32) > (size_t)optin) continue;
+        if ((d.f32 ? smem_ycols(C, d.M) : smem_ycols_fx(C, d.M, d.N)) + 2048 > (size_t)optin) continue;
         d.Ccol = C;
         float ms = 0;
         int s = time_stages_of(c, d, 0, 2, reps, &ms);
@@ -1458,7 +1484,7 @@ int ptt_autotune(ptt_ctx* c, int32_t* choices, int32_t max_groups) {
       int best = cc;
       float bt = 1e30f;
       for (int C : cand) {
-        if (smem_ycols(C, P, 0) > (size_t)optin) continue;
+        if (smem_ycols_fx(C, P, 0) + 2048 > (size_t)optin) continue;
         cc = C;
         float ms = 0;
         int s = time_stages_of(c, d, -1, -1, reps, &ms);
@@ -1473,7 +1499,7 @@ int ptt_autotune(ptt_ctx* c, int32_t* choices, int32_t max_groups) {
       int best = d.zC;
       float bt = 1e30f;
       for (int C : cand) {
-        if (C > d.K || smem_zcols3(C, d.Mz, d.f32) > (size_t)optin) continue;
+        if (C > d.K || smem_zcols3(C, d.Mz) + 2048 > (size_t)optin) continue;
         d.zC = C;
         float ms = 0;
         int s = time_stages_of(c, d, 0, 2, reps, &ms);

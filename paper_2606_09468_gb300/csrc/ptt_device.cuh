@@ -1,15 +1,17 @@
 // Device building blocks shared by the 2D and 3D kernels of the sPTT channel
 // step: complex arithmetic in double and single precision, mixed-radix
-// Stockham FFTs in shared memory, SBDF coefficients, warp-cooperative
+// Stockham FFTs in shared memory (single precision here; FP64-accurate in
+// 64-bit block fixed point, ptt_fx.cuh), SBDF coefficients, warp-cooperative
 // Chebyshev recurrences and quasi-tridiagonal tau sweeps, the Chebyshev
 // column transforms (Gauss and Gauss-Lobatto grids) and the Fourier row
 // transforms.  Included by each kernel translation unit (internal linkage).
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cstdint>
 #include <type_traits>
 
-#include "ptt_ds.cuh"
+#include "ptt_fx.cuh"
 #include "ptt_internal.h"
 
 namespace ptt {
@@ -76,31 +78,43 @@ __device__ __forceinline__ float2 cfma(float s, float2 a, float2 c) {
   return make_float2(fmaf(s, a.x, c.x), fmaf(s, a.y, c.y));
 }
 
-// compute types: double2 (FP64 path), float2 (mixed path), dsc (double-single:
-// the FP64-accurate path on the FP32 pipe, PTT_FP64_DS; see ptt_ds.cuh)
+// compute types of the transforms: float2 (mixed groups), fxc (FP64-accurate,
+// 64-bit block fixed point between FP64 arrays)
 template <typename C2> struct RealOf;
 template <> struct RealOf<double2> { using T = double; };
 template <> struct RealOf<float2> { using T = float; };
-template <> struct RealOf<dsc> { using T = dsf; };
 template <typename C2> __device__ __forceinline__ C2 zero2();
 template <> __device__ __forceinline__ double2 zero2<double2>() { return make_double2(0.0, 0.0); }
 template <> __device__ __forceinline__ float2 zero2<float2>() { return make_float2(0.f, 0.f); }
-template <> __device__ __forceinline__ dsc zero2<dsc>() { return mk_dsc(dsf(0.f, 0.f), dsf(0.f, 0.f)); }
 template <typename D> __device__ __forceinline__ D cvt2(double2 v);
 template <typename D> __device__ __forceinline__ D cvt2(float2 v);
-template <typename D> __device__ __forceinline__ D cvt2(dsc v);
 template <> __device__ __forceinline__ double2 cvt2<double2>(double2 v) { return v; }
 template <> __device__ __forceinline__ float2 cvt2<float2>(double2 v) { return make_float2((float)v.x, (float)v.y); }
 template <> __device__ __forceinline__ double2 cvt2<double2>(float2 v) { return make_double2(v.x, v.y); }
 template <> __device__ __forceinline__ float2 cvt2<float2>(float2 v) { return v; }
-template <> __device__ __forceinline__ dsc cvt2<dsc>(double2 v) { return dsc_from_double2(v); }
-template <> __device__ __forceinline__ dsc cvt2<dsc>(float2 v) {
-  return mk_dsc(dsf(v.x, 0.f), dsf(v.y, 0.f));
+
+// FP64 <-> FP32 by integer operations (no FP64 pipe work).  Truncated:
+// values below the FP32 normal range give zero, beyond it infinity, NaN
+// stays NaN.
+__device__ __forceinline__ float f32_from_f64_trunc(double d) {
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  const uint32_t sign = hi & 0x80000000u;
+  const int ef = (int)((hi >> 20) & 0x7FF) - 1023 + 127;
+  if (ef >= 255) {
+    const bool nan = (hi & 0x7FF00000u) == 0x7FF00000u && ((hi & 0xFFFFFu) | lo) != 0u;
+    return __uint_as_float(sign | 0x7F800000u | (nan ? 0x400000u : 0u));
+  }
+  if (ef <= 0) return __uint_as_float(sign);
+  return __uint_as_float(sign | ((uint32_t)ef << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
 }
-template <> __device__ __forceinline__ dsc cvt2<dsc>(dsc v) { return v; }
-template <> __device__ __forceinline__ double2 cvt2<double2>(dsc v) { return dsc_to_double2(v); }
-template <> __device__ __forceinline__ float2 cvt2<float2>(dsc v) {
-  return make_float2(__fadd_rn(v.x.h, v.x.l), __fadd_rn(v.y.h, v.y.l));
+// exact for normal values; zero and subnormals give a signed zero,
+// infinities stay, NaN is NaN
+__device__ __forceinline__ double f64_from_f32(float v) {
+  const uint32_t b = __float_as_uint(v);
+  const uint32_t sign = b & 0x80000000u, e = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu;
+  if (e == 0u) return __hiloint2double((int)sign, 0);
+  if (e == 255u) return __hiloint2double((int)(sign | 0x7FF00000u | (m ? 0x80000u : 0u)), 0);
+  return __hiloint2double((int)(sign | ((e + 896u) << 20) | (m >> 3)), (int)((m & 7u) << 29));
 }
 
 // ------------------------------------------- mean / fluctuation products
@@ -189,10 +203,7 @@ template <int DIR> struct Bfly<DIR, 5> {
   }
 };
 
-// Radix 8 (the FP32 plans; the FP64 plans keep radices up to 5 and their
-// tangent-form twiddles, the double-single ones too: there the eight
-// double-single values per butterfly cost more registers than the saved
-// pass gains, measured): with w = exp(DIR 2 pi i / 8),
+// Radix 8: with w = exp(DIR 2 pi i / 8),
 // a_r = v_r + v_{r+4}, b_r = (v_r - v_{r+4}) w^r (r < 4), the even outputs
 // are the 4-point DFT of a and the odd ones that of b:
 //   y_{2k} = sum_r a_r w^{2rk},  y_{2k+1} = sum_r b_r w^{2rk}.
@@ -236,72 +247,6 @@ template <int DIR> struct Bfly<DIR, 8> {
   }
 };
 
-// Odd prime radices 7, 11, 13 (the unpadded lengths nx, 2 (ny - 1) and nz
-// may carry one such factor).  With H = (R - 1)/2, t_k = v_k + v_{R-k},
-// d_k = v_k - v_{R-k} (k = 1..H) and w = exp(DIR 2 pi i / R):
-//   y_0 = v_0 + sum_k t_k,
-//   y_j, y_{R-j} = b_j +- i DIR e_j,  b_j = v_0 + sum_k cos(2 pi jk/R) t_k,
-//                                     e_j = sum_k sin(2 pi jk/R) d_k  (j = 1..H),
-// the cosines and sines of 2 pi m / R (m = 1..H) as literals, the others by
-// symmetry (jk reduced mod R).
-// cos and sin of 2 pi m / R, m = 1 .. (R - 1)/2 (folded to constants once
-// the butterfly's loops are unrolled).
-__device__ __forceinline__ constexpr double odd_cos(int R, int m) {
-  constexpr double c7[3] = {0.6234898018587335305250, -0.2225209339563144042890, -0.9009688679024191262361};
-  constexpr double c11[5] = {0.8412535328311811688618, 0.4154150130018864255292, -0.1423148382732851404438,
-                             -0.6548607339452850640569, -0.9594929736144973898904};
-  constexpr double c13[6] = {0.8854560256532098959003, 0.5680647467311558025118, 0.1205366802553230533490,
-                             -0.3546048870425356259696, -0.7485107481711010986346, -0.9709418174260520271570};
-  return R == 7 ? c7[m - 1] : R == 11 ? c11[m - 1] : c13[m - 1];
-}
-__device__ __forceinline__ constexpr double odd_sin(int R, int m) {
-  constexpr double s7[3] = {0.7818314824680298087084, 0.9749279121818236070181, 0.4338837391175581204757};
-  constexpr double s11[5] = {0.5406408174555975821076, 0.9096319953545183714117, 0.9898214418809327323760,
-                             0.7557495743542582837740, 0.2817325568414296977114};
-  constexpr double s13[6] = {0.4647231720437685456560, 0.8229838658936563945796, 0.9927088740980539928007,
-                             0.9350162426854148234397, 0.6631226582407952023767, 0.2393156642875577671487};
-  return R == 7 ? s7[m - 1] : R == 11 ? s11[m - 1] : s13[m - 1];
-}
-
-template <int DIR, int R> struct BflyOdd {
-  template <typename C2>
-  static __device__ __forceinline__ void run(C2* v) {
-    using T = typename RealOf<C2>::T;
-    constexpr int H = (R - 1) / 2;
-    C2 t[H], d[H];
-#pragma unroll
-    for (int k = 1; k <= H; ++k) {
-      t[k - 1] = cadd(v[k], v[R - k]);
-      d[k - 1] = csub(v[k], v[R - k]);
-    }
-    C2 y[R];
-    y[0] = v[0];
-#pragma unroll
-    for (int k = 0; k < H; ++k) y[0] = cadd(y[0], t[k]);
-#pragma unroll
-    for (int j = 1; j <= H; ++j) {
-      C2 b = v[0], e = zero2<C2>();
-#pragma unroll
-      for (int k = 1; k <= H; ++k) {
-        const int mm = (j * k) % R;                  // 1 .. R-1
-        const int mi = (mm <= H) ? mm : R - mm;      // cos even, sin odd about R/2
-        const T c = (T)odd_cos(R, mi);
-        const T sn = (T)((mm <= H) ? odd_sin(R, mi) : -odd_sin(R, mi));
-        b = cfma(c, t[k - 1], b);
-        e = cfma(sn, d[k - 1], e);
-      }
-      const C2 ie = cscl(mul_i(e), (T)DIR);
-      y[j] = cadd(b, ie);
-      y[R - j] = csub(b, ie);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = y[r];
-  }
-};
-template <int DIR> struct Bfly<DIR, 7> : BflyOdd<DIR, 7> {};
-template <int DIR> struct Bfly<DIR, 11> : BflyOdd<DIR, 11> {};
-template <int DIR> struct Bfly<DIR, 13> : BflyOdd<DIR, 13> {};
-
 // Division by a runtime divisor d through a multiply-high (the method of
 // Granlund and Montgomery, "Division by invariant integers using
 // multiplication", PLDI 1994, in its round-up form): with
@@ -337,14 +282,6 @@ __device__ __forceinline__ PassC pass_c(const FftPlan& pl, int s) {
   return c;
 }
 
-// read-only table loads (the double-single table as one 16-byte load)
-__device__ __forceinline__ double2 ldg_tw(const double2* p) { return __ldg(p); }
-__device__ __forceinline__ float2 ldg_tw(const float2* p) { return __ldg(p); }
-__device__ __forceinline__ dsc ldg_tw(const dsc* p) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
-  return mk_dsc(dsf(v.x, v.y), dsf(v.z, v.w));
-}
-
 // One Stockham pass of radix R over nl lines (line l at offset l*ls).
 template <int DIR, int R, typename C2>
 __device__ __forceinline__ void fft_pass(const C2* __restrict__ src, C2* __restrict__ dst,
@@ -366,7 +303,7 @@ __device__ __forceinline__ void fft_pass(const C2* __restrict__ src, C2* __restr
     if (Ns > 1) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        C2 w = ldg_tw(&tw[jm * r * st]);
+        C2 w = __ldg(&tw[jm * r * st]);
         if (DIR > 0) w.y = -w.y;
         v[r] = cmul(v[r], w);
       }
@@ -378,110 +315,8 @@ __device__ __forceinline__ void fft_pass(const C2* __restrict__ src, C2* __restr
   }
 }
 
-// ---------------------------------------------- tangent-form FP64 passes
-// A twiddle i^k c (1 + i t) applied as u = v + i t v (two FMAs), the quarter
-// turn i^k by swaps and sign flips (integer operations), and c folded into
-// the butterfly's sums as FMA coefficients: 6, 16, 22 and 44 FP64 operations
-// for a twiddled radix-2, 3, 4 and 5 butterfly against 8, 20, 28 and 52 with
-// plain complex products.  Tables: FftPlan::tt, tk.
 __device__ __forceinline__ double flip_sign(double v, bool c) {
   return __hiloint2double(__double2hiint(v) ^ (c ? (int)0x80000000 : 0), __double2loint(v));
-}
-__device__ __forceinline__ double2 rot_quarter(double2 u, int k) {   // i^k u, k in 0..3
-  const bool sw = k & 1;
-  const double x = sw ? u.y : u.x, y = sw ? u.x : u.y;
-  return make_double2(flip_sign(x, k == 1 || k == 2), flip_sign(y, k >= 2));
-}
-// i^k (1 + i t) v for the forward twiddle; the inverse uses the conjugate,
-// i^-k (1 - i t) v.
-template <int DIR>
-__device__ __forceinline__ double2 tan_rotate(double2 v, double t, int k) {
-  if (DIR > 0) { t = -t; k = (4 - k) & 3; }
-  return rot_quarter(make_double2(fma(-t, v.y, v.x), fma(t, v.x, v.y)), k);
-}
-
-template <int DIR, int R>
-__device__ __forceinline__ void fft_pass_tan(const double2* __restrict__ src, double2* __restrict__ dst,
-                                             int nl, int ls, const PassC& c,
-                                             const double* __restrict__ tt,
-                                             const int* __restrict__ tk) {
-  const int nb = c.nb, Ns = c.Ns;
-  const int total = nl * nb;
-  const FastDiv dnb = c.dnb, dns = c.dns;
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    const int l = (int)fdiv((unsigned)t, dnb);
-    const int j = t - l * nb;
-    const double2* s = src + l * ls;
-    double2* d = dst + l * ls;
-    const int jq = (int)fdiv((unsigned)j, dns);
-    const int jm = j - jq * Ns;
-    const double* rec = tt + (size_t)(R == 5 ? 16 : 6) * jm;
-    const int kp = tk[jm];
-    const int o = jq * Ns * R + jm;
-    const double2 v0 = s[j];
-    if (R == 2) {
-      const double2 u1 = tan_rotate<DIR>(s[j + nb], rec[0], kp & 3);
-      const double c1 = rec[1];
-      d[o] = make_double2(fma(c1, u1.x, v0.x), fma(c1, u1.y, v0.y));
-      d[o + Ns] = make_double2(fma(-c1, u1.x, v0.x), fma(-c1, u1.y, v0.y));
-    } else if (R == 3) {
-      const double2 u1 = tan_rotate<DIR>(s[j + nb], rec[0], kp & 3);
-      const double2 u2 = tan_rotate<DIR>(s[j + 2 * nb], rec[1], (kp >> 2) & 3);
-      const double c1 = rec[2], rho = rec[3], h = rec[4], sc = (DIR > 0) ? rec[5] : -rec[5];
-      const double2 q = make_double2(fma(rho, u2.x, u1.x), fma(rho, u2.y, u1.y));     // (a1 + a2)/c1
-      const double2 qm = make_double2(fma(-rho, u2.x, u1.x), fma(-rho, u2.y, u1.y));  // (a1 - a2)/c1
-      const double2 m = make_double2(fma(-h, q.x, v0.x), fma(-h, q.y, v0.y));
-      d[o] = make_double2(fma(c1, q.x, v0.x), fma(c1, q.y, v0.y));
-      // y1 = m + i s (a1 - a2), y2 = m - i s (a1 - a2), s = DIR sin(2 pi/3)
-      d[o + Ns] = make_double2(fma(-sc, qm.y, m.x), fma(sc, qm.x, m.y));
-      d[o + 2 * Ns] = make_double2(fma(sc, qm.y, m.x), fma(-sc, qm.x, m.y));
-    } else if (R == 5) {
-      // a_r = c_r u_r; with t1 = a1 + a4 = c1 q1, d1 = a1 - a4 = c1 m1,
-      // t2 = a2 + a3 = c2 q2, d2 = a2 - a3 = c2 m2 the radix-5 DFT reads
-      // y0 = v0 + t1 + t2, b1 = v0 + C1 t1 + C2 t2, b2 = v0 + C2 t1 + C1 t2,
-      // y1,4 = b1 +- i DIR (S1 d1 + S2 d2), y2,3 = b2 +- i DIR (S2 d1 - S1 d2)
-      const double2 u1 = tan_rotate<DIR>(s[j + nb], rec[0], kp & 3);
-      const double2 u2 = tan_rotate<DIR>(s[j + 2 * nb], rec[1], (kp >> 2) & 3);
-      const double2 u3 = tan_rotate<DIR>(s[j + 3 * nb], rec[2], (kp >> 4) & 3);
-      const double2 u4 = tan_rotate<DIR>(s[j + 4 * nb], rec[3], (kp >> 6) & 3);
-      const double r14 = rec[4], r23 = rec[5];
-      const double2 q1 = make_double2(fma(r14, u4.x, u1.x), fma(r14, u4.y, u1.y));
-      const double2 m1 = make_double2(fma(-r14, u4.x, u1.x), fma(-r14, u4.y, u1.y));
-      const double2 q2 = make_double2(fma(r23, u3.x, u2.x), fma(r23, u3.y, u2.y));
-      const double2 m2 = make_double2(fma(-r23, u3.x, u2.x), fma(-r23, u3.y, u2.y));
-      const double c1 = rec[6], c2 = rec[7];
-      d[o] = make_double2(fma(c1, q1.x, fma(c2, q2.x, v0.x)), fma(c1, q1.y, fma(c2, q2.y, v0.y)));
-      const double2 b1 = make_double2(fma(rec[8], q1.x, fma(rec[9], q2.x, v0.x)),
-                                      fma(rec[8], q1.y, fma(rec[9], q2.y, v0.y)));
-      const double2 b2 = make_double2(fma(rec[10], q1.x, fma(rec[11], q2.x, v0.x)),
-                                      fma(rec[10], q1.y, fma(rec[11], q2.y, v0.y)));
-      const double2 e1 = make_double2(fma(rec[12], m1.x, rec[13] * m2.x), fma(rec[12], m1.y, rec[13] * m2.y));
-      const double2 e2 = make_double2(fma(rec[14], m1.x, -rec[15] * m2.x), fma(rec[14], m1.y, -rec[15] * m2.y));
-      // i e = (-e.y, e.x); DIR < 0: y1 = b1 - i e1, y4 = b1 + i e1 (likewise y2, y3)
-      const double2 p1 = make_double2(b1.x - e1.y, b1.y + e1.x), n1 = make_double2(b1.x + e1.y, b1.y - e1.x);
-      const double2 p2 = make_double2(b2.x - e2.y, b2.y + e2.x), n2 = make_double2(b2.x + e2.y, b2.y - e2.x);
-      d[o + Ns] = (DIR < 0) ? n1 : p1;
-      d[o + 4 * Ns] = (DIR < 0) ? p1 : n1;
-      d[o + 2 * Ns] = (DIR < 0) ? n2 : p2;
-      d[o + 3 * Ns] = (DIR < 0) ? p2 : n2;
-    } else {
-      const double2 u1 = tan_rotate<DIR>(s[j + nb], rec[0], kp & 3);
-      const double2 u2 = tan_rotate<DIR>(s[j + 2 * nb], rec[1], (kp >> 2) & 3);
-      const double2 u3 = tan_rotate<DIR>(s[j + 3 * nb], rec[2], (kp >> 4) & 3);
-      const double c1 = rec[3], c2 = rec[4], rho = rec[5];
-      const double2 s02 = make_double2(fma(c2, u2.x, v0.x), fma(c2, u2.y, v0.y));
-      const double2 d02 = make_double2(fma(-c2, u2.x, v0.x), fma(-c2, u2.y, v0.y));
-      const double2 q = make_double2(fma(rho, u3.x, u1.x), fma(rho, u3.y, u1.y));     // (a1 + a3)/c1
-      const double2 qm = make_double2(fma(-rho, u3.x, u1.x), fma(-rho, u3.y, u1.y));  // (a1 - a3)/c1
-      d[o] = make_double2(fma(c1, q.x, s02.x), fma(c1, q.y, s02.y));
-      d[o + 2 * Ns] = make_double2(fma(-c1, q.x, s02.x), fma(-c1, q.y, s02.y));
-      // d13 = i (a1 - a3) = c1 (-qm.y, qm.x); forward y1 = d02 - d13, y3 = d02 + d13
-      const double2 yA = make_double2(fma(c1, qm.y, d02.x), fma(-c1, qm.x, d02.y));   // d02 - d13
-      const double2 yB = make_double2(fma(-c1, qm.y, d02.x), fma(c1, qm.x, d02.y));   // d02 + d13
-      d[o + Ns] = (DIR < 0) ? yA : yB;
-      d[o + 3 * Ns] = (DIR < 0) ? yB : yA;
-    }
-  }
 }
 
 // First pass of radix 3 (no twiddles) for lines that are zero in their
@@ -514,149 +349,34 @@ __device__ __forceinline__ void fft_pass_r3_zmid(const C2* __restrict__ src, C2*
   }
 }
 
-template <typename C2> __device__ __forceinline__ const C2* plan_tw(const FftPlan& pl);
-template <> __device__ __forceinline__ const double2* plan_tw<double2>(const FftPlan& pl) { return pl.tw; }
-template <> __device__ __forceinline__ const float2* plan_tw<float2>(const FftPlan& pl) { return pl.twf; }
-template <> __device__ __forceinline__ const dsc* plan_tw<dsc>(const FftPlan& pl) {
-  return reinterpret_cast<const dsc*>(pl.twd);
-}
-
-// Unnormalised DFT of nl lines of length pl.n held in `a`, using `b` as the
-// ping-pong buffer.  Returns the buffer holding the result.  Must be called
-// by the whole block after a __syncthreads(); ends with one.  zero_mid: the
-// lines are zero in their middle third and the plan starts with radix 3.
-// BIG: the plan may hold radices 7, 11, 13 (unpadded lengths); without it
-// only 2 to 5 are compiled in (the padded lengths, chosen 5-smooth), which
-// keeps the register budget of the hot transform kernels, and a pass of
-// another radix is skipped (the launch code never gives such a plan).
-template <int DIR, typename C2, bool BIG = false>
-__device__ C2* fft_lines(C2* a, C2* b, int nl, int ls, const FftPlan& pl, bool zero_mid = false) {
-  C2* src = a;
-  C2* dst = b;
-  const C2* tw = plan_tw<C2>(pl);
+// Unnormalised FP32 DFT of nl lines of length pl.n held in `a`, using `b` as
+// the ping-pong buffer.  Returns the buffer holding the result.  Must be
+// called by the whole block after a __syncthreads(); ends with one.
+// zero_mid: the lines are zero in their middle third and the plan starts
+// with radix 3.  Radices 2 to 5 and 8 (the padded lengths are 5-smooth).
+template <int DIR>
+__device__ float2* fft_lines(float2* a, float2* b, int nl, int ls, const FftPlan& pl, bool zero_mid = false) {
+  float2* src = a;
+  float2* dst = b;
+  const float2* tw = pl.twf;
   for (int s = 0; s < pl.nst; ++s) {
     const int R = pl.radix[s];
     const PassC c = pass_c(pl, s);
     if (s == 0 && zero_mid && R == 3) {
       fft_pass_r3_zmid<DIR>(src, dst, nl, ls, c);
-      __syncthreads();
-      C2* t = src; src = dst; dst = t;
-      continue;
-    }
-    if constexpr (std::is_same<C2, double2>::value) {
-      if (pl.tt && s > 0 && R <= 5) {
-        const double* tt = pl.tt + pl.tto[s];
-        const int* tk = pl.tk + pl.toff[s];
-        if (R == 5) fft_pass_tan<DIR, 5>(src, dst, nl, ls, c, tt, tk);
-        else if (R == 4) fft_pass_tan<DIR, 4>(src, dst, nl, ls, c, tt, tk);
-        else if (R == 3) fft_pass_tan<DIR, 3>(src, dst, nl, ls, c, tt, tk);
-        else fft_pass_tan<DIR, 2>(src, dst, nl, ls, c, tt, tk);
-        __syncthreads();
-        C2* t = src; src = dst; dst = t;
-        continue;
+    } else {
+      switch (R) {
+        case 2: fft_pass<DIR, 2>(src, dst, nl, ls, c, tw); break;
+        case 3: fft_pass<DIR, 3>(src, dst, nl, ls, c, tw); break;
+        case 4: fft_pass<DIR, 4>(src, dst, nl, ls, c, tw); break;
+        case 5: fft_pass<DIR, 5>(src, dst, nl, ls, c, tw); break;
+        default: fft_pass<DIR, 8>(src, dst, nl, ls, c, tw); break;
       }
-    }
-    switch (R) {
-      case 2: fft_pass<DIR, 2>(src, dst, nl, ls, c, tw); break;
-      case 3: fft_pass<DIR, 3>(src, dst, nl, ls, c, tw); break;
-      case 4: fft_pass<DIR, 4>(src, dst, nl, ls, c, tw); break;
-      case 5: fft_pass<DIR, 5>(src, dst, nl, ls, c, tw); break;
-      case 8:   // plans of FP32 groups only (see wide_plans); compiled for
-                // FP32 alone, so the FP64 and double-single kernels keep
-                // their register budgets
-        if constexpr (std::is_same<C2, float2>::value) fft_pass<DIR, 8>(src, dst, nl, ls, c, tw);
-        break;
-      default:
-        if constexpr (BIG) {
-          if (R == 7) fft_pass<DIR, 7>(src, dst, nl, ls, c, tw);
-          else if (R == 11) fft_pass<DIR, 11>(src, dst, nl, ls, c, tw);
-          else if (R == 13) fft_pass<DIR, 13>(src, dst, nl, ls, c, tw);
-        }
-        break;
     }
     __syncthreads();
-    C2* t = src; src = dst; dst = t;
+    float2* t = src; src = dst; dst = t;
   }
   return src;
-}
-
-// ---------------------------------------------- in-place FFT passes
-// For lines too long for two buffers in shared memory (the FP64 3D x pass
-// at Mx = 768): each pass gathers its butterflies' inputs into registers,
-// waits for the whole block, and writes the outputs over the same buffer.
-// Lines go in groups of at most kIpLines, so that a thread holds at most
-// ip_maxb(R) butterflies with blockDim.x = kIpThreads and n <= kIpMaxN.
-// Plain twiddles (FftPlan::tw).
-constexpr int kIpThreads = 512, kIpLines = 3, kIpMaxN = 768;
-__host__ __device__ constexpr int ip_maxb(int R) {
-  return (kIpLines * kIpMaxN / R + kIpThreads - 1) / kIpThreads;
-}
-
-template <int DIR, int R, typename C2>
-__device__ __forceinline__ void fft_pass_ip(C2* a, int nl, int ls, const PassC& c,
-                                            const C2* __restrict__ tw, bool zmid) {
-  constexpr int MB = ip_maxb(R);
-  const int nb = c.nb, st = c.st, Ns = c.Ns;
-  const int total = nl * nb;
-  const FastDiv dnb = c.dnb, dns = c.dns;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  C2 v[MB][R];
-#pragma unroll
-  for (int q = 0; q < MB; ++q) {
-    const int t = tid + q * nt;
-    if (t < total) {
-      const int l = (int)fdiv((unsigned)t, dnb), j = t - l * nb;
-      const C2* s = a + l * ls;
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[q][r] = (zmid && r == 1) ? zero2<C2>() : s[j + r * nb];
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < MB; ++q) {
-    const int t = tid + q * nt;
-    if (t < total) {
-      const int l = (int)fdiv((unsigned)t, dnb), j = t - l * nb;
-      C2* d = a + l * ls;
-      const int jq = (int)fdiv((unsigned)j, dns), jm = j - jq * Ns;
-      if (Ns > 1) {
-#pragma unroll
-        for (int r = 1; r < R; ++r) {
-          C2 w = ldg_tw(&tw[jm * r * st]);
-          if (DIR > 0) w.y = -w.y;
-          v[q][r] = cmul(v[q][r], w);
-        }
-      }
-      Bfly<DIR, R>::run(v[q]);
-      const int o = jq * Ns * R + jm;
-#pragma unroll
-      for (int r = 0; r < R; ++r) d[o + r * Ns] = v[q][r];
-    }
-  }
-  __syncthreads();
-}
-
-// In-place unnormalised DFT of nl lines of length pl.n (radices 2 to 5) in
-// `a`; zero_mid as for fft_lines.  Called by the whole block (kIpThreads
-// threads) after a __syncthreads(); ends with one.
-template <int DIR, typename C2>
-__device__ void fft_lines_inplace(C2* a, int nl, int ls, const FftPlan& pl, bool zero_mid = false) {
-  const C2* tw = plan_tw<C2>(pl);
-  for (int l0 = 0; l0 < nl; l0 += kIpLines) {
-    const int g = min(kIpLines, nl - l0);
-    C2* base = a + (size_t)l0 * ls;
-    for (int s = 0; s < pl.nst; ++s) {
-      const int R = pl.radix[s];
-      const PassC c = pass_c(pl, s);
-      const bool zm = (s == 0 && zero_mid && R == 3);
-      switch (R) {
-        case 2: fft_pass_ip<DIR, 2>(base, g, ls, c, tw, false); break;
-        case 3: fft_pass_ip<DIR, 3>(base, g, ls, c, tw, zm); break;
-        case 4: fft_pass_ip<DIR, 4>(base, g, ls, c, tw, false); break;
-        default: fft_pass_ip<DIR, 5>(base, g, ls, c, tw, false); break;
-      }
-    }
-  }
 }
 
 // SBDF coefficients, orders 1..4: a_0..a_4 and b_0..b_3 (Sec. 2: 4th-order
@@ -681,10 +401,10 @@ __constant__ float c_sbf[4][4] = {{1.f, 0.f, 0.f, 0.f},   // the same (exact in 
 // checkpoints copy the same byte ranges).  FP64 <-> FP32 by integer
 // operations.
 __device__ __forceinline__ float2 f2_trunc(double2 v) {
-  return make_float2(ds_from_double(v.x).h, ds_from_double(v.y).h);
+  return make_float2(f32_from_f64_trunc(v.x), f32_from_f64_trunc(v.y));
 }
 __device__ __forceinline__ double2 d2_exact(float2 v) {
-  return make_double2(ds_f32_to_f64(v.x), ds_f32_to_f64(v.y));
+  return make_double2(f64_from_f32(v.x), f64_from_f32(v.y));
 }
 
 // ------------------------------------------- warp-cooperative recurrences
@@ -1058,42 +778,26 @@ struct YJob {
   int gauss;          // 0: M+1 Gauss-Lobatto points (DCT-I, FFT length 2M);
                       // 1: M Gauss points (DCT-II/III, FFT length M, M even)
   int src_f32, dst_f32;  // element types of src / dst (0: complex double, 1: complex float)
-  const double2* tw4;    // gauss: quarter-period table of this direction, k < M:
+  const float2* tw4f;    // gauss, FP32: quarter-period table of this direction, k < M:
                          // forward (s_k/2) exp(-i pi k/(2M)) (s_0 = 1/M, s_k = 2/M),
                          // inverse (1/2) exp(+i pi k/(2M))
-  const float2* tw4f;    // the same in single precision
-  const float4* tw4d;    // the same in double-single (re.h, re.l, im.h, im.l)
+  const int4* tw4x;      // gauss, fixed point (GroupDev::tw4Px, tw4Pix): forward
+                         // with the factor 2^fexp times the normalisation of the
+                         // whole forward transform, inverse exp(+i pi k/(2M))
+  int fexp;
   int C;              // columns per block
   const int* status;  // skip members with status != 0 (may be null)
   FftPlan pl;
 };
 
 // Element formats of transform inputs and outputs (YJob / ZJob src_f32,
-// dst_f32): 0 complex double, 1 complex float, kFmtDS double-single as
-// computed (the intermediates of PTT_FP64_DS groups, in their FP64 arrays:
-// the same 16 bytes per element).  Only the double-single kernels read or
-// write kFmtDS.
-constexpr int kFmtDS = 2;
-template <typename CT>
-__device__ __forceinline__ CT ld2(const void* p, long long i, int f32) {
-  if constexpr (std::is_same<CT, dsc>::value) {
-    if (f32 == kFmtDS) return static_cast<const dsc*>(p)[i];
-  }
-  return f32 ? cvt2<CT>(static_cast<const float2*>(p)[i]) : cvt2<CT>(static_cast<const double2*>(p)[i]);
+// dst_f32): 0 complex double, 1 complex float.
+__device__ __forceinline__ float2 ld2(const void* p, long long i, int f32) {
+  return f32 ? static_cast<const float2*>(p)[i] : cvt2<float2>(static_cast<const double2*>(p)[i]);
 }
-template <typename CT>
-__device__ __forceinline__ void st2(void* p, long long i, int f32, CT v) {
-  if constexpr (std::is_same<CT, dsc>::value) {
-    if (f32 == kFmtDS) { static_cast<dsc*>(p)[i] = v; return; }
-  }
-  if (f32) static_cast<float2*>(p)[i] = cvt2<float2>(v);
+__device__ __forceinline__ void st2(void* p, long long i, int f32, float2 v) {
+  if (f32) static_cast<float2*>(p)[i] = v;
   else static_cast<double2*>(p)[i] = cvt2<double2>(v);
-}
-template <typename CT> __device__ __forceinline__ CT ld_tw4(const YJob& J, int k);
-template <> __device__ __forceinline__ double2 ld_tw4<double2>(const YJob& J, int k) { return __ldg(&J.tw4[k]); }
-template <> __device__ __forceinline__ float2 ld_tw4<float2>(const YJob& J, int k) { return __ldg(&J.tw4f[k]); }
-template <> __device__ __forceinline__ dsc ld_tw4<dsc>(const YJob& J, int k) {
-  return ldg_tw(reinterpret_cast<const dsc*>(J.tw4d) + k);
 }
 
 // Values at the M Gauss points y_j = cos(pi (2j+1)/(2M)) from coefficients
@@ -1101,21 +805,20 @@ template <> __device__ __forceinline__ dsc ld_tw4<dsc>(const YJob& J, int k) {
 // output (input) order is permuted v_n = f_{2n}, v_{M-1-n} = f_{2n+1}, and a
 // quarter-period twiddle exp(-+ i pi k/(2M)) maps between the two (Makhoul's
 // construction; the real and imaginary parts of a column ride in one FFT).
-template <typename CT>
+// FP32 form.
 __device__ void ycols_gauss(const YJob& J, const void* src, const void* src2, const void* src3,
-                            void* dst, CT* A, CT* B, int c0, int nc, int f) {
-  using T = typename RealOf<CT>::T;
+                            void* dst, float2* A, float2* B, int c0, int nc, int f) {
   const int C = J.C, N = J.N, Mg = J.M;
   const int tid = threadIdx.x, nt = blockDim.x;
   if (J.inverse) {
     for (int i = tid; i < Mg * C; i += nt) {
       const int c = (int)fdiv((unsigned)i, fast_div((unsigned)Mg)), n = i - c * Mg;
-      CT v = zero2<CT>();
+      float2 v = zero2<float2>();
       if (c < nc && n < N) {
         const long long o = (c0 + c) * J.cm + n * J.cn;
-        v = ld2<CT>(src, o, J.src_f32);
-        if (src2) v = cadd(v, ld2<CT>(src2, o, J.src_f32));
-        if (src3) v = cadd(v, ld2<CT>(src3, o, J.src_f32));
+        v = ld2(src, o, J.src_f32);
+        if (src2) v = cadd(v, ld2(src2, o, J.src_f32));
+        if (src3) v = cadd(v, ld2(src3, o, J.src_f32));
       }
       A[i] = v;
     }
@@ -1133,130 +836,218 @@ __device__ void ycols_gauss(const YJob& J, const void* src, const void* src2, co
     // taken from the inverse table
     for (int i = tid; i < Mg * C; i += nt) {
       const int c = (int)fdiv((unsigned)i, fast_div((unsigned)Mg)), k = i - c * Mg;
-      const CT ak = A[i];
-      CT V;
+      const float2 ak = A[i];
+      float2 V;
       if (k == 0) {
         V = ak;
       } else {
-        const CT amk = A[c * Mg + Mg - k];
-        CT z;
+        const float2 amk = A[c * Mg + Mg - k];
+        float2 z;
         z.x = ak.x + amk.y;
         z.y = ak.y - amk.x;
-        V = cmul(ld_tw4<CT>(J, k), z);
+        V = cmul(__ldg(&J.tw4f[k]), z);
       }
       B[i] = V;
     }
     __syncthreads();
-    CT* res = fft_lines<+1>(B, A, C, Mg, J.pl);
+    float2* res = fft_lines<+1>(B, A, C, Mg, J.pl);
     for (int i = tid; i < Mg * C; i += nt) {
       const int j = (int)fdiv((unsigned)i, fast_div((unsigned)C)), c = i - j * C;
       if (c < nc) {
         const int pos = (j & 1) ? (Mg - 1 - (j >> 1)) : (j >> 1);
-        st2<CT>(dst, j * J.vj + (c0 + c) * J.vm, J.dst_f32, res[c * Mg + pos]);
+        st2(dst, j * J.vj + (c0 + c) * J.vm, J.dst_f32, res[c * Mg + pos]);
       }
     }
   } else {
     for (int i = tid; i < Mg * C; i += nt) {
       const int j = (int)fdiv((unsigned)i, fast_div((unsigned)C)), c = i - j * C;
       const int pos = (j & 1) ? (Mg - 1 - (j >> 1)) : (j >> 1);
-      A[c * Mg + pos] = (c < nc) ? ld2<CT>(src, j * J.vj + (c0 + c) * J.vm, J.src_f32) : zero2<CT>();
+      A[c * Mg + pos] = (c < nc) ? ld2(src, j * J.vj + (c0 + c) * J.vm, J.src_f32) : zero2<float2>();
     }
     __syncthreads();
-    CT* res = fft_lines<-1>(A, B, C, Mg, J.pl);
+    float2* res = fft_lines<-1>(A, B, C, Mg, J.pl);
     // with s = V_k + conj V_{M-k}, d = V_k - conj V_{M-k} (the transforms of
     // the real and imaginary parts, times 2 and 2i) and the forward table
     // F_k = (s_k/2) exp(-i pi k/(2M)):  a_k = (Re(F_k s), Re(F_k (-i d)))
     for (int i = tid; i < N * C; i += nt) {
       const int c = (int)fdiv((unsigned)i, fast_div((unsigned)N)), k = i - c * N;
       if (c < nc) {
-        const CT Vk = res[c * Mg + k];
-        const CT Rm = res[c * Mg + (k == 0 ? 0 : Mg - k)];
-        const T sx = Vk.x + Rm.x, sy = Vk.y - Rm.y;
-        const T dx = Vk.x - Rm.x, dy = Vk.y + Rm.y;
-        const CT w = ld_tw4<CT>(J, k);
-        CT o;
+        const float2 Vk = res[c * Mg + k];
+        const float2 Rm = res[c * Mg + (k == 0 ? 0 : Mg - k)];
+        const float sx = Vk.x + Rm.x, sy = Vk.y - Rm.y;
+        const float dx = Vk.x - Rm.x, dy = Vk.y + Rm.y;
+        const float2 w = __ldg(&J.tw4f[k]);
+        float2 o;
         o.x = w.x * sx - w.y * sy;
         o.y = w.x * dy + w.y * dx;
-        st2<CT>(dst, (c0 + c) * J.cm + k * J.cn, J.dst_f32, o);
+        st2(dst, (c0 + c) * J.cm + k * J.cn, J.dst_f32, o);
       }
     }
   }
 }
 
-// Gauss-Lobatto path (FP64, or double-single in PTT_FP64_DS groups; FP64
-// arrays in and out): DCT-I by the even extension.
-template <typename CT>
-__device__ void ycols_lobatto(const YJob& J, const void* src, const void* src2, const void* src3,
-                              void* dst, CT* A, CT* B, CT* a0s, int c0, int nc, int f) {
-  using T = typename RealOf<CT>::T;
-  const int C = J.C, N = J.N, M = J.M, P = 2 * J.M;
-  const int tid = threadIdx.x, nt = blockDim.x;
+// The same in fixed point, FP64 in and out: a warp per column outside the
+// FFT.  Bd: room for the derivative of the block's columns (only for fields
+// with deriv).
+constexpr int kFxCols = 16;   // columns per block, at most
+__device__ void ycols_gauss_fx(const YJob& J, const double2* src, const double2* src2, const double2* src3,
+                               double2* dst, fxc* A, double2* Bd, FxS* fs, int c0, int nc, int f) {
+  const int C = J.C, N = J.N, Mg = J.M;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, nw = nt >> 5;
+  const FastDiv dC = fast_div((unsigned)C);
+  const FastDiv dN = fast_div((unsigned)N);
   if (J.inverse) {
-    for (int i = tid; i < N * C; i += nt) {
-      const int c = (int)fdiv((unsigned)i, fast_div((unsigned)N)), n = i - c * N;
-      CT v = zero2<CT>();
-      if (c < nc) {
-        const long long o = (c0 + c) * J.cm + n * J.cn;
-        v = ld2<CT>(src, o, 0);
-        if (src2) v = cadd(v, ld2<CT>(src2, o, 0));
-        if (src3) v = cadd(v, ld2<CT>(src3, o, 0));
-      }
-      A[c * P + n] = v;
+    for (int i = tid; i < nc * N; i += nt) {
+      const int c = (int)fdiv((unsigned)i, dN), n = i - c * N;
+      const long long o = (c0 + c) * J.cm + n * J.cn;
+      double2 v = src[o];
+      if (src2) v = cadd(v, src2[o]);
+      if (src3) v = cadd(v, src3[o]);
+      reinterpret_cast<double2*>(A)[c * Mg + n] = v;
     }
     __syncthreads();
-    if (J.deriv[f]) {
-      for (int c = tid >> 5; c < C; c += (nt >> 5)) warp_cheb_deriv(A + c * P, B + c * P, N);
-      __syncthreads();
-      for (int i = tid; i < N * C; i += nt) {
-        const int c = (int)fdiv((unsigned)i, fast_div((unsigned)N)), n = i - c * N;
-        A[c * P + n] = B[c * P + n];
+    const bool dy = J.deriv[f] != 0;
+    for (int c = tid >> 5; c < nc; c += nw) {
+      const double2* raw = reinterpret_cast<const double2*>(A + c * Mg);
+      if (dy) {
+        double2* D = Bd + c * N;
+        warp_cheb_deriv(raw, D, N);
+        raw = D;
       }
-      __syncthreads();
-    }
-    if (tid < C) {
-      a0s[tid] = A[tid * P];
-      a0s[C + tid] = (N > M) ? A[tid * P + M] : zero2<CT>();
-    }
-    // even extension: A[n] = a_n (n <= M, zero for n >= N), A[P-n] = a_n
-    for (int i = tid; i < C * P; i += nt) {
-      const int c = (int)fdiv((unsigned)i, fast_div((unsigned)P)), n = i - c * P;
-      if (n >= N && n <= M) A[i] = zero2<CT>();
-      else if (n > M) { const int r = P - n; A[i] = (r < N) ? A[c * P + r] : zero2<CT>(); }
+      unsigned m = 0u;
+      for (int n = lane; n < N; n += 32) m = max(m, fx_mag2(raw[n]));
+      const FxS s = fx_warp_scale(m, N, [raw](int n) { return raw[n]; }, 1);
+      if (lane == 0) fs[c] = s;
     }
     __syncthreads();
-    CT* res = fft_lines<-1, CT, true>(A, B, C, P, J.pl);
-    // f_j = (F_j + a_0 + (-1)^j a_M) / 2
-    for (int i = tid; i < (M + 1) * C; i += nt) {
-      const int j = (int)fdiv((unsigned)i, fast_div((unsigned)C)), c = i - j * C;
+    // twice the V_k: V_0 = 2 a_0, V_k = exp(+i pi k/(2M)) (a_k - i a_{M-k}), the
+    // pair k, M - k by one thread (in place when raw is the column itself); by the
+    // whole block, as a block of one column (the mean's) has one warp at work above
+    const int np = Mg / 2 + 1;
+    const FastDiv dP = fast_div((unsigned)np);
+    for (int i = tid; i < nc * np; i += nt) {
+      const int c = (int)fdiv((unsigned)i, dP), k = i - c * np, km = Mg - k;
+      fxc* V = A + c * Mg;
+      const fxc* rx = dy ? reinterpret_cast<const fxc*>(Bd + c * N) : V;
+      const int base = fs[c].base;
+      const fxc a = (k < N) ? fx_from2(fx_raw(rx[k]), base) : fx_zero();
+      if (k == 0) {
+        V[0] = cadd(a, a);
+      } else {
+        const fxc b = (km < N) ? fx_from2(fx_raw(rx[km]), base) : fx_zero();
+        V[k] = fx_cmul<false>(mk_fxc(a.x + b.y, a.y - b.x), __ldg(&J.tw4x[k]));
+        if (km != k) V[km] = fx_cmul<false>(mk_fxc(b.x + a.y, b.y - a.x), __ldg(&J.tw4x[km]));
+      }
+    }
+    __syncthreads();
+    fx_lines<+1, false>(A, nc, Mg, &J.pl, false);
+    for (int i = tid; i < Mg * C; i += nt) {
+      const int j = (int)fdiv((unsigned)i, dC), c = i - j * C;
       if (c < nc) {
-        CT v = cadd(res[c * P + j], a0s[c]);
-        v = (j & 1) ? csub(v, a0s[C + c]) : cadd(v, a0s[C + c]);
-        st2<CT>(dst, j * J.vj + (c0 + c) * J.vm, 0, cscl(v, (T)0.5));
+        const int pos = (j & 1) ? (Mg - 1 - (j >> 1)) : (j >> 1);
+        dst[j * J.vj + (c0 + c) * J.vm] = fx_to2(A[c * Mg + pos], fs[c], 1);
       }
     }
   } else {
-    for (int i = tid; i < (M + 1) * C; i += nt) {
-      const int j = (int)fdiv((unsigned)i, fast_div((unsigned)C)), c = i - j * C;
-      A[c * P + j] = (c < nc) ? ld2<CT>(src, j * J.vj + (c0 + c) * J.vm, 0) : zero2<CT>();
+    double2* R = reinterpret_cast<double2*>(A);
+    for (int i = tid; i < Mg * C; i += nt) {
+      const int j = (int)fdiv((unsigned)i, dC), c = i - j * C;
+      const int pos = (j & 1) ? (Mg - 1 - (j >> 1)) : (j >> 1);
+      if (c < nc) R[c * Mg + pos] = src[j * J.vj + (c0 + c) * J.vm];
     }
     __syncthreads();
-    for (int i = tid; i < C * P; i += nt) {
-      const int c = (int)fdiv((unsigned)i, fast_div((unsigned)P)), j = i - c * P;
-      if (j > M) A[i] = A[c * P + (P - j)];
+    for (int c = tid >> 5; c < nc; c += nw) {
+      const double2* raw = R + c * Mg;
+      unsigned m = 0u;
+      for (int n = lane; n < Mg; n += 32) m = max(m, fx_mag2(raw[n]));
+      const FxS s = fx_warp_scale(m, Mg, [raw](int n) { return raw[n]; }, 0);
+      if (lane == 0) fs[c] = s;
     }
     __syncthreads();
-    CT* res = fft_lines<-1, CT, true>(A, B, C, P, J.pl);
-    const T inv = T(1.0 / M);
-    for (int i = tid; i < N * C; i += nt) {
-      const int c = (int)fdiv((unsigned)i, fast_div((unsigned)N)), n = i - c * N;
-      if (c < nc) {
-        const T s = (n == 0 || n == M) ? (T)0.5 * inv : inv;
-        st2<CT>(dst, (c0 + c) * J.cm + n * J.cn, 0, cscl(res[c * P + n], s));
-      }
+    const FastDiv dM = fast_div((unsigned)Mg);
+    for (int i = tid; i < nc * Mg; i += nt)
+      A[i] = fx_from2(fx_raw(A[i]), fs[fdiv((unsigned)i, dM)].base);
+    __syncthreads();
+    fx_lines<-1, false>(A, nc, Mg, &J.pl, false);
+    for (int i = tid; i < nc * N; i += nt) {
+      const int c = (int)fdiv((unsigned)i, dN), k = i - c * N;
+      const fxc* V = A + c * Mg;
+      const fxc Vk = V[k], Rm = V[k == 0 ? 0 : Mg - k];
+      const int4 w = __ldg(&J.tw4x[k]);
+      dst[(c0 + c) * J.cm + k * J.cn] =
+          make_double2(fx_to(fx_dot(Vk.x + Rm.x, Vk.y - Rm.y, w), fs[c], J.fexp),
+                       fx_to(fx_dot(Vk.y + Rm.y, Rm.x - Vk.x, w), fs[c], J.fexp));
     }
   }
 }
 
+// Gauss-Lobatto path (fixed point, FP64 in and out): DCT-I by the even
+// extension.
+__device__ void ycols_lobatto(const YJob& J, const double2* src, const double2* src2, const double2* src3,
+                              double2* dst, fxc* A, fxc* a0s, FxS* fs, int c0, int nc) {
+  const int C = J.C, N = J.N, M = J.M, P = 2 * J.M;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, nw = nt >> 5;
+  const FastDiv dC = fast_div((unsigned)C);
+  if (!J.inverse) {
+    double2* R = reinterpret_cast<double2*>(A);
+    for (int i = tid; i < (M + 1) * C; i += nt) {
+      const int j = (int)fdiv((unsigned)i, dC), c = i - j * C;
+      if (c < nc) R[c * P + j] = src[j * J.vj + (c0 + c) * J.vm];
+    }
+    __syncthreads();
+  }
+  const int cnt = J.inverse ? N : M + 1;
+  for (int c = tid >> 5; c < nc; c += nw) {
+    double2* R = reinterpret_cast<double2*>(A + c * P);
+    unsigned m = 0u;
+    for (int n = lane; n < cnt; n += 32) {
+      double2 v;
+      if (J.inverse) {
+        const long long o = (c0 + c) * J.cm + n * J.cn;
+        v = src[o];
+        if (src2) v = cadd(v, src2[o]);
+        if (src3) v = cadd(v, src3[o]);
+        R[n] = v;
+      } else {
+        v = R[n];
+      }
+      m = max(m, fx_mag2(v));
+    }
+    const FxS s = fx_warp_scale(m, cnt, [R](int n) { return R[n]; }, 1);
+    if (lane == 0) fs[c] = s;
+    __syncwarp();
+    // even extension: A[n] = a_n (n <= M, zero for n >= N), A[P - n] = a_n
+    fxc* V = A + c * P;
+    for (int n = lane; n <= M; n += 32) {
+      const fxc a = (n < cnt) ? fx_from2(fx_raw(V[n]), s.base) : fx_zero();
+      V[n] = a;
+      if (n > 0 && n < M) V[P - n] = a;
+      if (n == 0) a0s[c] = a;
+      if (n == M) a0s[C + c] = a;
+    }
+  }
+  __syncthreads();
+  fx_lines<-1, true>(A, nc, P, &J.pl, false);
+  if (J.inverse) {   // f_j = (F_j + a_0 + (-1)^j a_M) / 2
+    for (int i = tid; i < (M + 1) * C; i += nt) {
+      const int j = (int)fdiv((unsigned)i, dC), c = i - j * C;
+      if (c < nc) {
+        fxc v = cadd(A[c * P + j], a0s[c]);
+        v = (j & 1) ? csub(v, a0s[C + c]) : cadd(v, a0s[C + c]);
+        dst[j * J.vj + (c0 + c) * J.vm] = fx_to2(v, fs[c], 1);
+      }
+    }
+  } else {
+    const double inv = 1.0 / M;
+    for (int c = tid >> 5; c < nc; c += nw)
+      for (int n = lane; n < N; n += 32) {
+        const double s = (n == 0 || n == M) ? 0.5 * inv : inv;
+        dst[(c0 + c) * J.cm + n * J.cn] = cscl(fx_to2(A[c * P + n], fs[c]), s);
+      }
+  }
+}
+
+// FP32 columns (CT = float2, Gauss grid only) or fixed point (CT = fxc).
 // BIG: the Gauss-Lobatto (unpadded) path, whose FFT length 2 (ny - 1) may
 // hold radices 7, 11, 13; the Gauss (padded) path runs without it.
 template <typename CT, bool BIG = false>
@@ -1265,15 +1056,15 @@ __device__ __forceinline__ void ycols_block(const YJob& J, Blk bk) {
   if (J.status && J.status[b]) return;
   const int f = bk.y;
   // FFT length per column: M on the Gauss grid, 2M (even extension) on the
-  // Gauss-Lobatto grid; shared memory holds 2 C lines of it (+ 2 C scalars)
+  // Gauss-Lobatto grid (shared memory: smem_ycols, smem_ycols_fx)
   const int C = J.C, K = J.K, P = J.gauss ? J.M : 2 * J.M;
   const int c0 = bk.x * C;
   const int nc = min(C, K - c0);
   extern __shared__ __align__(16) unsigned char smraw[];
   CT* A = reinterpret_cast<CT*>(smraw);
   CT* B = A + (size_t)C * P;
-  const size_t es = (J.src_f32 == 1) ? sizeof(float2) : sizeof(double2);
-  const size_t ed = (J.dst_f32 == 1) ? sizeof(float2) : sizeof(double2);
+  const size_t es = J.src_f32 ? sizeof(float2) : sizeof(double2);
+  const size_t ed = J.dst_f32 ? sizeof(float2) : sizeof(double2);
   const void* src = static_cast<const char*>(J.src) + (b * J.src_mstride + J.src_field[f] * J.src_fstride) * es;
   void* dst = static_cast<char*>(J.dst) + (b * J.dst_mstride + J.dst_field[f] * J.dst_fstride) * ed;
   const void* src2 = (J.inverse && J.src_field2[f] >= 0)
@@ -1282,21 +1073,25 @@ __device__ __forceinline__ void ycols_block(const YJob& J, Blk bk) {
   const void* src3 = (J.inverse && J.src_field3[f] >= 0)
       ? static_cast<const char*>(J.src) + (b * J.src_mstride + J.src_field3[f] * J.src_fstride) * es
       : nullptr;
-  if (J.gauss) {
-    ycols_gauss<CT>(J, src, src2, src3, dst, A, B, c0, nc, f);
-  } else if constexpr (!std::is_same<CT, float2>::value && BIG) {
-    ycols_lobatto<CT>(J, src, src2, src3, dst, A, B, B + (size_t)C * P, c0, nc, f);
+  if constexpr (std::is_same<CT, fxc>::value) {
+    __shared__ FxS fs[kFxCols];
+    const double2 *s1 = static_cast<const double2*>(src), *s2 = static_cast<const double2*>(src2),
+                  *s3 = static_cast<const double2*>(src3);
+    if constexpr (BIG) ycols_lobatto(J, s1, s2, s3, static_cast<double2*>(dst), A, B, fs, c0, nc);
+    else ycols_gauss_fx(J, s1, s2, s3, static_cast<double2*>(dst), A, reinterpret_cast<double2*>(B), fs, c0, nc, f);
+  } else {
+    ycols_gauss(J, src, src2, src3, dst, A, B, c0, nc, f);
   }
 }
 
 template <typename CT, bool BIG = false>
-__global__ void __launch_bounds__(256) k_ycols(YJob J) {
+__global__ void __launch_bounds__(256, BIG ? 3 : 4) k_ycols(const __grid_constant__ YJob J) {
   ycols_block<CT, BIG>(J, this_blk());
 }
 
 // The same over the shape groups of a context (job q of jobs for group q).
 template <typename CT, bool BIG = false>
-__global__ void __launch_bounds__(256) k_ycols_multi(const YJob* __restrict__ jobs, MultiMap mm) {
+__global__ void __launch_bounds__(256, BIG ? 3 : 4) k_ycols_multi(const YJob* __restrict__ jobs, MultiMap mm) {
   Blk bk;
   const int q = multi_locate(mm, bk);
   ycols_block<CT, BIG>(jobs[q], bk);
@@ -1315,86 +1110,170 @@ struct XJob {
   int nf;                    // fields (packed in pairs, (nf + 1) / 2 lines)
   int K, n;
   int c2r;
-  // c2r with nf = 1: block r synthesises rows 2r and 2r + 1 (< nrows) as the
-  // real and imaginary parts of one line (grid over ceil(nrows / 2) rows)
+  // c2r with nf = 1: pair_rows lines per block, line p of all synthesises rows
+  // 2p and 2p + 1 (< nrows) as its real and imaginary parts (xrows_pairs)
   int pair_rows, nrows;
   const int* status;
   FftPlan pl;
 };
 
+// Fixed-point lines of real fields, shared by the x transforms: two fields
+// per line of n points, field q of the block on scale fs[q] (line q >> 1).
+
+// One field of a line from its Fourier modes, by a warp: raw modes get(k),
+// k < K, waiting at h[k] (the even field) or h[n - k], h[K] for k = 0 (the odd
+// one).  Converted by fx_xpack once both fields are there.
+__device__ __forceinline__ int fx_xslot(int odd, int k, int K, int n) {
+  return odd ? (k == 0 ? K : n - k) : k;
+}
+// The packed line F + iG of Hermitian pairs, in place, by a warp.
+__device__ __forceinline__ void fx_xpack(fxc* h, int n, int K, int bF, int bG) {
+  for (int k = threadIdx.x & 31; k < K; k += 32) {
+    const int g = fx_xslot(1, k, K, n);
+    const fxc F = fx_from2(fx_raw(h[k]), bF), G = fx_from2(fx_raw(h[g]), bG);
+    h[k] = mk_fxc(F.x - G.y, F.y + G.x);
+    h[g] = (k == 0) ? fx_zero() : mk_fxc(F.x + G.y, G.x - F.y);
+  }
+}
+// Scales and packing of a line whose raw modes (of both fields) wait in h; mF,
+// mG: the lane's largest fx_mag of each.
+__device__ __forceinline__ void fx_xline(fxc* h, int n, int K, unsigned mF, unsigned mG, FxS& sF, FxS& sG) {
+  const FxS a = fx_warp_scale(mF, K, [h](int k) { return fx_raw(h[k]); }, 2);
+  const FxS b = fx_warp_scale(mG, K, [=](int k) { return fx_raw(h[fx_xslot(1, k, K, n)]); }, 2);
+  if ((threadIdx.x & 31) == 0) { sF = a; sG = b; }
+  __syncwarp();
+  fx_xpack(h, n, K, a.base, b.base);
+}
+// A line of raw values of two real fields (re, im), n points, by a warp: less
+// their first values (returned, for k = 0), each on its own scale.  A row that
+// hardly varies is then held to the size of its variation.
+__device__ __forceinline__ double2 fx_fields(fxc* h, int n, FxS& sF, FxS& sG) {
+  const int lane = threadIdx.x & 31;
+  const double2 ref = fx_raw(h[0]);
+  __syncwarp();
+  unsigned m0 = 0u, m1 = 0u;
+  for (int i = lane; i < n; i += 32) {
+    const double2 v = csub(fx_raw(h[i]), ref);
+    h[i] = fx_bits(v.x, v.y);
+    m0 = max(m0, fx_mag(v.x));
+    m1 = max(m1, fx_mag(v.y));
+  }
+  const int e0 = (int)(__reduce_max_sync(0xffffffffu, m0) >> 20), e1 = (int)(__reduce_max_sync(0xffffffffu, m1) >> 20);
+  unsigned q0 = 0u, q1 = 0u;
+  for (int i = lane; i < n; i += 32) {
+    const double2 v = fx_raw(h[i]);
+    q0 += fx_units(v.x, e0);
+    q1 += fx_units(v.y, e1);
+  }
+  const FxS a = fx_scale(e0, __reduce_add_sync(0xffffffffu, q0), 1);
+  const FxS b = fx_scale(e1, __reduce_add_sync(0xffffffffu, q1), 1);
+  if (lane == 0) { sF = a; sG = b; }
+  for (int i = lane; i < n; i += 32) {
+    const double2 v = fx_raw(h[i]);
+    h[i] = mk_fxc(fx_from(v.x, a.base), fx_from(v.y, b.base));
+  }
+  return ref;
+}
+// Mode k of the two fields of a transformed line, unnormalised: F = (h_k +
+// conj h_{-k})/2, G = (h_k - conj h_{-k})/(2i), plus n times the first values
+// on k = 0.
+__device__ __forceinline__ double2 fx_mode_f(const fxc* h, int n, int k, const FxS& f, double ref) {
+  const fxc hk = h[k], hm = h[k == 0 ? 0 : n - k];
+  double2 F = fx_to2(mk_fxc(hk.x + hm.x, hk.y - hm.y), f, 1);
+  if (k == 0) F.x = fma((double)n, ref, F.x);
+  return F;
+}
+__device__ __forceinline__ double2 fx_mode_g(const fxc* h, int n, int k, const FxS& f, double ref) {
+  const fxc hk = h[k], hm = h[k == 0 ? 0 : n - k];
+  double2 G = fx_to2(mk_fxc(hk.y + hm.y, hm.x - hk.x), f, 1);
+  if (k == 0) G.x = fma((double)n, ref, G.x);
+  return G;
+}
+
+// Lines per block of the paired rows: a warp each, within 48 KB.
+inline int xrows_pairs(int n, int nrows) {
+  int l = 48 * 1024 / (n * 16);
+  if (l > 8) l = 8;
+  while (l > 1 && (long long)l * 304 > (nrows + 1) / 2) l >>= 1;   // at least two blocks per SM
+  return l < 1 ? 1 : l;
+}
+inline unsigned xrows_pair_blocks(int lines, int nrows) { return (unsigned)(((nrows + 1) / 2 + lines - 1) / lines); }
+
 __device__ __forceinline__ void xrows_block(const XJob& J, Blk bk) {
   const int b = bk.y;
   if (J.status && J.status[b]) return;
   const int row = bk.x;
-  const int K = J.K, n = J.n, nf = J.nf, nl = (nf + 1) / 2;
-  extern __shared__ double2 sm[];
-  double2* A = sm;
-  double2* Bb = sm + (size_t)nl * n;
-  const int tid = threadIdx.x, nt = blockDim.x;
+  const bool pr = J.pair_rows != 0;
+  const int K = J.K, n = J.n, nf = J.nf;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ FxS fs[16];
+  __shared__ double2 ref[8];
+  fxc* A = reinterpret_cast<fxc*>(smraw);
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, nw = nt >> 5;
+  const FastDiv dn = fast_div((unsigned)n);
   if (J.c2r) {
-    // paired rows: the second line's source and destination are the next row
-    const bool pr = J.pair_rows != 0;
-    const int r0 = pr ? 2 * row : row;
-    const int nfe = pr ? ((r0 + 1 < J.nrows) ? 2 : 1) : nf;
+    // real field q of the block: a field of the row, or (paired rows) the row
+    // r0 + q of the one field
+    const int r0 = pr ? 2 * J.pair_rows * row : row;
+    const int nq = pr ? min(2 * J.pair_rows, J.nrows - r0) : nf, nl = (nq + 1) / 2;
     const long long sfs = pr ? (long long)J.src_rstep * K : J.src_fstride;
     const long long dfs = pr ? (long long)J.dst_rstep * n : J.dst_fstride;
     const double2* src = J.srcC + b * J.src_mstride + (long long)r0 * J.src_rstep * K;
-    for (int i = tid; i < nl * n; i += nt) {
-      const int l = (int)fdiv((unsigned)i, fast_div((unsigned)n)), k = i - l * n;
-      const int fa = 2 * l, fb = 2 * l + 1;
-      int kk = -1;
-      bool cj = false;
-      if (k < K) kk = k;
-      else if (k > n - K) { kk = n - k; cj = true; }
-      double2 h = czero();
-      if (kk >= 0) {
-        double2 F = src[fa * sfs + kk];
-        double2 G = (fb < nfe) ? src[fb * sfs + kk] : czero();
-        if (kk == 0) { F.y = 0.0; G.y = 0.0; }
-        if (cj) { F = cconj(F); G = cconj(G); }
-        h = cadd(F, mul_i(G));
+    for (int l = tid >> 5; l < nl; l += nw) {
+      fxc* h = A + l * n;
+      unsigned mF = 0u, mG = 0u;
+#pragma unroll 2
+      for (int k = lane; k < K; k += 32) {
+        double2 F = src[(2 * l) * sfs + k];
+        double2 G = (2 * l + 1 < nq) ? src[(2 * l + 1) * sfs + k] : czero();
+        if (k == 0) { F.y = 0.0; G.y = 0.0; }
+        h[k] = fx_bits(F.x, F.y);
+        h[fx_xslot(1, k, K, n)] = fx_bits(G.x, G.y);
+        mF = max(mF, fx_mag2(F));
+        mG = max(mG, fx_mag2(G));
       }
-      A[i] = h;
+      __syncwarp();
+      fx_xline(h, n, K, mF, mG, fs[2 * l], fs[2 * l + 1]);
     }
     __syncthreads();
-    double2* res = fft_lines<+1, double2, true>(A, Bb, nl, n, J.pl);
+    fx_lines<+1, true>(A, nl, n, &J.pl, false);
     double* dst = J.dstR + b * J.dst_mstride + (long long)r0 * J.dst_rstep * n;
     for (int i = tid; i < nl * n; i += nt) {
-      const int l = (int)fdiv((unsigned)i, fast_div((unsigned)n)), x = i - l * n;
-      const double2 h = res[i];
-      dst[(2 * l) * dfs + x] = h.x;
-      if (2 * l + 1 < nfe) dst[(2 * l + 1) * dfs + x] = h.y;
+      const int l = (int)fdiv((unsigned)i, dn), x = i - l * n;
+      const fxc h = A[i];
+      dst[(2 * l) * dfs + x] = fx_to(h.x, fs[2 * l]);
+      if (2 * l + 1 < nq) dst[(2 * l + 1) * dfs + x] = fx_to(h.y, fs[2 * l + 1]);
     }
   } else {
+    const int nl = (nf + 1) / 2;
     const double* src = J.srcR + b * J.src_mstride + (long long)row * J.src_rstep * n;
-    for (int i = tid; i < nl * n; i += nt) {
-      const int l = (int)fdiv((unsigned)i, fast_div((unsigned)n)), x = i - l * n;
-      const double fa = src[(2 * l) * J.src_fstride + x];
-      const double fb = (2 * l + 1 < nf) ? src[(2 * l + 1) * J.src_fstride + x] : 0.0;
-      A[i] = make_double2(fa, fb);
+    for (int l = tid >> 5; l < nl; l += nw) {
+      fxc* h = A + l * n;
+      for (int x = lane; x < n; x += 32)
+        h[x] = fx_bits(src[(2 * l) * J.src_fstride + x], (2 * l + 1 < nf) ? src[(2 * l + 1) * J.src_fstride + x] : 0.0);
+      __syncwarp();
+      const double2 r = fx_fields(h, n, fs[2 * l], fs[2 * l + 1]);
+      if (lane == 0) ref[l] = r;
     }
     __syncthreads();
-    double2* res = fft_lines<-1, double2, true>(A, Bb, nl, n, J.pl);
+    fx_lines<-1, true>(A, nl, n, &J.pl, false);
     double2* dst = J.dstC + b * J.dst_mstride + (long long)row * J.dst_rstep * K;
     const double inv = 1.0 / n;
-    for (int i = tid; i < nl * K; i += nt) {
-      const int l = (int)fdiv((unsigned)i, fast_div((unsigned)K)), k = i - l * K;
-      const double2 hk = res[l * n + k];
-      const double2 hm = cconj(res[l * n + (k == 0 ? 0 : n - k)]);
-      // F = (hk + conj(h_{-k}))/2, G = (hk - conj(h_{-k}))/(2i)
-      const double2 F = cscl(cadd(hk, hm), 0.5 * inv);
-      const double2 d = csub(hk, hm);
-      const double2 G = make_double2(0.5 * inv * d.y, -0.5 * inv * d.x);
-      dst[(2 * l) * J.dst_fstride + k] = F;
-      if (2 * l + 1 < nf) dst[(2 * l + 1) * J.dst_fstride + k] = G;
-    }
+    for (int l = tid >> 5; l < nl; l += nw)
+      for (int k = lane; k < K; k += 32) {
+        dst[(2 * l) * J.dst_fstride + k] = cscl(fx_mode_f(A + l * n, n, k, fs[2 * l], ref[l].x), inv);
+        if (2 * l + 1 < nf)
+          dst[(2 * l + 1) * J.dst_fstride + k] = cscl(fx_mode_g(A + l * n, n, k, fs[2 * l + 1], ref[l].y), inv);
+      }
   }
 }
 
 
-__global__ void __launch_bounds__(256) k_xrows(XJob J) { xrows_block(J, this_blk()); }
+constexpr int kFxThreads = 256;   // threads per block of the 2D fixed-point x pass, at most
 
-__global__ void __launch_bounds__(256) k_xrows_multi(const XJob* __restrict__ jobs, MultiMap mm) {
+__global__ void __launch_bounds__(256, 3) k_xrows(const __grid_constant__ XJob J) { xrows_block(J, this_blk()); }
+
+__global__ void __launch_bounds__(256, 3) k_xrows_multi(const XJob* __restrict__ jobs, MultiMap mm) {
   Blk bk;
   const int q = multi_locate(mm, bk);
   xrows_block(jobs[q], bk);

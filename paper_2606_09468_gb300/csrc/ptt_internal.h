@@ -9,40 +9,31 @@
 
 namespace ptt {
 
-constexpr int kMaxStages = 16;
+constexpr int kMaxStages = 8;    // passes of a plan (n <= 1080: at most 7)
 constexpr int kRing = 1024;       // diagnostics records kept per member
 constexpr int kNumHist = 4;       // SBDF4 history depth
 
-// Mixed-radix (2, 3, 4, 5, 7, 11, 13) Stockham FFT plan of length n.
+// Mixed-radix Stockham FFT plan of length n: FP32 plans of radices 2 to 5 and
+// 8, fixed-point plans of 2 to 8, 11 and 13.
 struct FftPlan {
   int n;
   int nst;
   int radix[kMaxStages];
-  const double2* tw;  // tw[k] = exp(-2 pi i k / n), k < n (device)
-  const float2* twf;  // the same in single precision (mixed groups), or null
-  const float4* twd;  // the same in double-single, (re.h, re.l, im.h, im.l) with
-                      // re = re.h + re.l (PTT_FP64_DS groups), or null
-  // Tangent-form twiddles of the FP64 passes s >= 1 of radix 2 to 5 (null:
-  // use tw; passes of radix 7, 11, 13 always use tw).  Forward
-  // twiddle r of stride index jm:
-  //   exp(-2 pi i jm r st / n) = i^k_r cos(t'_r) (1 + i tan(t'_r)), |t'_r| <= pi/4,
-  // record jm of pass s at tt[tto[s] + RS jm] (RS = 16 for radix 5, else 6),
-  // quadrants k_r packed in tk[toff[s] + jm] (2 bits each).  Records:
-  // radix 5 (tan1..tan4, cos4/cos1, cos3/cos2, cos1, cos2, C1 cos1, C2 cos2,
-  // C2 cos1, C1 cos2, S1 cos1, S2 cos2, S2 cos1, S1 cos2 with C_q, S_q the
-  // cosine and sine of 2 pi q/5); radix 4 (tan1, tan2, tan3, cos1, cos2,
-  // cos3/cos1); radix 3 (tan1, tan2, cos1, cos2/cos1, cos1/2,
-  // sin(2 pi/3) cos1); radix 2 (tan1, cos1).
-  const double* tt;
-  const int* tk;
-  int toff[kMaxStages];
-  int tto[kMaxStages];
+  const float2* twf;  // FP32: twf[k] = exp(-2 pi i k / n), k < n (device), or null
+  // Fixed point (ptt_fx.cuh): the twiddles of passes s >= 1, entry
+  // [r - 1][jm] (1 <= r < radix, jm < Ns) of pass s at twx[xoff[s] + (r - 1) Ns + jm]:
+  // exp(-2 pi i jm r st / n) as (cos high, cos low, sin high, sin low), 62
+  // fractional bits each; or null.
+  const int4* twx;
+  int xoff[kMaxStages];
   // Per-pass constants (plan_pass_consts): butterflies per line n/R, twiddle
   // stride n/(Ns R), span Ns before the pass, and the multiply-high
   // reciprocals of n/R and Ns (0 for 1), so that a pass divides nothing.
   int pnb[kMaxStages], pst[kMaxStages], pns[kMaxStages];
   unsigned pmb[kMaxStages], pms[kMaxStages];
 };
+// Butterflies of radix R held by a thread in a fixed-point pass.
+__host__ __device__ constexpr int fx_mb(int R) { return R == 2 ? 2 : 1; }
 // Fills the per-pass constants of pl from pl.n, pl.nst and pl.radix.
 void plan_pass_consts(FftPlan& pl);
 
@@ -74,10 +65,6 @@ struct GroupDev {
   int xthreads;      // threads per block of the fused x kernels (ptt_autotune)
   int zC;            // 3D: x-mode lines per block of the z passes (ptt_autotune)
   int f32;           // 1: mixed precision (FP32 transforms and products)
-  int ds;            // 1: FP64-accurate transforms and products in double-single
-                     //    arithmetic on the FP32 pipe (PTT_FP64_DS); the arrays are
-                     //    those of an FP64 group, the padded-grid intermediates
-                     //    holding double-single values
   int nx, K, N;      // Fourier points / modes (K = nx/2), Chebyshev modes
   int nz, Mz, KZ;    // z modes (1 in 2D), padded z points, modes per Chebyshev index (K * nz)
   double invMx;      // 1 / Mx (host-computed), and its FP32 rounding
@@ -138,22 +125,23 @@ struct GroupDev {
   double* statout;   // [kMacc] results of the window-statistics kernels (one call at a time)
   double* stage;     // [5][N][nx] host<->device staging (one member at a time)
   double2* stageS;   // [5][N][K]  values on the unpadded y grid, x analysed
-  // quarter-period twiddles of the Gauss-grid transforms, with the constant
-  // factors of each direction folded in:
-  const double2* tw4P;   // [M]  forward: (s_k/2) exp(-i pi k/(2M)), s_0 = 1/M, s_k = 2/M
-  const float2* tw4Pf;   // the same in single precision (mixed groups)
-  const double2* tw4Pi;  // [M]  inverse: (1/2) exp(+i pi k/(2M))
-  const float2* tw4Pif;  // the same in single precision (mixed groups)
-  const double2* tw4E;   // [Me] inverse on the diagnostic Gauss grid: (1/2) exp(+i pi k/(2Me))
-  const float2* tw4Ef;   // the same in single precision (mixed groups: FP32 energy transform)
-  const float4* tw4Pd;   // double-single forward, inverse and diagnostic tables
-  const float4* tw4Pid;  // (PTT_FP64_DS groups)
-  const float4* tw4Ed;
+  // quarter-period twiddles of the Gauss-grid transforms.  FP32, with the
+  // constant factors of each direction folded in:
+  const float2* tw4Pf;   // [M]  forward: (s_k/2) exp(-i pi k/(2M)), s_0 = 1/M, s_k = 2/M
+  const float2* tw4Pif;  // [M]  inverse: (1/2) exp(+i pi k/(2M))
+  const float2* tw4Ef;   // [Me] inverse on the diagnostic Gauss grid (mixed groups)
+  // Fixed point (as FftPlan::twx): forward [M] h_k q exp(-i pi k/(2M)), h_0 = 1/2,
+  // h_k = 1, q = 2^fexpP / (the normalisation of the whole forward transform:
+  // M Mx Mz, or M for the mean column of a mixed group) in (1/2, 1]; inverse
+  // exp(+i pi k/(2M)) on the padded and the diagnostic grid
+  const int4* tw4Px;
+  const int4* tw4Pix;
+  const int4* tw4Ex;     // [Me] (null in mixed groups)
+  int fexpP;
   FftPlan plP, plMx, plNx, plPu, plPe;   // lengths M, Mx, nx, 2(N-1), Me
   FftPlan plMz, plNz;                    // 3D: lengths Mz, nz
-  FftPlan plPn;      // mixed groups: length M with radices up to 5 (the
-                     // double-single passes of the mean column; plP may
-                     // hold radix-8 passes there)
+  FftPlan plPn;      // length M in fixed point (mixed groups: the mean column; plP
+                     // is an FP32 plan there)
 };
 
 constexpr int kPart = 48;  // values per diagnostics tile
@@ -243,13 +231,11 @@ cudaError_t launch_explicit3(const GroupDev& g, cudaStream_t st);
 cudaError_t launch_phys_to_state3(const GroupDev& g, int b, cudaStream_t st);
 cudaError_t launch_state_to_phys3(const GroupDev& g, int b, cudaStream_t st);
 cudaError_t launch_reset_member3(const GroupDev& g, int b, cudaStream_t st);
-// Shared memory of the 3D fused x pass: two buffers of 18 lines, or one
-// (in-place passes, 512 threads) where two do not fit and one does (FP64,
-// Mx <= 768); 0 when neither fits.
+// Shared memory of the 3D fused x pass (18 lines: two FP32 buffers, or one in
+// fixed point); 0 when it does not fit.
 size_t smem_xfused3(int Mx, int f32);
-bool xfused3_inplace(int Mx, int f32);
 size_t spec3_scratch_columns();
-size_t smem_zcols3(int C, int Mz, int f32);
+size_t smem_zcols3(int C, int Mz);
 
 // Tensor-core Chebyshev passes of mixed groups (ptt_mma.cu).
 bool cheb_mma_supported(int M, int N);
@@ -260,13 +246,15 @@ cudaError_t launch_cheb_mma(const GroupDev& g, bool inverse, cudaStream_t st, in
 
 // Host helpers (ptt_capi.cu) used by the workspace-free entry point.
 void set_last_error(const char* msg);
-// tt[0], tk[0] / tt[1], tk[1]: tangent-form twiddle records of the padded
-// Chebyshev and padded x plans (FftPlan::tt, ::tk).
-int shape_plan(const ptt_params& p, GroupDev& d, std::vector<double2>& twP,
-               std::vector<double2>& twMx, std::vector<double2>& tw4, MemberPrm& prm,
-               std::vector<double>* tt, std::vector<int>* tk);
+// Sizes and plans of an FP64 2D shape with its tables packed in one array
+// (the offsets of the fixed-point twiddles of the padded Chebyshev and x plans
+// and of the two quarter-period tables in `off`).
+int shape_plan(const ptt_params& p, GroupDev& d, std::vector<int4>& tables, size_t (&off)[4],
+               MemberPrm& prm);
 
-size_t smem_ycols(int C, int P, int f32);
+size_t smem_ycols(int C, int P);               // FP32
+size_t smem_ycols_fx(int C, int P, int Nd);    // fixed point; Nd: ny where derivatives are taken, else 0
+constexpr size_t kSmemMax = 227 * 1024;        // shared memory of a block
 size_t smem_xfused(int Mx, int f32);
 size_t smem_xrows(int nl, int n);
 size_t smem_spec(int N);

@@ -1,10 +1,10 @@
-// Device code of the FP64 pseudo-spectral sPTT channel step (2D, sm_103a).
+// Device code of the 2D pseudo-spectral sPTT channel step (sm_103a).
 //
 // One step (Sec. 2: fully dealiased Fourier-Chebyshev pseudo-spectral method,
 // fourth-order semi-implicit BDF) is the launch sequence
-//   k_ycols  (inverse)  spectral (m, n) -> values on the padded Gauss-Lobatto
-//                       y grid, with d/dy by the Chebyshev recurrence
-//   k_xfused            per padded y row: inverse x FFTs of 14 fields, the
+//   k_ycols  (inverse)  spectral (m, n) -> values on the padded Gauss y grid,
+//                       with d/dy by the Chebyshev recurrence
+//   k_xfused(_fx)       per padded y row: inverse x FFTs of 14 fields, the
 //                       sPTT / advection products of Eqs. 1-2, forward x FFTs
 //   k_ycols  (forward)  padded y values -> Chebyshev coefficients (truncated)
 //   k_spec              per Fourier mode, out of shared memory: linear
@@ -12,9 +12,9 @@
 //                       quasi-tridiagonal tau solves, u from continuity
 //   k_tick              step counters
 // followed by the diagnostics of Sec. 3 (k_ycols x2, k_xrows, k_diag_part,
-// k_diag_count, k_diag_mid, k_diag_final).  All transforms are mixed-radix (2, 3, 4, 5) Stockham FFTs
-// in shared memory; the Chebyshev transforms are discrete cosine transforms
-// of type I computed as FFTs of the even extension.
+// k_diag_count, k_diag_mid, k_diag_final).  All transforms are mixed-radix
+// Stockham FFTs in shared memory: FP32 in the mixed groups' step, 64-bit block
+// fixed point (ptt_fx.cuh) where FP64 accuracy is wanted.
 //
 // Layouts: spectral arrays [member][field][m][n] (each mode's Chebyshev
 // column contiguous); values on a y grid [member][field][j][m] (each y row's
@@ -33,17 +33,6 @@ namespace {
 // (cxx_y, cxy_y) (cyy_y, cxx_x) (cxy_x, cyy_x).
 __constant__ int c_xsrc[14] = {0, 1, 2, 0, 1, 3, 4, 5, 6, 7, 8, 3, 4, 5};
 __constant__ int c_xik[14] = {0, 0, 0, 1, 1, 0, 0, 0, 0, 0, 0, 1, 1, 1};
-
-template <typename C2> __device__ __forceinline__ const C2* yp_ptr(const GroupDev& g);
-template <> __device__ __forceinline__ const double2* yp_ptr<double2>(const GroupDev& g) { return g.Yp; }
-template <> __device__ __forceinline__ const float2* yp_ptr<float2>(const GroupDev& g) { return g.Ypf; }
-template <> __device__ __forceinline__ const dsc* yp_ptr<dsc>(const GroupDev& g) {
-  return reinterpret_cast<const dsc*>(g.Yp);
-}
-template <typename C2> __device__ __forceinline__ C2* zp_ptr(const GroupDev& g);
-template <> __device__ __forceinline__ double2* zp_ptr<double2>(const GroupDev& g) { return g.Zp; }
-template <> __device__ __forceinline__ float2* zp_ptr<float2>(const GroupDev& g) { return g.Zpf; }
-template <> __device__ __forceinline__ dsc* zp_ptr<dsc>(const GroupDev& g) { return reinterpret_cast<dsc*>(g.Zp); }
 
 // The products of Eqs. 1-2 at one point of the padded grid, from the 14
 // physical fields q = (u, v, du/dy, du/dx, dv/dx, c_xx, c_xy, c_yy, dc_xx/dy,
@@ -64,17 +53,107 @@ __device__ __forceinline__ void products2d(const T (&q)[14], T eps, T iwi, T (&o
   o[4] = -(u * vx - v * ux);
 }
 
-// C2 = double2: the FP64 path; C2 = float2: the mixed path (FP32 transforms
-// and products, FP64 state and solves); C2 = dsc: the double-single path
-// (FP64-accurate transforms and products on the FP32 pipe, PTT_FP64_DS).
-// Mixed groups split the products into mean and fluctuation parts (mfl):
-// the FP32 lines carry the fluctuations (their mean mode kk = 0 left out),
-// the row's means come in FP64 from g.Ym, the mean products are formed once
-// per row in FP64, and the mean column of the explicit terms goes to g.Zm
-// in FP64 (the FP32 output's mean mode is left zero).
-template <typename C2>
+// The same in FP64 with the fewest FP64 instructions (21 against 30; each
+// holds the pipe for 64 cycles): every output one chain of fused
+// multiply-adds, the "+ rw" of -(c - 1) rw and the constants of the relaxation
+// factor folded into its start, factors 2 as exponent increments on the
+// integer pipe.  e1 = eps/Wi, e0 = (1 - 2 eps)/Wi.
+__device__ __forceinline__ double twice(double x) {   // 2 x by the exponent
+  const int h = __double2hiint(x);
+  const bool n = (h & 0x7FF00000) != 0 && (h & 0x7FF00000) < 0x7FE00000;
+  return n ? __hiloint2double(h + 0x100000, __double2loint(x)) : x + x;
+}
+__device__ __forceinline__ void products2d_fp64(const double (&q)[14], double e1, double e0, double (&o)[5]) {
+  const double u = q[0], v = q[1], uy = q[2], ux = q[3], vx = q[4], cxx = q[5], cxy = q[6], cyy = q[7];
+  const double ux2 = twice(ux), uy2 = twice(uy), vx2 = twice(vx);
+  const double rw = fma(e1, cxx + cyy, e0);
+  o[0] = fma(-cxx, rw, fma(uy2, cxy, fma(ux2, cxx, fma(-v, q[8], fma(-u, q[11], rw)))));
+  o[1] = fma(-cxy, rw, fma(vx, cxx, fma(uy, cyy, fma(-v, q[9], -u * q[12]))));
+  o[2] = fma(-cyy, rw, fma(-ux2, cyy, fma(vx2, cxy, fma(-v, q[10], fma(-u, q[13], rw)))));
+  o[3] = fma(-v, uy, -u * ux);
+  o[4] = fma(v, ux, -u * vx);
+}
+
+// FP64-accurate form: fixed-point transforms (ptt_fx.cuh) between FP64 arrays,
+// products in FP64.  Seven lines of Mx in one shared-memory buffer.  Zp is
+// left without its 1/Mx (the y table's normalisation holds it).  Bound by
+// instruction issue and latency: four blocks of 256 threads per SM (64
+// registers) take 0.70 ms over the 27-run sweep, three 0.74, five 0.79 (FP64
+// lines on the FP64 pipe: 1.84).
+__device__ __forceinline__ void xfused_fx_block(const GroupDev& g, Blk bk) {
+  const int b = bk.y;
+  if (g.status[b]) return;
+  const int j = bk.x;
+  const int K = g.K, Mx = g.Mx, rows = g.M;
+  const MemberPrm pr = g.prm[b];
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ FxS fs[14], fo[6];
+  __shared__ double2 ref[3];
+  fxc* A = reinterpret_cast<fxc*>(smraw);
+  const double2* Y = g.Yp + (size_t)b * 9 * rows * K + (size_t)j * K;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, nw = nt >> 5;
+  // a warp per line: its two fields' modes (x-derivatives i k), then their
+  // scales and the packed line; the padded middle is zero
+  for (int l = tid >> 5; l < 7; l += nw) {
+    fxc* h = A + l * Mx;
+    const double2* yF = Y + (size_t)c_xsrc[2 * l] * rows * K;
+    const double2* yG = Y + (size_t)c_xsrc[2 * l + 1] * rows * K;
+    const int dF = c_xik[2 * l], dG = c_xik[2 * l + 1];
+    unsigned mF = 0u, mG = 0u;
+#pragma unroll 2
+    for (int k = lane; k < K; k += 32) {
+      double2 F = yF[k], G = yG[k];
+      if (k == 0) { F.y = 0; G.y = 0; }
+      if (dF) F = cscl(mul_i(F), pr.kx1 * k);
+      if (dG) G = cscl(mul_i(G), pr.kx1 * k);
+      h[k] = fx_bits(F.x, F.y);
+      h[fx_xslot(1, k, K, Mx)] = fx_bits(G.x, G.y);
+      mF = max(mF, fx_mag2(F));
+      mG = max(mG, fx_mag2(G));
+    }
+    for (int k = K + 1 + lane; k <= Mx - K; k += 32) h[k] = fx_zero();
+    __syncwarp();
+    fx_xline(h, Mx, K, mF, mG, fs[2 * l], fs[2 * l + 1]);
+  }
+  __syncthreads();
+  fx_lines<+1, false>(A, 7, Mx, &g.plMx, g.plMx.radix[0] % 3 == 0);
+  const double e1 = pr.eps * pr.inv_wi, e0 = (1.0 - 2.0 * pr.eps) * pr.inv_wi;
+  for (int x = tid; x < Mx; x += nt) {
+    double q[14], o[5];
+#pragma unroll
+    for (int l = 0; l < 7; ++l) {
+      const fxc h = A[l * Mx + x];
+      q[2 * l] = fx_to(h.x, fs[2 * l]);
+      q[2 * l + 1] = fx_to(h.y, fs[2 * l + 1]);
+    }
+    products2d_fp64(q, e1, e0, o);
+    A[x] = fx_bits(o[0], o[1]);
+    A[Mx + x] = fx_bits(o[2], o[3]);
+    A[2 * Mx + x] = fx_bits(o[4], 0.0);
+  }
+  __syncthreads();
+  for (int l = tid >> 5; l < 3; l += nw) {
+    const double2 r = fx_fields(A + l * Mx, Mx, fo[2 * l], fo[2 * l + 1]);
+    if (lane == 0) ref[l] = r;
+  }
+  __syncthreads();
+  fx_lines<-1, false>(A, 3, Mx, &g.plMx, false);
+  double2* Z = g.Zp + (size_t)b * 5 * rows * K + (size_t)j * K;
+  const FastDiv dK = fast_div((unsigned)K);
+  for (int i = tid; i < 3 * K; i += nt) {
+    const int l = (int)fdiv((unsigned)i, dK), k = i - l * K;
+    Z[(size_t)(2 * l) * rows * K + k] = fx_mode_f(A + l * Mx, Mx, k, fo[2 * l], ref[l].x);
+    if (l < 2) Z[(size_t)(2 * l + 1) * rows * K + k] = fx_mode_g(A + l * Mx, Mx, k, fo[2 * l + 1], ref[l].y);
+  }
+}
+
+// Mixed form: FP32 transforms, the products split into mean and fluctuation
+// parts (mfl): the FP32 lines carry the fluctuations (their mean mode kk = 0
+// left out), the row's means come in FP64 from g.Ym, the mean products are
+// formed once per row in FP64, and the mean column of the explicit terms goes
+// to g.Zm in FP64 (the FP32 output's mean mode is left zero).
 __device__ __forceinline__ void xfused_block(const GroupDev& g, Blk bk) {
-  using T = typename RealOf<C2>::T;
+  using C2 = float2;
   const int b = bk.y;
   if (g.status[b]) return;
   const int j = bk.x;
@@ -83,13 +162,12 @@ __device__ __forceinline__ void xfused_block(const GroupDev& g, Blk bk) {
   extern __shared__ __align__(16) unsigned char smraw[];
   C2* A = reinterpret_cast<C2*>(smraw);
   C2* B = A + 7 * Mx;
-  const C2* Y = yp_ptr<C2>(g) + (size_t)b * 9 * rows * K + (size_t)j * K;
-  const T kfac = as_prec<T>(pr.kx1, pr.kx1f);
+  const C2* Y = g.Ypf + (size_t)b * 9 * rows * K + (size_t)j * K;
+  const float kfac = pr.kx1f;
   const int tid = threadIdx.x, nt = blockDim.x;
-  constexpr bool kSplit = std::is_same<C2, float2>::value;
-  __shared__ float s_mq[14];    // the row's means as FP32 multipliers (split)
-  __shared__ double s_nb[5];    // the row's mean products (split)
-  if constexpr (kSplit) {
+  __shared__ float s_mq[14];    // the row's means as FP32 multipliers
+  __shared__ double s_nb[5];    // the row's mean products
+  {
     const double2* ym = g.Ym + (size_t)b * 9 * rows + j;
     if (tid < 14) s_mq[tid] = c_xik[tid] ? 0.f : (float)ym[(size_t)c_xsrc[tid] * rows].x;
     if (tid == 32) {   // another warp: the mean products, in FP64
@@ -132,9 +210,8 @@ __device__ __forceinline__ void xfused_block(const GroupDev& g, Blk bk) {
         if (it >= nitem) continue;
         const int l = (int)fdiv((unsigned)it, dK), kk = it - l * K;
         C2 f = F[u], gg = G[u];
-        if (kk == 0) { f.y = 0; gg.y = 0; }
-        if (kSplit && kk == 0) { f.x = 0; gg.x = 0; }   // the mean is in g.Ym
-        const T km = kfac * kk;
+        if (kk == 0) f = gg = zero2<C2>();   // the mean is in g.Ym
+        const float km = kfac * kk;
         if (c_xik[2 * l]) f = cscl(mul_i(f), km);
         if (c_xik[2 * l + 1]) gg = cscl(mul_i(gg), km);
         A[l * Mx + kk] = cadd(f, mul_i(gg));
@@ -147,73 +224,53 @@ __device__ __forceinline__ void xfused_block(const GroupDev& g, Blk bk) {
   // when Mx has no factor 5)
   C2* res = fft_lines<+1>(A, B, 7, Mx, g.plMx, g.plMx.radix[0] == 3);
   C2* oth = (res == A) ? B : A;
-  const T eps = as_prec<T>(pr.eps, pr.epsf), iwi = as_prec<T>(pr.inv_wi, pr.inv_wif);
   for (int x = tid; x < Mx; x += nt) {
-    T o[5];
-    if constexpr (kSplit) {
-      mfl q[14], om[5];
+    mfl q[14], om[5];
 #pragma unroll
-      for (int l = 0; l < 7; ++l) {
-        const C2 h = res[l * Mx + x];
-        q[2 * l] = mfl(s_mq[2 * l], h.x);
-        q[2 * l + 1] = mfl(s_mq[2 * l + 1], h.y);
-      }
-      products2d<mfl>(q, mfl(pr.epsf, 0.f), mfl(pr.inv_wif, 0.f), om);
-#pragma unroll
-      for (int i = 0; i < 5; ++i) o[i] = om[i].f;
-    } else {
-      T q[14];
-#pragma unroll
-      for (int l = 0; l < 7; ++l) {
-        const C2 h = res[l * Mx + x];
-        q[2 * l] = h.x;
-        q[2 * l + 1] = h.y;
-      }
-      products2d<T>(q, eps, iwi, o);
+    for (int l = 0; l < 7; ++l) {
+      const C2 h = res[l * Mx + x];
+      q[2 * l] = mfl(s_mq[2 * l], h.x);
+      q[2 * l + 1] = mfl(s_mq[2 * l + 1], h.y);
     }
-    C2 o0, o1, o2;
-    o0.x = o[0]; o0.y = o[1];
-    o1.x = o[2]; o1.y = o[3];
-    o2.x = o[4]; o2.y = 0;
-    oth[x] = o0;
-    oth[Mx + x] = o1;
-    oth[2 * Mx + x] = o2;
+    products2d<mfl>(q, mfl(pr.epsf, 0.f), mfl(pr.inv_wif, 0.f), om);
+    oth[x] = make_float2(om[0].f, om[1].f);
+    oth[Mx + x] = make_float2(om[2].f, om[3].f);
+    oth[2 * Mx + x] = make_float2(om[4].f, 0.f);
   }
   __syncthreads();
   C2* r2 = fft_lines<-1>(oth, res, 3, Mx, g.plMx);
-  C2* Z = zp_ptr<C2>(g) + (size_t)b * 5 * rows * K + (size_t)j * K;
-  const T inv = as_prec<T>(g.invMx, g.invMxf);
+  C2* Z = g.Zpf + (size_t)b * 5 * rows * K + (size_t)j * K;
+  const float inv = g.invMxf;
   for (int i = tid; i < 3 * K; i += nt) {
     const int l = (int)fdiv((unsigned)i, fast_div((unsigned)K)), k = i - l * K;
     const C2 hk = r2[l * Mx + k];
     const C2 hm = cconj(r2[l * Mx + (k == 0 ? 0 : Mx - k)]);
-    C2 F = cscl(cadd(hk, hm), (T)0.5 * inv);
+    C2 F = cscl(cadd(hk, hm), 0.5f * inv);
     const C2 d = csub(hk, hm);
-    C2 G;
-    G.x = (T)0.5 * inv * d.y;
-    G.y = (T)-0.5 * inv * d.x;
-    if constexpr (kSplit) {
-      if (k == 0) {   // mean column: the mean products plus the fluctuations' mean, FP64
-        double2* zm = g.Zm + (size_t)b * 5 * rows + j;
-        zm[(size_t)(2 * l) * rows] = make_double2(s_nb[2 * l] + (double)F.x, 0.0);
-        if (l < 2) zm[(size_t)(2 * l + 1) * rows] = make_double2(s_nb[2 * l + 1] + (double)G.x, 0.0);
-        F = zero2<C2>();
-        G = zero2<C2>();
-      }
+    C2 G = make_float2(0.5f * inv * d.y, -0.5f * inv * d.x);
+    if (k == 0) {   // mean column: the mean products plus the fluctuations' mean, FP64
+      double2* zm = g.Zm + (size_t)b * 5 * rows + j;
+      zm[(size_t)(2 * l) * rows] = make_double2(s_nb[2 * l] + (double)F.x, 0.0);
+      if (l < 2) zm[(size_t)(2 * l + 1) * rows] = make_double2(s_nb[2 * l + 1] + (double)G.x, 0.0);
+      F = zero2<C2>();
+      G = zero2<C2>();
     }
     Z[(size_t)(2 * l) * rows * K + k] = F;
     if (l < 2) Z[(size_t)(2 * l + 1) * rows * K + k] = G;
   }
 }
 
-template <typename C2>
-__global__ void __launch_bounds__(512) k_xfused(GroupDev g) { xfused_block<C2>(g, this_blk()); }
-
-template <typename C2>
+__global__ void __launch_bounds__(512) k_xfused(GroupDev g) { xfused_block(g, this_blk()); }
 __global__ void __launch_bounds__(512) k_xfused_multi(const GroupDev* __restrict__ gs, MultiMap mm) {
   Blk bk;
   const int q = multi_locate(mm, bk);
-  xfused_block<C2>(gs[q], bk);
+  xfused_block(gs[q], bk);
+}
+__global__ void __launch_bounds__(kFxThreads, 4) k_xfused_fx(const __grid_constant__ GroupDev g) { xfused_fx_block(g, this_blk()); }
+__global__ void __launch_bounds__(kFxThreads, 4) k_xfused_fx_multi(const GroupDev* __restrict__ gs, MultiMap mm) {
+  Blk bk;
+  const int q = multi_locate(mm, bk);
+  xfused_fx_block(gs[q], bk);
 }
 
 // The tau system solved per (mode, system, parity) by warp_qt_solve:
@@ -650,7 +707,8 @@ __device__ __forceinline__ void diag_final_block(const GroupDev& g, Blk bk) {
   const int b = bk.x;
   if (g.status[b]) return;
   __shared__ double sh[32];
-  extern __shared__ double2 dsm[];
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ FxS fs[6];
   const int K = g.K, N = g.N, nx = g.nx;
   const size_t NK = (size_t)N * K;
   const MemberPrm pr = g.prm[b];
@@ -681,26 +739,39 @@ __device__ __forceinline__ void diag_final_block(const GroupDev& g, Blk bk) {
     if ((n & 1) == 0) mt += (X[2 * NK + n].x + X[4 * NK + n].x) * (2.0 / (1.0 - (double)n * n));
   mt = block_sum(mt, sh);
   // mid-plane lines from the per-mode sums: (Tr c, u') (v, du/dx) (dv/dx, du/dy)
-  double2* L = dsm;              // 3 lines of nx
-  double2* L2 = dsm + 3 * nx;    // ping-pong
+  fxc* A = reinterpret_cast<fxc*>(smraw);          // 3 lines of nx
   const double kfac = 2.0 * 3.14159265358979323846 / pr.lx;
-  for (int i = threadIdx.x; i < 3 * nx; i += blockDim.x) L[i] = czero();
-  __syncthreads();
   const double2* DM = g.DM + (size_t)b * 4 * K;
-  for (int m = threadIdx.x; m < K; m += blockDim.x) {
-    double2 tr = DM[m], u = DM[K + m], v = DM[2 * K + m], uy = DM[3 * K + m];
-    const double km = kfac * m;
-    double2 ux = cscl(mul_i(u), km), vx = cscl(mul_i(v), km);
-    if (m == 0) { tr.x += 1.0; u = czero(); tr.y = v.y = uy.y = 0.0; ux = vx = czero(); }
-    const double2 F[6] = {tr, u, v, ux, vx, uy};
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      L[l * nx + m] = cadd(F[2 * l], mul_i(F[2 * l + 1]));
-      if (m > 0) L[l * nx + nx - m] = cadd(cconj(F[2 * l]), mul_i(cconj(F[2 * l + 1])));
+  if (threadIdx.x < 96) {   // a warp per line
+    const int l = threadIdx.x >> 5;
+    fxc* h = A + l * nx;
+    unsigned mF = 0u, mG = 0u;
+    for (int m = threadIdx.x & 31; m < K; m += 32) {
+      const double km = kfac * m;
+      double2 F, G;
+      if (l == 0) {
+        F = DM[m];
+        G = DM[K + m];
+        if (m == 0) { F.x += 1.0; F.y = 0.0; G = czero(); }
+      } else if (l == 1) {
+        F = DM[2 * K + m];
+        G = cscl(mul_i(DM[K + m]), km);
+        if (m == 0) { F.y = 0.0; G = czero(); }
+      } else {
+        F = cscl(mul_i(DM[2 * K + m]), km);
+        G = DM[3 * K + m];
+        if (m == 0) { F = czero(); G.y = 0.0; }
+      }
+      h[m] = fx_bits(F.x, F.y);
+      h[fx_xslot(1, m, K, nx)] = fx_bits(G.x, G.y);
+      mF = max(mF, fx_mag2(F));
+      mG = max(mG, fx_mag2(G));
     }
+    __syncwarp();
+    fx_xline(h, nx, K, mF, mG, fs[2 * l], fs[2 * l + 1]);
   }
   __syncthreads();
-  double2* res = fft_lines<+1, double2, true>(L, L2, 3, nx, g.plNx);
+  fx_lines<+1, true>(A, 3, nx, &g.plNx, false);
   // mid-plane histograms of the 6 quantities (shared-memory counts)
   constexpr int HS = PTT_HIST_BINS + 2;
   __shared__ unsigned int hsm[6 * HS];
@@ -720,7 +791,11 @@ __device__ __forceinline__ void diag_final_block(const GroupDev& g, Blk bk) {
   for (int x = threadIdx.x; x < nx; x += blockDim.x) {
     double q[6];
 #pragma unroll
-    for (int l = 0; l < 3; ++l) { q[2 * l] = res[l * nx + x].x; q[2 * l + 1] = res[l * nx + x].y; }
+    for (int l = 0; l < 3; ++l) {
+      const fxc h = A[l * nx + x];
+      q[2 * l] = fx_to(h.x, fs[2 * l]);
+      q[2 * l + 1] = fx_to(h.y, fs[2 * l + 1]);
+    }
     if (hon) {
 #pragma unroll
       for (int qq = 0; qq < 6; ++qq) {
@@ -791,7 +866,7 @@ __global__ void __launch_bounds__(256) k_diag_mid_multi(const GroupDev* __restri
   const int q = multi_locate(mm, bk);
   diag_mid_block(gs[q], bk);
 }
-__global__ void __launch_bounds__(256) k_diag_final(GroupDev g) { diag_final_block(g, this_blk()); }
+__global__ void __launch_bounds__(256) k_diag_final(const __grid_constant__ GroupDev g) { diag_final_block(g, this_blk()); }
 __global__ void __launch_bounds__(256) k_diag_final_multi(const GroupDev* __restrict__ gs, MultiMap mm) {
   Blk bk;
   const int q = multi_locate(mm, bk);
@@ -897,12 +972,12 @@ __global__ void k_reset(GroupDev g, int b) {
 // Spectral coefficients (internal layout [member][field][m][n]) <-> values on
 // a y grid stored [member][field][j][m].
 YJob make_yjob(const GroupDev& g, bool inverse, int M, int C, const FftPlan& pl,
-               const double2* tw4 = nullptr) {
+               bool gauss = false) {
   YJob J{};
-  J.gauss = tw4 ? 1 : 0;
-  J.tw4 = tw4;  // the quarter-period table of this direction
-  J.tw4f = inverse ? g.tw4Pif : g.tw4Pf;
-  J.tw4d = inverse ? g.tw4Pid : g.tw4Pd;
+  J.gauss = gauss ? 1 : 0;
+  J.tw4f = inverse ? g.tw4Pif : g.tw4Pf;   // the quarter-period tables of this direction
+  J.tw4x = inverse ? g.tw4Pix : g.tw4Px;
+  J.fexp = g.fexpP;
   J.K = g.K;
   J.N = g.N;
   J.M = M;
@@ -945,11 +1020,12 @@ cudaError_t launch_hist_l1(const unsigned long long* ha, const unsigned long lon
 }
 
 
-size_t smem_ycols(int C, int P, int f32) {
-  return (size_t)(2 * C * P + 2 * C) * (f32 ? sizeof(float2) : sizeof(double2));
+size_t smem_ycols(int C, int P) { return (size_t)2 * C * P * sizeof(float2); }
+size_t smem_ycols_fx(int C, int P, int Nd) { return (size_t)C * (P + Nd + 2) * sizeof(fxc); }
+size_t smem_xfused(int Mx, int f32) {
+  return f32 ? (size_t)14 * Mx * sizeof(float2) : (size_t)7 * Mx * sizeof(fxc);
 }
-size_t smem_xfused(int Mx, int f32) { return (size_t)14 * Mx * (f32 ? sizeof(float2) : sizeof(double2)); }
-size_t smem_xrows(int nl, int n) { return (size_t)2 * nl * n * sizeof(double2); }
+size_t smem_xrows(int nl, int n) { return (size_t)nl * n * sizeof(fxc); }
 size_t smem_spec(int N) { return (size_t)12 * N * sizeof(double2) + (size_t)10 * N * sizeof(double); }
 
 template <typename F>
@@ -963,27 +1039,21 @@ static cudaError_t optin(F* fn, int optin_bytes) {
 
 cudaError_t set_kernel_attributes(int optin_bytes) {
   cudaError_t e;
-  if ((e = optin(k_ycols<double2>, optin_bytes))) return e;
   if ((e = optin(k_ycols<float2>, optin_bytes))) return e;
-  if ((e = optin(k_ycols<dsc>, optin_bytes))) return e;
-  if ((e = optin(k_ycols<double2, true>, optin_bytes))) return e;
-  if ((e = optin(k_ycols<dsc, true>, optin_bytes))) return e;
-  if ((e = optin(k_ycols_multi<double2>, optin_bytes))) return e;
+  if ((e = optin(k_ycols<fxc>, optin_bytes))) return e;
+  if ((e = optin(k_ycols<fxc, true>, optin_bytes))) return e;
   if ((e = optin(k_ycols_multi<float2>, optin_bytes))) return e;
-  if ((e = optin(k_ycols_multi<double2, true>, optin_bytes))) return e;
-  if ((e = optin(k_xfused_multi<double2>, optin_bytes))) return e;
-  if ((e = optin(k_xfused_multi<float2>, optin_bytes))) return e;
-  if ((e = optin(k_xfused_multi<dsc>, optin_bytes))) return e;
-  if ((e = optin(k_ycols_multi<dsc>, optin_bytes))) return e;
-  if ((e = optin(k_ycols_multi<dsc, true>, optin_bytes))) return e;
+  if ((e = optin(k_ycols_multi<fxc>, optin_bytes))) return e;
+  if ((e = optin(k_ycols_multi<fxc, true>, optin_bytes))) return e;
+  if ((e = optin(k_xfused, optin_bytes))) return e;
+  if ((e = optin(k_xfused_multi, optin_bytes))) return e;
+  if ((e = optin(k_xfused_fx, optin_bytes))) return e;
+  if ((e = optin(k_xfused_fx_multi, optin_bytes))) return e;
   if ((e = optin(k_spec_multi<2>, optin_bytes))) return e;
   if ((e = optin(k_spec_multi<4>, optin_bytes))) return e;
   if ((e = optin(k_spec_multi<kMaxChunk>, optin_bytes))) return e;
   if ((e = optin(k_xrows_multi, optin_bytes))) return e;
   if ((e = optin(k_diag_final_multi, optin_bytes))) return e;
-  if ((e = optin(k_xfused<double2>, optin_bytes))) return e;
-  if ((e = optin(k_xfused<float2>, optin_bytes))) return e;
-  if ((e = optin(k_xfused<dsc>, optin_bytes))) return e;
   if ((e = optin(k_xrows, optin_bytes))) return e;
   if ((e = optin(k_spec<2>, optin_bytes))) return e;
   if ((e = optin(k_spec<4>, optin_bytes))) return e;
@@ -1010,9 +1080,9 @@ static void launch_spec(const GroupDev& g, int mode, cudaStream_t st) {
 // the per-group launches and the launches over all groups).
 static YJob yjob_inverse(const GroupDev& g) {   // 9 fields on the padded Gauss grid
   const size_t NK = (size_t)g.N * g.K;
-  YJob J = make_yjob(g, true, g.M, g.Ccol, g.plP, g.tw4Pi);
+  YJob J = make_yjob(g, true, g.M, g.Ccol, g.plP, true);
   J.src = g.X; J.dst = g.f32 ? (void*)g.Ypf : (void*)g.Yp;
-  J.dst_f32 = g.ds ? kFmtDS : g.f32;
+  J.dst_f32 = g.f32;
   J.src_mstride = 5 * NK; J.dst_mstride = 9LL * g.M * g.K;
   J.src_fstride = NK; J.dst_fstride = (long long)g.M * g.K;
   const int sf[9] = {0, 1, 0, 2, 3, 4, 2, 3, 4};
@@ -1022,18 +1092,17 @@ static YJob yjob_inverse(const GroupDev& g) {   // 9 fields on the padded Gauss 
 }
 static YJob yjob_forward(const GroupDev& g) {   // the 5 explicit fields to coefficients
   const size_t NK = (size_t)g.N * g.K;
-  YJob F = make_yjob(g, false, g.M, g.Ccol, g.plP, g.tw4P);
+  YJob F = make_yjob(g, false, g.M, g.Ccol, g.plP, true);
   F.src = g.f32 ? (const void*)g.Zpf : (const void*)g.Zp; F.dst = g.NR;
-  F.src_f32 = g.ds ? kFmtDS : g.f32;
+  F.src_f32 = g.f32;
   F.src_mstride = 5LL * g.M * g.K; F.dst_mstride = 5 * NK;
   F.src_fstride = (long long)g.M * g.K; F.dst_fstride = NK;
   for (int i = 0; i < 5; ++i) { F.src_field[i] = i; F.dst_field[i] = i; F.deriv[i] = 0; }
   return F;
 }
 // Mixed groups: the mean column (m = 0) of the inverse and forward y passes
-// in double-single, FP64 in and out (g.Ym, g.Zm; see xfused_block).  One
-// column per block; the narrow plan plPn (the double-single passes take
-// radices up to 5).
+// in fixed point, FP64 in and out (g.Ym, g.Zm; see xfused_block).  One
+// column per block.
 static YJob yjob_mean_inverse(const GroupDev& g) {
   YJob J = yjob_inverse(g);
   J.K = 1; J.C = 1; J.pl = g.plPn;
@@ -1052,9 +1121,9 @@ static YJob yjob_mean_forward(const GroupDev& g) {
 }
 static YJob yjob_energy(const GroupDev& g) {    // u, v on the Me Gauss points
   const size_t NK = (size_t)g.N * g.K;
-  YJob J = make_yjob(g, true, g.Me, g.CcolE, g.plPe, g.tw4E);
+  YJob J = make_yjob(g, true, g.Me, g.CcolE, g.plPe, true);
   J.tw4f = g.tw4Ef;   // mixed groups transform in FP32 (the sums stay FP64)
-  J.tw4d = g.tw4Ed;   // double-single groups in double-single
+  J.tw4x = g.tw4Ex;
   J.src = g.X; J.dst = g.DY;
   J.src_mstride = 5 * NK; J.dst_mstride = 2LL * g.Me * g.K;
   J.src_fstride = NK; J.dst_fstride = (long long)g.Me * g.K;
@@ -1077,7 +1146,7 @@ static XJob xjob_trc(const GroupDev& g) {       // Tr c rows to the unpadded x g
   X.src_fstride = 0; X.dst_fstride = 0;
   X.src_rstep = 1; X.dst_rstep = 1;
   X.nf = 1; X.K = g.K; X.n = g.nx; X.c2r = 1; X.status = g.status; X.pl = g.plNx;
-  X.pair_rows = 1; X.nrows = g.N;
+  X.nrows = g.N; X.pair_rows = xrows_pairs(g.nx, g.N * g.nb);
   return X;
 }
 
@@ -1094,22 +1163,20 @@ cudaError_t launch_stage(const GroupDev& g, int stage, cudaStream_t st, int* nl)
         n = 1;
       } else {
         const YJob J = yjob_inverse(g);
-        const size_t sm = smem_ycols(g.Ccol, g.M, g.f32);
-        if (g.f32) k_ycols<float2><<<dim3(cdiv(g.K, g.Ccol), 9, g.nb), 256, sm, st>>>(J);
-        else if (g.ds) k_ycols<dsc><<<dim3(cdiv(g.K, g.Ccol), 9, g.nb), 256, sm, st>>>(J);
-        else k_ycols<double2><<<dim3(cdiv(g.K, g.Ccol), 9, g.nb), 256, sm, st>>>(J);
+        const dim3 grid(cdiv(g.K, g.Ccol), 9, g.nb);
+        if (g.f32) k_ycols<float2><<<grid, 256, smem_ycols(g.Ccol, g.M), st>>>(J);
+        else k_ycols<fxc><<<grid, 256, smem_ycols_fx(g.Ccol, g.M, g.N), st>>>(J);
         n = 1;
       }
-      if (g.f32) {   // the mean column in double-single
-        k_ycols<dsc><<<dim3(1, 9, g.nb), 256, smem_ycols(1, g.M, 0), st>>>(yjob_mean_inverse(g));
+      if (g.f32) {   // the mean column in fixed point
+        k_ycols<fxc><<<dim3(1, 9, g.nb), 256, smem_ycols_fx(1, g.M, g.N), st>>>(yjob_mean_inverse(g));
         ++n;
       }
       break;
     }
     case 1:
-      if (g.f32) k_xfused<float2><<<dim3(rows, g.nb), g.xthreads, smem_xfused(g.Mx, 1), st>>>(g);
-      else if (g.ds) k_xfused<dsc><<<dim3(rows, g.nb), g.xthreads, smem_xfused(g.Mx, 0), st>>>(g);
-      else k_xfused<double2><<<dim3(rows, g.nb), g.xthreads, smem_xfused(g.Mx, 0), st>>>(g);
+      if (g.f32) k_xfused<<<dim3(rows, g.nb), g.xthreads, smem_xfused(g.Mx, 1), st>>>(g);
+      else k_xfused_fx<<<dim3(rows, g.nb), g.xthreads, smem_xfused(g.Mx, 0), st>>>(g);
       n = 1;
       break;
     case 2: {  // forward y of the 5 explicit fields
@@ -1119,14 +1186,13 @@ cudaError_t launch_stage(const GroupDev& g, int stage, cudaStream_t st, int* nl)
         n = 1;
       } else {
         const YJob F = yjob_forward(g);
-        const size_t sm = smem_ycols(g.Ccol, g.M, g.f32);
-        if (g.f32) k_ycols<float2><<<dim3(cdiv(g.K, g.Ccol), 5, g.nb), 256, sm, st>>>(F);
-        else if (g.ds) k_ycols<dsc><<<dim3(cdiv(g.K, g.Ccol), 5, g.nb), 256, sm, st>>>(F);
-        else k_ycols<double2><<<dim3(cdiv(g.K, g.Ccol), 5, g.nb), 256, sm, st>>>(F);
+        const dim3 grid(cdiv(g.K, g.Ccol), 5, g.nb);
+        if (g.f32) k_ycols<float2><<<grid, 256, smem_ycols(g.Ccol, g.M), st>>>(F);
+        else k_ycols<fxc><<<grid, 256, smem_ycols_fx(g.Ccol, g.M, 0), st>>>(F);
         n = 1;
       }
-      if (g.f32) {   // the mean column in double-single, over the FP32 pass's zeros
-        k_ycols<dsc><<<dim3(1, 5, g.nb), 256, smem_ycols(1, g.M, 0), st>>>(yjob_mean_forward(g));
+      if (g.f32) {   // the mean column in fixed point, over the FP32 pass's zeros
+        k_ycols<fxc><<<dim3(1, 5, g.nb), 256, smem_ycols_fx(1, g.M, 0), st>>>(yjob_mean_forward(g));
         ++n;
       }
       break;
@@ -1168,23 +1234,13 @@ static cudaError_t diag_join(const DiagStreams& d) {
 // Gauss points of the energy quadrature; c_xx + c_yy on the unpadded
 // Gauss-Lobatto rows (DCT-I).
 static void diag_energy_y(const GroupDev& g, cudaStream_t st) {
-  if (g.f32)
-    k_ycols<float2><<<dim3(cdiv(g.K, g.CcolE), 2, g.nb), 256, smem_ycols(g.CcolE, g.Me, 1), st>>>(
-        yjob_energy(g));
-  else if (g.ds)
-    k_ycols<dsc><<<dim3(cdiv(g.K, g.CcolE), 2, g.nb), 256, smem_ycols(g.CcolE, g.Me, 0), st>>>(
-        yjob_energy(g));
-  else
-    k_ycols<double2><<<dim3(cdiv(g.K, g.CcolE), 2, g.nb), 256, smem_ycols(g.CcolE, g.Me, 0), st>>>(
-        yjob_energy(g));
+  const dim3 grid(cdiv(g.K, g.CcolE), 2, g.nb);
+  if (g.f32) k_ycols<float2><<<grid, 256, smem_ycols(g.CcolE, g.Me), st>>>(yjob_energy(g));
+  else k_ycols<fxc><<<grid, 256, smem_ycols_fx(g.CcolE, g.Me, 0), st>>>(yjob_energy(g));
 }
 static void diag_trc_y(const GroupDev& g, cudaStream_t st) {
-  if (g.ds || g.f32)   // double-single (FP64 in and out, FP64 sums downstream)
-    k_ycols<dsc, true><<<dim3(cdiv(g.K, g.CcolU), 1, g.nb), 256, smem_ycols(g.CcolU, g.Pu, 0), st>>>(
-        yjob_trc(g));
-  else
-    k_ycols<double2, true><<<dim3(cdiv(g.K, g.CcolU), 1, g.nb), 256, smem_ycols(g.CcolU, g.Pu, 0), st>>>(
-        yjob_trc(g));
+  k_ycols<fxc, true><<<dim3(cdiv(g.K, g.CcolU), 1, g.nb), 256, smem_ycols_fx(g.CcolU, g.Pu, 0), st>>>(
+      yjob_trc(g));
 }
 
 cudaError_t launch_diag_transforms(const GroupDev& g, cudaStream_t st) {
@@ -1201,7 +1257,8 @@ cudaError_t launch_diag_split(const GroupDev& g, const DiagStreams& d, int* nl) 
   k_diag_mid<<<dim3(cdiv(g.K, kMidModesPerBlock), g.nb), 256, 0, d.s[2]>>>(g);
   // Tr c on the unpadded grid: y, then x
   diag_trc_y(g, d.s[0]);
-  k_xrows<<<dim3(cdiv(g.N, 2), g.nb), 256, smem_xrows(1, g.nx), d.s[0]>>>(xjob_trc(g));
+  const XJob X = xjob_trc(g);
+  k_xrows<<<dim3(xrows_pair_blocks(X.pair_rows, X.nrows), g.nb), 256, smem_xrows(X.pair_rows, g.nx), d.s[0]>>>(X);
   if ((e = cudaGetLastError()) || (e = diag_join(d))) return e;
   k_diag_part<<<dim3(g.ntile, g.nb), 256, 0, d.s[0]>>>(g);
   k_diag_count<<<dim3(g.ntile, g.nb), 256, 0, d.s[0]>>>(g);
@@ -1212,7 +1269,7 @@ cudaError_t launch_diag_split(const GroupDev& g, const DiagStreams& d, int* nl) 
 
 // ------------------------------------------------- launches over all groups
 struct Multi2DPlan {
-  int ng = 0, f32 = 0, ds = 0;
+  int ng = 0, f32 = 0;
   const GroupDev* dg = nullptr;
   // [6][ng]: inverse, forward, energy, Tr c, mean-column inverse and forward
   // (mixed groups)
@@ -1250,7 +1307,6 @@ Multi2DPlan* multi2d_create(const std::vector<const GroupDev*>& groups, void* de
   Multi2DPlan* p = new Multi2DPlan();
   p->ng = ng;
   p->f32 = groups[0]->f32;
-  p->ds = groups[0]->ds;
   std::vector<GroupDev> hg(ng);
   std::vector<YJob> hy(6 * (size_t)ng);
   std::vector<XJob> hx(ng);
@@ -1263,7 +1319,7 @@ Multi2DPlan* multi2d_create(const std::vector<const GroupDev*>& groups, void* de
   std::vector<Ent> e_inv, e_fwd, e_xf, e_spec[3], e_ye, e_yt, e_xr, e_mid, e_part, e_fin, e_ymi, e_ymf;
   for (int q = 0; q < ng; ++q) {
     const GroupDev& g = *groups[q];
-    if (g.nz != 1 || g.f32 != p->f32 || g.ds != p->ds || g.ymma) {
+    if (g.nz != 1 || g.f32 != p->f32 || g.ymma) {
       delete p;
       *err = cudaErrorInvalidValue;
       return nullptr;
@@ -1278,7 +1334,7 @@ Multi2DPlan* multi2d_create(const std::vector<const GroupDev*>& groups, void* de
       hy[5 * (size_t)ng + q] = yjob_mean_forward(g);
       e_ymi.push_back({(double)g.M, q, 1, 9, (unsigned)g.nb});
       e_ymf.push_back({(double)g.M, q, 1, 5, (unsigned)g.nb});
-      p->sm_ym = std::max(p->sm_ym, smem_ycols(1, g.M, 0));
+      p->sm_ym = std::max(p->sm_ym, smem_ycols_fx(1, g.M, g.N));
     }
     hx[q] = xjob_trc(g);
     e_inv.push_back({(double)g.Ccol * g.M, q, cdiv(g.K, g.Ccol), 9, (unsigned)g.nb});
@@ -1289,17 +1345,17 @@ Multi2DPlan* multi2d_create(const std::vector<const GroupDev*>& groups, void* de
     e_spec[cls].push_back({(double)g.N, q, (unsigned)g.K, (unsigned)g.nb, 1});
     e_ye.push_back({(double)g.CcolE * g.Me, q, cdiv(g.K, g.CcolE), 2, (unsigned)g.nb});
     e_yt.push_back({(double)g.CcolU * g.Pu, q, cdiv(g.K, g.CcolU), 1, (unsigned)g.nb});
-    e_xr.push_back({(double)g.nx, q, cdiv(g.N, 2), (unsigned)g.nb, 1});
+    e_xr.push_back({(double)g.nx * hx[q].pair_rows, q, xrows_pair_blocks(hx[q].pair_rows, g.N), (unsigned)g.nb, 1});
     e_mid.push_back({(double)g.N, q, cdiv(g.K, kMidModesPerBlock), (unsigned)g.nb, 1});
     e_part.push_back({(double)g.N * g.nx / g.ntile, q, (unsigned)g.ntile, (unsigned)g.nb, 1});
     e_fin.push_back({(double)g.nx + g.ntile, q, (unsigned)g.nb, 1, 1});
-    p->sm_inv = std::max(p->sm_inv, smem_ycols(g.Ccol, g.M, g.f32));
-    p->sm_fwd = p->sm_inv;
+    p->sm_inv = std::max(p->sm_inv, g.f32 ? smem_ycols(g.Ccol, g.M) : smem_ycols_fx(g.Ccol, g.M, g.N));
+    p->sm_fwd = std::max(p->sm_fwd, g.f32 ? smem_ycols(g.Ccol, g.M) : smem_ycols_fx(g.Ccol, g.M, 0));
     p->sm_xf = std::max(p->sm_xf, smem_xfused(g.Mx, g.f32));
     p->sm_spec[cls] = std::max(p->sm_spec[cls], smem_spec(g.N));
-    p->sm_ye = std::max(p->sm_ye, smem_ycols(g.CcolE, g.Me, g.f32));
-    p->sm_yt = std::max(p->sm_yt, smem_ycols(g.CcolU, g.Pu, 0));
-    p->sm_xr = std::max(p->sm_xr, smem_xrows(1, g.nx));
+    p->sm_ye = std::max(p->sm_ye, g.f32 ? smem_ycols(g.CcolE, g.Me) : smem_ycols_fx(g.CcolE, g.Me, 0));
+    p->sm_yt = std::max(p->sm_yt, smem_ycols_fx(g.CcolU, g.Pu, 0));
+    p->sm_xr = std::max(p->sm_xr, smem_xrows(hx[q].pair_rows, g.nx));
     p->sm_fin = std::max(p->sm_fin, smem_xrows(3, g.nx));
   }
   auto fill = [](MultiMap& m, std::vector<Ent>& v) {
@@ -1344,27 +1400,24 @@ cudaError_t launch_stage_multi(const Multi2DPlan* p, int stage, cudaStream_t st,
   switch (stage) {
     case 0:
       if (p->f32) k_ycols_multi<float2><<<mm_blocks(p->inv), 256, p->sm_inv, st>>>(p->dyj, p->inv);
-      else if (p->ds) k_ycols_multi<dsc><<<mm_blocks(p->inv), 256, p->sm_inv, st>>>(p->dyj, p->inv);
-      else k_ycols_multi<double2><<<mm_blocks(p->inv), 256, p->sm_inv, st>>>(p->dyj, p->inv);
+      else k_ycols_multi<fxc><<<mm_blocks(p->inv), 256, p->sm_inv, st>>>(p->dyj, p->inv);
       n = 1;
-      if (p->ymi.ng) {   // mixed groups: the mean columns in double-single
-        k_ycols_multi<dsc><<<mm_blocks(p->ymi), 256, p->sm_ym, st>>>(p->dyj + 4 * ng, p->ymi);
+      if (p->ymi.ng) {   // mixed groups: the mean columns in fixed point
+        k_ycols_multi<fxc><<<mm_blocks(p->ymi), 256, p->sm_ym, st>>>(p->dyj + 4 * ng, p->ymi);
         ++n;
       }
       break;
     case 1:
-      if (p->f32) k_xfused_multi<float2><<<mm_blocks(p->xf), 512, p->sm_xf, st>>>(p->dg, p->xf);
-      else if (p->ds) k_xfused_multi<dsc><<<mm_blocks(p->xf), 512, p->sm_xf, st>>>(p->dg, p->xf);
-      else k_xfused_multi<double2><<<mm_blocks(p->xf), 512, p->sm_xf, st>>>(p->dg, p->xf);
+      if (p->f32) k_xfused_multi<<<mm_blocks(p->xf), 512, p->sm_xf, st>>>(p->dg, p->xf);
+      else k_xfused_fx_multi<<<mm_blocks(p->xf), kFxThreads, p->sm_xf, st>>>(p->dg, p->xf);
       n = 1;
       break;
     case 2:
       if (p->f32) k_ycols_multi<float2><<<mm_blocks(p->fwd), 256, p->sm_fwd, st>>>(p->dyj + ng, p->fwd);
-      else if (p->ds) k_ycols_multi<dsc><<<mm_blocks(p->fwd), 256, p->sm_fwd, st>>>(p->dyj + ng, p->fwd);
-      else k_ycols_multi<double2><<<mm_blocks(p->fwd), 256, p->sm_fwd, st>>>(p->dyj + ng, p->fwd);
+      else k_ycols_multi<fxc><<<mm_blocks(p->fwd), 256, p->sm_fwd, st>>>(p->dyj + ng, p->fwd);
       n = 1;
       if (p->ymf.ng) {
-        k_ycols_multi<dsc><<<mm_blocks(p->ymf), 256, p->sm_ym, st>>>(p->dyj + 5 * ng, p->ymf);
+        k_ycols_multi<fxc><<<mm_blocks(p->ymf), 256, p->sm_ym, st>>>(p->dyj + 5 * ng, p->ymf);
         ++n;
       }
       break;
@@ -1394,12 +1447,9 @@ cudaError_t launch_diag_multi(const Multi2DPlan* p, const DiagStreams& d, int* n
   cudaError_t e = diag_fork(d);
   if (e) return e;
   if (p->f32) k_ycols_multi<float2><<<mm_blocks(p->ye), 256, p->sm_ye, d.s[1]>>>(p->dyj + 2 * ng, p->ye);
-  else if (p->ds) k_ycols_multi<dsc><<<mm_blocks(p->ye), 256, p->sm_ye, d.s[1]>>>(p->dyj + 2 * ng, p->ye);
-  else k_ycols_multi<double2><<<mm_blocks(p->ye), 256, p->sm_ye, d.s[1]>>>(p->dyj + 2 * ng, p->ye);
+  else k_ycols_multi<fxc><<<mm_blocks(p->ye), 256, p->sm_ye, d.s[1]>>>(p->dyj + 2 * ng, p->ye);
   k_diag_mid_multi<<<mm_blocks(p->mid), 256, 0, d.s[2]>>>(p->dg, p->mid);
-  if (p->ds || p->f32)
-    k_ycols_multi<dsc, true><<<mm_blocks(p->yt), 256, p->sm_yt, d.s[0]>>>(p->dyj + 3 * ng, p->yt);
-  else k_ycols_multi<double2, true><<<mm_blocks(p->yt), 256, p->sm_yt, d.s[0]>>>(p->dyj + 3 * ng, p->yt);
+  k_ycols_multi<fxc, true><<<mm_blocks(p->yt), 256, p->sm_yt, d.s[0]>>>(p->dyj + 3 * ng, p->yt);
   k_xrows_multi<<<mm_blocks(p->xr), 256, p->sm_xr, d.s[0]>>>(p->dxj, p->xr);
   if ((e = cudaGetLastError()) || (e = diag_join(d))) return e;
   k_diag_part_multi<<<mm_blocks(p->part), 256, 0, d.s[0]>>>(p->dg, p->part);
@@ -1456,7 +1506,7 @@ cudaError_t launch_phys_to_state(const GroupDev& g, int b, cudaStream_t st) {
   J.src = g.stageS; J.dst = g.X + (size_t)b * 5 * NK;
   J.src_fstride = NK; J.dst_fstride = NK;
   for (int i = 0; i < 5; ++i) { J.src_field[i] = i; J.dst_field[i] = i; J.deriv[i] = 0; }
-  k_ycols<double2, true><<<dim3(cdiv(g.K, g.CcolU), 5, 1), 256, smem_ycols(g.CcolU, g.Pu, 0), st>>>(J);
+  k_ycols<fxc, true><<<dim3(cdiv(g.K, g.CcolU), 5, 1), 256, smem_ycols_fx(g.CcolU, g.Pu, 0), st>>>(J);
   k_reset<<<1, 32, 0, st>>>(g, b);
   return cudaGetLastError();
 }
@@ -1468,7 +1518,7 @@ cudaError_t launch_state_to_phys(const GroupDev& g, int b, cudaStream_t st) {
   J.src = g.X + (size_t)b * 5 * NK; J.dst = g.stageS;
   J.src_fstride = NK; J.dst_fstride = NK;
   for (int i = 0; i < 5; ++i) { J.src_field[i] = i; J.dst_field[i] = i; J.deriv[i] = 0; }
-  k_ycols<double2, true><<<dim3(cdiv(g.K, g.CcolU), 5, 1), 256, smem_ycols(g.CcolU, g.Pu, 0), st>>>(J);
+  k_ycols<fxc, true><<<dim3(cdiv(g.K, g.CcolU), 5, 1), 256, smem_ycols_fx(g.CcolU, g.Pu, 0), st>>>(J);
   XJob X{};
   X.srcC = g.stageS; X.dstR = g.stage;
   X.src_fstride = NK; X.dst_fstride = (long long)g.N * g.nx;

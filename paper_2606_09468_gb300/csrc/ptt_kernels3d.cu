@@ -32,7 +32,6 @@ namespace {
 struct ZJob {
   const void* src;
   void* dst;
-  int src_f32, dst_f32;
   long long src_mstride, dst_mstride;  // per member (elements)
   long long src_fstride, dst_fstride;  // per field (elements)
   int src_field[32];
@@ -55,11 +54,96 @@ struct ZJob {
   double2* zm;
 };
 
-// BIG: unpadded z length nz (radices 7, 11, 13 possible); the padded length
-// Mz of the step runs without it.
-template <typename CT, bool BIG = false>
+// Fixed-point z lines between FP64 arrays.  BIG: unpadded z length nz
+// (radices 7, 11, 13 possible); the padded length Mz of the step runs
+// without it.  Forward: times J.inv (1 in the step, whose y table holds the
+// normalisation).
+template <bool BIG>
+__global__ void __launch_bounds__(256, BIG ? 3 : 5) k_zcols_fx(const __grid_constant__ ZJob J) {
+  const int b = blockIdx.z;
+  if (J.status && J.status[b]) return;
+  const int f = blockIdx.y / J.rows;
+  const int j = blockIdx.y - f * J.rows;
+  const int C = J.C, K = J.K, nz = J.nz, Mz = J.Mz;
+  const int m0 = blockIdx.x * C;
+  const int nc = min(C, K - m0);
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ FxS fs[64];
+  fxc* A = reinterpret_cast<fxc*>(smraw);
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, nw = nt >> 5;
+  const int hz = nz / 2;
+  const FastDiv dC = fast_div((unsigned)C);
+  if (J.inverse) {
+    const double2* src = static_cast<const double2*>(J.src) + b * J.src_mstride +
+                         J.src_field[f] * J.src_fstride + (long long)j * K * nz;
+    double2* dst = static_cast<double2*>(J.dst) + b * J.dst_mstride + J.dst_field[f] * J.dst_fstride +
+                   (long long)j * Mz * K;
+    const double kfac = J.prm[b].kz1;
+    const int dz = J.dz[f], gap = Mz - nz;
+    for (int c = tid >> 5; c < nc; c += nw) {   // a warp per line
+      fxc* h = A + c * Mz;
+      const double2* s = src + (long long)(m0 + c) * nz;
+      unsigned m = 0u;
+#pragma unroll 2
+      for (int q = lane; q < nz; q += 32) {   // modes 0 .. hz-1, the slot hz (zero), the negative ones
+        double2 v = czero();
+        if (q != hz) {
+          v = s[q];
+          if (dz) v = cscl(mul_i(v), kfac * (q < hz ? q : q - nz));
+        }
+        h[q <= hz ? q : q + gap] = fx_bits(v.x, v.y);
+        m = max(m, fx_mag2(v));
+      }
+      for (int q = hz + 1 + lane; q <= hz + gap; q += 32) h[q] = fx_zero();
+      __syncwarp();
+      auto at = [=](int q) { return q <= hz ? q : q + gap; };
+      const FxS sc = fx_warp_scale(m, nz, [=](int q) { return fx_raw(h[at(q)]); }, 0);
+      if (lane == 0) fs[c] = sc;
+      __syncwarp();
+      for (int q = lane; q < nz; q += 32) h[at(q)] = fx_from2(fx_raw(h[at(q)]), sc.base);
+    }
+    __syncthreads();
+    // padded synthesis (Mz >= 3 nz/2): the slots nz/2 .. Mz - nz/2 are zero
+    fx_lines<+1, BIG>(A, nc, Mz, &J.pl, J.pl.radix[0] % 3 == 0 && Mz >= 3 * hz);
+    for (int i = tid; i < Mz * C; i += nt) {
+      const int z = (int)fdiv((unsigned)i, dC), c = i - z * C;
+      if (c < nc) dst[(long long)z * K + m0 + c] = fx_to2(A[c * Mz + z], fs[c]);
+    }
+  } else {
+    const double2* src = static_cast<const double2*>(J.src) + b * J.src_mstride +
+                         J.src_field[f] * J.src_fstride + (long long)j * Mz * K;
+    double2* dst = static_cast<double2*>(J.dst) + b * J.dst_mstride + J.dst_field[f] * J.dst_fstride +
+                   (long long)j * K * nz;
+    double2* R = reinterpret_cast<double2*>(smraw);
+    for (int i = tid; i < Mz * C; i += nt) {
+      const int z = (int)fdiv((unsigned)i, dC), c = i - z * C;
+      if (c < nc) {
+        // the kx = 0 line (the x means) less its first value: it may hardly vary
+        double2 v = src[(long long)z * K + m0 + c];
+        if (m0 + c == 0) v = csub(v, src[0]);
+        R[c * Mz + z] = v;
+      }
+    }
+    __syncthreads();
+    for (int c = tid >> 5; c < nc; c += nw) fx_line(A + c * Mz, Mz, fs[c]);
+    __syncthreads();
+    fx_lines<-1, BIG>(A, nc, Mz, &J.pl, false);
+    for (int c = tid >> 5; c < nc; c += nw)
+      for (int q = lane; q < nz; q += 32) {
+        double2 v = czero();
+        if (q != hz) {
+          v = fx_to2(A[c * Mz + (q < hz ? q : q - nz + Mz)], fs[c]);
+          if (q == 0 && m0 + c == 0) v = cfma((double)Mz, src[0], v);
+          if (J.inv != 1.0) v = cscl(v, J.inv);
+        }
+        dst[(long long)(m0 + c) * nz + q] = v;
+      }
+  }
+}
+
+// FP32 z lines (mixed groups' step).
 __global__ void __launch_bounds__(256) k_zcols(ZJob J) {
-  using T = typename RealOf<CT>::T;
+  using CT = float2;
   const int b = blockIdx.z;
   if (J.status && J.status[b]) return;
   const int f = blockIdx.y / J.rows;
@@ -70,16 +154,14 @@ __global__ void __launch_bounds__(256) k_zcols(ZJob J) {
   extern __shared__ __align__(16) unsigned char smraw[];
   CT* A = reinterpret_cast<CT*>(smraw);
   CT* B = A + (size_t)C * Mz;
-  const size_t es = (J.src_f32 == 1) ? sizeof(float2) : sizeof(double2);
-  const size_t ed = (J.dst_f32 == 1) ? sizeof(float2) : sizeof(double2);
   const int tid = threadIdx.x, nt = blockDim.x;
   const int hz = nz / 2;
   if (J.inverse) {
-    const void* src = static_cast<const char*>(J.src) +
-        (b * J.src_mstride + J.src_field[f] * J.src_fstride + (long long)j * K * nz) * es;
-    void* dst = static_cast<char*>(J.dst) +
-        (b * J.dst_mstride + J.dst_field[f] * J.dst_fstride + (long long)j * Mz * K) * ed;
-    const T kfac = as_prec<T>(J.prm[b].kz1, J.prm[b].kz1f);
+    const CT* src = static_cast<const CT*>(J.src) + b * J.src_mstride + J.src_field[f] * J.src_fstride +
+                    (long long)j * K * nz;
+    CT* dst = static_cast<CT*>(J.dst) + b * J.dst_mstride + J.dst_field[f] * J.dst_fstride +
+              (long long)j * Mz * K;
+    const float kfac = J.prm[b].kz1f;
     const int dz = J.dz[f];
     for (int i = tid; i < C * Mz; i += nt) A[i] = zero2<CT>();
     __syncthreads();
@@ -88,30 +170,30 @@ __global__ void __launch_bounds__(256) k_zcols(ZJob J) {
       const int c = (int)fdiv((unsigned)i, fast_div((unsigned)nz)), mz = i - c * nz;
       if (c < nc && mz != hz && !(skip0 && c == 0 && mz == 0)) {
         const int s = (mz < hz) ? mz : mz - nz;
-        CT v = ld2<CT>(src, (long long)(m0 + c) * nz + mz, J.src_f32);
-        if (dz) v = cscl(mul_i(v), kfac * (T)s);
+        CT v = src[(long long)(m0 + c) * nz + mz];
+        if (dz) v = cscl(mul_i(v), kfac * (float)s);
         A[c * Mz + (s >= 0 ? s : s + Mz)] = v;
       }
     }
     __syncthreads();
     // padded synthesis (Mz >= 3 nz/2): the slots nz/2 .. Mz - nz/2 are zero
-    CT* res = fft_lines<+1, CT, BIG>(A, B, C, Mz, J.pl, J.pl.radix[0] == 3 && Mz >= 3 * hz);
+    CT* res = fft_lines<+1>(A, B, C, Mz, J.pl, J.pl.radix[0] == 3 && Mz >= 3 * hz);
     for (int i = tid; i < Mz * C; i += nt) {
       const int z = (int)fdiv((unsigned)i, fast_div((unsigned)C)), c = i - z * C;
-      if (c < nc) st2<CT>(dst, (long long)z * K + m0 + c, J.dst_f32, res[c * Mz + z]);
+      if (c < nc) dst[(long long)z * K + m0 + c] = res[c * Mz + z];
     }
   } else {
-    const void* src = static_cast<const char*>(J.src) +
-        (b * J.src_mstride + J.src_field[f] * J.src_fstride + (long long)j * Mz * K) * es;
-    void* dst = static_cast<char*>(J.dst) +
-        (b * J.dst_mstride + J.dst_field[f] * J.dst_fstride + (long long)j * K * nz) * ed;
+    const CT* src = static_cast<const CT*>(J.src) + b * J.src_mstride + J.src_field[f] * J.src_fstride +
+                    (long long)j * Mz * K;
+    CT* dst = static_cast<CT*>(J.dst) + b * J.dst_mstride + J.dst_field[f] * J.dst_fstride +
+              (long long)j * K * nz;
     for (int i = tid; i < Mz * C; i += nt) {
       const int z = (int)fdiv((unsigned)i, fast_div((unsigned)C)), c = i - z * C;
-      A[c * Mz + z] = (c < nc) ? ld2<CT>(src, (long long)z * K + m0 + c, J.src_f32) : zero2<CT>();
+      A[c * Mz + z] = (c < nc) ? src[(long long)z * K + m0 + c] : zero2<CT>();
     }
     __syncthreads();
-    CT* res = fft_lines<-1, CT, BIG>(A, B, C, Mz, J.pl);
-    const T inv = as_prec<T>(J.inv, J.invf);
+    CT* res = fft_lines<-1>(A, B, C, Mz, J.pl);
+    const float inv = J.invf;
     for (int i = tid; i < C * nz; i += nt) {
       const int c = (int)fdiv((unsigned)i, fast_div((unsigned)nz)), mz = i - c * nz;
       if (c < nc) {
@@ -120,13 +202,11 @@ __global__ void __launch_bounds__(256) k_zcols(ZJob J) {
           const int s = (mz < hz) ? mz : mz - nz;
           v = cscl(res[c * Mz + (s >= 0 ? s : s + Mz)], inv);
         }
-        if constexpr (std::is_same<CT, float2>::value) {
-          if (J.mean == 2 && m0 + c == 0 && mz == 0) {
-            J.zm[((size_t)b * 9 + J.dst_field[f]) * J.rows + j].x += (double)v.x;
-            v = zero2<CT>();
-          }
+        if (J.mean == 2 && m0 + c == 0 && mz == 0) {
+          J.zm[((size_t)b * 9 + J.dst_field[f]) * J.rows + j].x += (double)v.x;
+          v = zero2<CT>();
         }
-        st2<CT>(dst, (long long)(m0 + c) * nz + mz, J.dst_f32, v);
+        dst[(long long)(m0 + c) * nz + mz] = v;
       }
     }
   }
@@ -138,17 +218,6 @@ __global__ void __launch_bounds__(256) k_zcols(ZJob J) {
 // 20-25 c_z.  Physical fields (35): the 26 plus x-derivatives of fields 0-8
 // (26 ux, 27 vx, 28 wx, 29-34 c_x), packed in pairs into 18 complex lines.
 // W3 outputs (9): N_cxx, N_cxy, N_cxz, N_cyy, N_cyz, N_czz, N_u, N_v, N_w.
-template <typename C2> __device__ __forceinline__ const C2* z3_ptr(const GroupDev& g);
-template <> __device__ __forceinline__ const double2* z3_ptr<double2>(const GroupDev& g) { return g.Z3; }
-template <> __device__ __forceinline__ const float2* z3_ptr<float2>(const GroupDev& g) { return g.Z3f; }
-template <> __device__ __forceinline__ const dsc* z3_ptr<dsc>(const GroupDev& g) {
-  return reinterpret_cast<const dsc*>(g.Z3);
-}
-template <typename C2> __device__ __forceinline__ C2* w3_ptr(const GroupDev& g);
-template <> __device__ __forceinline__ double2* w3_ptr<double2>(const GroupDev& g) { return g.W3; }
-template <> __device__ __forceinline__ float2* w3_ptr<float2>(const GroupDev& g) { return g.W3f; }
-template <> __device__ __forceinline__ dsc* w3_ptr<dsc>(const GroupDev& g) { return reinterpret_cast<dsc*>(g.W3); }
-
 // The products of Eqs. 1-2 at one point from the 35 physical fields q (Z3
 // order, then the x-derivatives of fields 0-8 at 26-34; q[35] unused) to
 // N_cxx, N_cxy, N_cxz, N_cyy, N_cyz, N_czz, N_u, N_v, N_w.
@@ -180,12 +249,127 @@ __device__ __forceinline__ void products3d(const T (&q)[36], T eps, T iwi, T (&o
   for (int i = 0; i < 3; ++i) out[6 + i] = -(uu[0] * L[i][0] + uu[1] * L[i][1] + uu[2] * L[i][2]);
 }
 
-// IP: the lines stay in one buffer and every FFT pass works in place
-// (fft_lines_inplace; kIpThreads threads), for the FP64 lines too long for
-// two buffers in shared memory (Mx up to kIpMaxN).
-template <typename C2, bool IP = false>
+// The same in FP64 with the fewest FP64 instructions (67 against about 100;
+// each holds the pipe for 64 cycles): every output one chain of fused
+// multiply-adds, the "+ rw" of -(c - 1) rw and the constants of the relaxation
+// factor folded into its start, factors 2 as exponent increments on the
+// integer pipe.  e1 = eps/Wi, e0 = (1 - 3 eps)/Wi.
+__device__ __forceinline__ double twice3(double x) {   // 2 x by the exponent
+  const int h = __double2hiint(x);
+  const bool n = (h & 0x7FF00000) != 0 && (h & 0x7FF00000) < 0x7FE00000;
+  return n ? __hiloint2double(h + 0x100000, __double2loint(x)) : x + x;
+}
+// get(i): field i, read where it is used (the velocity, its gradient and c stay
+// in registers, the gradients of c do not).
+template <typename Get>
+__device__ __forceinline__ void products3d_fp64(Get get, double e1, double e0, double (&out)[9]) {
+  const double u = get(0), v = get(1), w = get(2);
+  const double c3 = get(3), c4 = get(4), c5 = get(5), c6 = get(6), c7 = get(7), c8 = get(8);
+  const double C[3][3] = {{c3, c4, c5}, {c4, c6, c7}, {c5, c7, c8}};
+  const double ux = get(26), wz = get(19);
+  const double L[3][3] = {{ux, get(9), get(17)}, {get(27), -ux - wz, get(18)}, {get(28), get(10), wz}};
+  const double rw = fma(e1, c3 + c6 + c8, e0);
+  const int ci[6] = {0, 0, 0, 1, 1, 2}, cj[6] = {0, 1, 2, 1, 2, 2};
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const int i = ci[c], j = cj[c];
+    const double gx = get(29 + c), gy = get(11 + c), gz = get(20 + c);
+    double t = (i == j) ? fma(-u, gx, rw) : -u * gx;
+    t = fma(-w, gz, fma(-v, gy, t));
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      t = (i == j) ? fma(twice3(L[i][k]), C[k][j], t) : fma(C[i][k], L[j][k], fma(L[i][k], C[k][j], t));
+    out[c] = fma(-C[i][j], rw, t);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) out[6 + i] = fma(-w, L[i][2], fma(-v, L[i][1], -u * L[i][0]));
+}
+
+// FP64-accurate form: fixed-point transforms (ptt_fx.cuh) between FP64 arrays,
+// products in FP64; 18 lines of Mx in one shared-memory buffer.  W3 is left
+// without its 1/Mx (the y table's normalisation holds it).  Bound by
+// instruction issue and latency, next the FP64 pipe of the products: four
+// blocks of 256 threads per SM take 0.94 ms at 128 x 97 x 64, three 1.08, two
+// 1.26 (FP64 lines on the FP64 pipe: 3.40).  Beyond 256 threads (ptt_autotune,
+// where one block fills the shared memory) one block per SM.
+template <int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_xfused3_fx(const __grid_constant__ GroupDev g) {
+  const int b = blockIdx.y;
+  if (g.status[b]) return;
+  const int row = blockIdx.x;  // j * Mz + z
+  const int K = g.K, Mx = g.Mx;
+  const long long plane = (long long)g.M * g.Mz * K;  // one field of one member
+  const MemberPrm pr = g.prm[b];
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ FxS fs[36], fo[10];
+  __shared__ double2 ref[5];
+  fxc* A = reinterpret_cast<fxc*>(smraw);
+  const double2* Z = g.Z3 + (size_t)b * 26 * plane + (size_t)row * K;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, nw = nt >> 5;
+  // lines 0-12: the 26 loaded fields in pairs (2l, 2l+1); line 13 + r
+  // (r < 5): their x-derivatives i k (fields 2r, 2r+1; line 17 field 8
+  // alone).  A warp per line: its two fields' modes, then their scales and
+  // the packed line; the padded middle is zero.
+  for (int l = tid >> 5; l < 18; l += nw) {
+    fxc* h = A + l * Mx;
+    const int r = (l < 13) ? l : l - 13;
+    const double2* zF = Z + (size_t)(2 * r) * plane;
+    unsigned mF = 0u, mG = 0u;
+#pragma unroll 2
+    for (int k = lane; k < K; k += 32) {
+      double2 F = zF[k], G = (l < 17) ? zF[plane + k] : czero();
+      if (k == 0) { F.y = 0; G.y = 0; }
+      if (l >= 13) {
+        const double fk = pr.kx1 * k;
+        F = cscl(mul_i(F), fk);
+        G = cscl(mul_i(G), fk);
+      }
+      h[k] = fx_bits(F.x, F.y);
+      h[fx_xslot(1, k, K, Mx)] = fx_bits(G.x, G.y);
+      mF = max(mF, fx_mag2(F));
+      mG = max(mG, fx_mag2(G));
+    }
+    for (int k = K + 1 + lane; k <= Mx - K; k += 32) h[k] = fx_zero();
+    __syncwarp();
+    fx_xline(h, Mx, K, mF, mG, fs[2 * l], fs[2 * l + 1]);
+  }
+  __syncthreads();
+  fx_lines<+1, false>(A, 18, Mx, &g.plMx, g.plMx.radix[0] % 3 == 0);
+  const double e1 = pr.eps * pr.inv_wi, e0 = (1.0 - 3.0 * pr.eps) * pr.inv_wi;
+  for (int x = tid; x < Mx; x += nt) {   // a column x is read and rewritten by one thread
+    double out[9];
+    products3d_fp64(
+        [&](int i) {
+          const fxc h = A[(i >> 1) * Mx + x];
+          return fx_to((i & 1) ? h.y : h.x, fs[i]);
+        },
+        e1, e0, out);
+#pragma unroll
+    for (int l = 0; l < 5; ++l) A[l * Mx + x] = fx_bits(out[2 * l], (2 * l + 1 < 9) ? out[2 * l + 1] : 0.0);
+  }
+  __syncthreads();
+  for (int l = tid >> 5; l < 5; l += nw) {
+    const double2 r = fx_fields(A + l * Mx, Mx, fo[2 * l], fo[2 * l + 1]);
+    if (lane == 0) ref[l] = r;
+  }
+  __syncthreads();
+  fx_lines<-1, false>(A, 5, Mx, &g.plMx, false);
+  double2* W = g.W3 + (size_t)b * 9 * plane + (size_t)row * K;
+  const FastDiv dK = fast_div((unsigned)K);
+  for (int i = tid; i < 5 * K; i += nt) {
+    const int l = (int)fdiv((unsigned)i, dK), k = i - l * K;
+    W[(size_t)(2 * l) * plane + k] = fx_mode_f(A + l * Mx, Mx, k, fo[2 * l], ref[l].x);
+    if (2 * l + 1 < 9) W[(size_t)(2 * l + 1) * plane + k] = fx_mode_g(A + l * Mx, Mx, k, fo[2 * l + 1], ref[l].y);
+  }
+}
+
+// Mixed form: FP32 transforms; mean/fluctuation split of the products (see
+// xfused_block in the 2D kernels): the z pass left the mean mode out of the
+// lines, the means of the 17 y-pass fields at this row's y come from g.Ym (the
+// z- and x-derivatives have zero mean), the mean products go to g.Zm (written
+// by the rows at z = 0; the forward z pass adds the fluctuations' mean).
 __global__ void __launch_bounds__(512) k_xfused3(GroupDev g) {
-  using T = typename RealOf<C2>::T;
+  using C2 = float2;
   const int b = blockIdx.y;
   if (g.status[b]) return;
   const int row = blockIdx.x;  // j * Mz + z
@@ -195,17 +379,11 @@ __global__ void __launch_bounds__(512) k_xfused3(GroupDev g) {
   extern __shared__ __align__(16) unsigned char smraw[];
   C2* A = reinterpret_cast<C2*>(smraw);
   C2* B = A + 18 * Mx;
-  const C2* Z = z3_ptr<C2>(g) + (size_t)b * 26 * plane + (size_t)row * K;
-  const T kfac = as_prec<T>(pr.kx1, pr.kx1f);
+  const C2* Z = g.Z3f + (size_t)b * 26 * plane + (size_t)row * K;
+  const float kfac = pr.kx1f;
   const int tid = threadIdx.x, nt = blockDim.x;
-  // mixed groups: mean/fluctuation split of the products (see xfused_block
-  // in the 2D kernels): the z pass left the mean mode out of the lines, the
-  // means of the 17 y-pass fields at this row's y come from g.Ym (the z- and
-  // x-derivatives have zero mean), the mean products go to g.Zm (written by
-  // the rows at z = 0; the forward z pass adds the fluctuations' mean)
-  constexpr bool kSplit = std::is_same<C2, float2>::value;
   __shared__ float s_mq[17];
-  if constexpr (kSplit) {
+  {
     const int jy = row / g.Mz;
     const double2* ym = g.Ym + (size_t)b * 17 * g.M + jy;
     if (tid < 17) s_mq[tid] = (float)ym[(size_t)tid * g.M].x;
@@ -225,11 +403,7 @@ __global__ void __launch_bounds__(512) k_xfused3(GroupDev g) {
       A[l * Mx + k] = zero2<C2>();
     }
   }
-  // lines 0-12: the 26 loaded fields in pairs (2l, 2l+1); line 13 + r
-  // (r < 5): their x-derivatives i k (fields 2r, 2r+1; line 17 field 8
-  // alone).  Items (l < 13, mode kk): both fields' coefficients loaded by
-  // one thread, coalesced along kk, a batch of items in flight at once, then
-  // written at k = kk and (conjugated) at Mx - kk.
+  // the lines and items of the fixed-point form
   {
     constexpr int kB = 4;   // items in flight per thread
     const int nitem = 13 * K;
@@ -256,7 +430,7 @@ __global__ void __launch_bounds__(512) k_xfused3(GroupDev g) {
         A[l * Mx + kk] = cadd(f, mul_i(gg));
         if (kk > 0) A[l * Mx + Mx - kk] = cadd(cconj(f), mul_i(cconj(gg)));
         if (l < 5) {
-          const T fk = kfac * (T)kk;
+          const float fk = kfac * (float)kk;
           C2 df = cscl(mul_i(F[u]), fk), dg = cscl(mul_i(G[u]), fk);
           if (l == 4) dg = zero2<C2>();
           if (kk == 0) { df.y = 0; dg.y = 0; }
@@ -268,68 +442,32 @@ __global__ void __launch_bounds__(512) k_xfused3(GroupDev g) {
     }
   }
   __syncthreads();
-  C2* res;
-  C2* oth;
-  if constexpr (IP) {
-    fft_lines_inplace<+1>(A, 18, Mx, g.plMx, g.plMx.radix[0] == 3);
-    res = oth = A;   // each column x is read and rewritten by one thread
-  } else {
-    res = fft_lines<+1>(A, B, 18, Mx, g.plMx, g.plMx.radix[0] == 3);
-    oth = (res == A) ? B : A;
-  }
-  const T eps = as_prec<T>(pr.eps, pr.epsf), iwi = as_prec<T>(pr.inv_wi, pr.inv_wif);
+  C2* res = fft_lines<+1>(A, B, 18, Mx, g.plMx, g.plMx.radix[0] == 3);
+  C2* oth = (res == A) ? B : A;
   for (int x = tid; x < Mx; x += nt) {
-    T out[9];
-    if constexpr (kSplit) {
-      mfl q[36], om[9];
+    mfl q[36], om[9];
 #pragma unroll
-      for (int l = 0; l < 18; ++l) {
-        const C2 h = res[l * Mx + x];
-        q[2 * l] = mfl(2 * l < 17 ? s_mq[2 * l] : 0.f, h.x);
-        q[2 * l + 1] = mfl(2 * l + 1 < 17 ? s_mq[2 * l + 1] : 0.f, h.y);
-      }
-      products3d<mfl>(q, mfl(pr.epsf, 0.f), mfl(pr.inv_wif, 0.f), om);
-#pragma unroll
-      for (int i = 0; i < 9; ++i) out[i] = om[i].f;
-    } else {
-      T q[36];
-#pragma unroll
-      for (int l = 0; l < 18; ++l) {
-        const C2 h = res[l * Mx + x];
-        q[2 * l] = h.x;
-        q[2 * l + 1] = h.y;
-      }
-      products3d<T>(q, eps, iwi, out);
+    for (int l = 0; l < 18; ++l) {
+      const C2 h = res[l * Mx + x];
+      q[2 * l] = mfl(2 * l < 17 ? s_mq[2 * l] : 0.f, h.x);
+      q[2 * l + 1] = mfl(2 * l + 1 < 17 ? s_mq[2 * l + 1] : 0.f, h.y);
     }
+    products3d<mfl>(q, mfl(pr.epsf, 0.f), mfl(pr.inv_wif, 0.f), om);
 #pragma unroll
-    for (int l = 0; l < 5; ++l) {
-      C2 o;
-      o.x = out[2 * l];
-      o.y = (2 * l + 1 < 9) ? out[2 * l + 1] : (T)0;
-      oth[l * Mx + x] = o;
-    }
+    for (int l = 0; l < 5; ++l) oth[l * Mx + x] = make_float2(om[2 * l].f, (2 * l + 1 < 9) ? om[2 * l + 1].f : 0.f);
   }
   __syncthreads();
-  C2* r2;
-  if constexpr (IP) {
-    fft_lines_inplace<-1>(oth, 5, Mx, g.plMx);
-    r2 = oth;
-  } else {
-    r2 = fft_lines<-1>(oth, res, 5, Mx, g.plMx);
-  }
-  C2* W = w3_ptr<C2>(g) + (size_t)b * 9 * plane + (size_t)row * K;
-  const T inv = as_prec<T>(g.invMx, g.invMxf);
+  C2* r2 = fft_lines<-1>(oth, res, 5, Mx, g.plMx);
+  C2* W = g.W3f + (size_t)b * 9 * plane + (size_t)row * K;
+  const float inv = g.invMxf;
   for (int i = tid; i < 5 * K; i += nt) {
     const int l = (int)fdiv((unsigned)i, fast_div((unsigned)K)), k = i - l * K;
     const C2 hk = r2[l * Mx + k];
     const C2 hm = cconj(r2[l * Mx + (k == 0 ? 0 : Mx - k)]);
-    const C2 F = cscl(cadd(hk, hm), (T)0.5 * inv);
+    const C2 F = cscl(cadd(hk, hm), 0.5f * inv);
     const C2 d = csub(hk, hm);
-    C2 G;
-    G.x = (T)0.5 * inv * d.y;
-    G.y = (T)-0.5 * inv * d.x;
     W[(size_t)(2 * l) * plane + k] = F;
-    if (2 * l + 1 < 9) W[(size_t)(2 * l + 1) * plane + k] = G;
+    if (2 * l + 1 < 9) W[(size_t)(2 * l + 1) * plane + k] = make_float2(0.5f * inv * d.y, -0.5f * inv * d.x);
   }
 }
 
@@ -850,12 +988,12 @@ __global__ void k_reset3(GroupDev g, int b) {
   }
 }
 
-YJob yjob3(const GroupDev& g, bool inverse, int M, int C, const FftPlan& pl, const double2* tw4) {
+YJob yjob3(const GroupDev& g, bool inverse, int M, int C, const FftPlan& pl, bool gauss) {
   YJob J{};
-  J.gauss = tw4 ? 1 : 0;
-  J.tw4 = tw4;  // the quarter-period table of this direction
-  J.tw4f = inverse ? g.tw4Pif : g.tw4Pf;
-  J.tw4d = inverse ? g.tw4Pid : g.tw4Pd;
+  J.gauss = gauss ? 1 : 0;
+  J.tw4f = inverse ? g.tw4Pif : g.tw4Pf;   // the quarter-period tables of this direction
+  J.tw4x = inverse ? g.tw4Pix : g.tw4Px;
+  J.fexp = g.fexpP;
   J.K = g.KZ;
   J.N = g.N;
   J.M = M;
@@ -887,7 +1025,7 @@ ZJob zjob(const GroupDev& g, bool inverse, int Mz, int rows, const FftPlan& pl) 
   return Z;
 }
 
-size_t smem_zcols(int C, int Mz, int f32) { return (size_t)2 * C * Mz * (f32 ? sizeof(float2) : sizeof(double2)); }
+size_t smem_zcols(int C, int Mz) { return (size_t)C * Mz * 16; }   // two FP32 buffers, or one of fxc
 
 template <typename F>
 cudaError_t optin3(F* fn, int optin_bytes) {
@@ -900,37 +1038,25 @@ cudaError_t optin3(F* fn, int optin_bytes) {
 
 }  // namespace
 
-namespace {
-constexpr size_t kXfusedSmemMax = 227 * 1024;
-}
-bool xfused3_inplace(int Mx, int f32) {
-  return !f32 && (size_t)36 * Mx * sizeof(double2) > kXfusedSmemMax && Mx <= kIpMaxN;
-}
 size_t smem_xfused3(int Mx, int f32) {
-  const size_t es = f32 ? sizeof(float2) : sizeof(double2);
-  const size_t b = (xfused3_inplace(Mx, f32) ? 18 : 36) * (size_t)Mx * es;
-  return b <= kXfusedSmemMax ? b : 0;
+  (void)f32;                                   // two FP32 buffers take what one of fxc takes
+  const size_t b = (size_t)18 * Mx * 16;
+  return b <= kSmemMax - 2048 ? b : 0;
 }
 size_t spec3_scratch_columns() { return kScr3; }
-size_t smem_zcols3(int C, int Mz, int f32) { return smem_zcols(C, Mz, f32); }
+size_t smem_zcols3(int C, int Mz) { return smem_zcols(C, Mz); }
 
 cudaError_t set_kernel_attributes3(int optin_bytes) {
   cudaError_t e;
-  if ((e = optin3(k_ycols<double2>, optin_bytes))) return e;
   if ((e = optin3(k_ycols<float2>, optin_bytes))) return e;
-  if ((e = optin3(k_ycols<dsc>, optin_bytes))) return e;
-  if ((e = optin3(k_zcols<dsc>, optin_bytes))) return e;
-  if ((e = optin3(k_xfused3<dsc>, optin_bytes))) return e;
-  if ((e = optin3(k_xfused3<dsc, true>, optin_bytes))) return e;
-  if ((e = optin3(k_zcols<double2>, optin_bytes))) return e;
-  if ((e = optin3(k_zcols<float2>, optin_bytes))) return e;
-  if ((e = optin3(k_zcols<double2, true>, optin_bytes))) return e;
-  if ((e = optin3(k_zcols<dsc, true>, optin_bytes))) return e;
-  if ((e = optin3(k_ycols<dsc, true>, optin_bytes))) return e;
-  if ((e = optin3(k_ycols<double2, true>, optin_bytes))) return e;
-  if ((e = optin3(k_xfused3<double2>, optin_bytes))) return e;
-  if ((e = optin3(k_xfused3<float2>, optin_bytes))) return e;
-  if ((e = optin3(k_xfused3<double2, true>, optin_bytes))) return e;
+  if ((e = optin3(k_ycols<fxc>, optin_bytes))) return e;
+  if ((e = optin3(k_ycols<fxc, true>, optin_bytes))) return e;
+  if ((e = optin3(k_zcols, optin_bytes))) return e;
+  if ((e = optin3(k_zcols_fx<false>, optin_bytes))) return e;
+  if ((e = optin3(k_zcols_fx<true>, optin_bytes))) return e;
+  if ((e = optin3(k_xfused3, optin_bytes))) return e;
+  if ((e = optin3(k_xfused3_fx<256, 4>, optin_bytes))) return e;
+  if ((e = optin3(k_xfused3_fx<512, 1>, optin_bytes))) return e;
   if ((e = optin3(k_xrows, optin_bytes))) return e;
   return cudaSuccess;
 }
@@ -946,46 +1072,41 @@ cudaError_t launch_stage3(const GroupDev& g, int stage, cudaStream_t st, int* nl
   const long long yplane = (long long)M * KZ;          // Y3 / V3 field size
   const long long zplane = (long long)M * Mz * K;      // Z3 / W3 field size
   const int f32 = g.f32;
-  // element format of the padded-grid intermediates (double-single values
-  // in the FP64 arrays of PTT_FP64_DS groups)
-  const int fmt = g.ds ? kFmtDS : f32;
   int n = 0;
   switch (stage) {
     case 0: {  // inverse y (17 fields) then inverse z (26 lines)
-      YJob J = yjob3(g, true, M, g.Ccol, g.plP, g.tw4Pi);
+      YJob J = yjob3(g, true, M, g.Ccol, g.plP, true);
       J.src = g.X;
       J.dst = f32 ? (void*)g.Y3f : (void*)g.Y3;
-      J.dst_f32 = fmt;
+      J.dst_f32 = f32;
       J.src_mstride = 9 * NK; J.dst_mstride = 17 * yplane;
       J.src_fstride = NK; J.dst_fstride = yplane;
       const int sf[17] = {0, 1, 2, 3, 4, 5, 6, 7, 8, 0, 2, 3, 4, 5, 6, 7, 8};
       const int dv[17] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 1, 1};
-      const size_t sm = smem_ycols(g.Ccol, M, f32);
       for (int i = 0; i < 17; ++i) { J.src_field[i] = sf[i]; J.dst_field[i] = i; J.deriv[i] = dv[i]; }
+      const dim3 grid(cdiv(KZ, g.Ccol), 17, g.nb);
       if (f32 && g.ymma) {
         cudaError_t e = launch_cheb_mma(g, true, st, g.nsm);
         if (e) return e;
       } else if (f32) {
-        k_ycols<float2><<<dim3(cdiv(KZ, g.Ccol), 17, g.nb), 256, sm, st>>>(J);
-      } else if (g.ds) {
-        k_ycols<dsc><<<dim3(cdiv(KZ, g.Ccol), 17, g.nb), 256, sm, st>>>(J);
+        k_ycols<float2><<<grid, 256, smem_ycols(g.Ccol, M), st>>>(J);
       } else {
-        k_ycols<double2><<<dim3(cdiv(KZ, g.Ccol), 17, g.nb), 256, sm, st>>>(J);
+        k_ycols<fxc><<<grid, 256, smem_ycols_fx(g.Ccol, M, g.N), st>>>(J);
       }
       ++n;
-      if (f32) {   // the mean column (kx = kz = 0) in double-single, FP64 out
+      if (f32) {   // the mean column (kx = kz = 0) in fixed point, FP64 out
         YJob Jm = J;
         Jm.K = 1; Jm.C = 1; Jm.pl = g.plPn;
         Jm.dst = g.Ym; Jm.dst_f32 = 0;
         Jm.dst_mstride = 17LL * M; Jm.dst_fstride = M;
         Jm.vm = 1; Jm.vj = 1;
-        k_ycols<dsc><<<dim3(1, 17, g.nb), 256, smem_ycols(1, M, 0), st>>>(Jm);
+        k_ycols<fxc><<<dim3(1, 17, g.nb), 256, smem_ycols_fx(1, M, g.N), st>>>(Jm);
         ++n;
       }
       ZJob Z = zjob(g, true, Mz, M, g.plMz);
       Z.C = g.zC;
-      Z.src = J.dst; Z.src_f32 = fmt;
-      Z.dst = f32 ? (void*)g.Z3f : (void*)g.Z3; Z.dst_f32 = fmt;
+      Z.src = J.dst;
+      Z.dst = f32 ? (void*)g.Z3f : (void*)g.Z3;
       Z.mean = f32 ? 1 : 0;
       Z.src_mstride = 17 * yplane; Z.dst_mstride = 26 * zplane;
       Z.src_fstride = yplane; Z.dst_fstride = zplane;
@@ -994,62 +1115,58 @@ cudaError_t launch_stage3(const GroupDev& g, int stage, cudaStream_t st, int* nl
         Z.dst_field[i] = i;
         Z.dz[i] = (i >= 17) ? 1 : 0;
       }
-      const size_t smz = smem_zcols(Z.C, Mz, f32);
-      if (f32) k_zcols<float2><<<dim3(cdiv(K, Z.C), 26 * M, g.nb), 256, smz, st>>>(Z);
-      else if (g.ds) k_zcols<dsc><<<dim3(cdiv(K, Z.C), 26 * M, g.nb), 256, smz, st>>>(Z);
-      else k_zcols<double2><<<dim3(cdiv(K, Z.C), 26 * M, g.nb), 256, smz, st>>>(Z);
+      const dim3 zgrid(cdiv(K, Z.C), 26 * M, g.nb);
+      if (f32) k_zcols<<<zgrid, 256, smem_zcols(Z.C, Mz), st>>>(Z);
+      else k_zcols_fx<false><<<zgrid, 256, smem_zcols(Z.C, Mz), st>>>(Z);
       ++n;
       break;
     }
-    case 1:
-      if (f32) k_xfused3<float2><<<dim3(M * Mz, g.nb), g.xthreads, smem_xfused3(g.Mx, 1), st>>>(g);
-      else if (g.ds && xfused3_inplace(g.Mx, 0))
-        k_xfused3<dsc, true><<<dim3(M * Mz, g.nb), kIpThreads, smem_xfused3(g.Mx, 0), st>>>(g);
-      else if (g.ds) k_xfused3<dsc><<<dim3(M * Mz, g.nb), g.xthreads, smem_xfused3(g.Mx, 0), st>>>(g);
-      else if (xfused3_inplace(g.Mx, 0))
-        k_xfused3<double2, true><<<dim3(M * Mz, g.nb), kIpThreads, smem_xfused3(g.Mx, 0), st>>>(g);
-      else k_xfused3<double2><<<dim3(M * Mz, g.nb), g.xthreads, smem_xfused3(g.Mx, 0), st>>>(g);
+    case 1: {
+      const dim3 grid(M * Mz, g.nb);
+      const size_t sm = smem_xfused3(g.Mx, f32);
+      if (f32) k_xfused3<<<grid, g.xthreads, sm, st>>>(g);
+      else if (g.xthreads <= 256) k_xfused3_fx<256, 4><<<grid, g.xthreads, sm, st>>>(g);
+      else k_xfused3_fx<512, 1><<<grid, g.xthreads, sm, st>>>(g);
       n = 1;
       break;
+    }
     case 2: {  // forward z (9) then forward y (9)
       ZJob Z = zjob(g, false, Mz, M, g.plMz);
       Z.C = g.zC;
-      Z.src = f32 ? (const void*)g.W3f : (const void*)g.W3; Z.src_f32 = fmt;
-      Z.dst = f32 ? (void*)g.V3f : (void*)g.V3; Z.dst_f32 = fmt;
+      Z.src = f32 ? (const void*)g.W3f : (const void*)g.W3;
+      Z.dst = f32 ? (void*)g.V3f : (void*)g.V3;
       Z.mean = f32 ? 2 : 0;
       Z.zm = g.Zm;
+      Z.inv = 1.0;   // fixed point: the y table holds the normalisation
       Z.src_mstride = 9 * zplane; Z.dst_mstride = 9 * yplane;
       Z.src_fstride = zplane; Z.dst_fstride = yplane;
       for (int i = 0; i < 9; ++i) { Z.src_field[i] = i; Z.dst_field[i] = i; Z.dz[i] = 0; }
-      const size_t smz = smem_zcols(Z.C, Mz, f32);
-      if (f32) k_zcols<float2><<<dim3(cdiv(K, Z.C), 9 * M, g.nb), 256, smz, st>>>(Z);
-      else if (g.ds) k_zcols<dsc><<<dim3(cdiv(K, Z.C), 9 * M, g.nb), 256, smz, st>>>(Z);
-      else k_zcols<double2><<<dim3(cdiv(K, Z.C), 9 * M, g.nb), 256, smz, st>>>(Z);
-      YJob F = yjob3(g, false, M, g.Ccol, g.plP, g.tw4P);
-      F.src = Z.dst; F.src_f32 = fmt;
+      const dim3 zgrid(cdiv(K, Z.C), 9 * M, g.nb);
+      if (f32) k_zcols<<<zgrid, 256, smem_zcols(Z.C, Mz), st>>>(Z);
+      else k_zcols_fx<false><<<zgrid, 256, smem_zcols(Z.C, Mz), st>>>(Z);
+      YJob F = yjob3(g, false, M, g.Ccol, g.plP, true);
+      F.src = Z.dst; F.src_f32 = f32;
       F.dst = g.NR;
       F.src_mstride = 9 * yplane; F.dst_mstride = 9 * NK;
       F.src_fstride = yplane; F.dst_fstride = NK;
-      const size_t sm = smem_ycols(g.Ccol, M, f32);
       for (int i = 0; i < 9; ++i) { F.src_field[i] = i; F.dst_field[i] = i; F.deriv[i] = 0; }
+      const dim3 grid(cdiv(KZ, g.Ccol), 9, g.nb);
       if (f32 && g.ymma) {
         cudaError_t e = launch_cheb_mma(g, false, st, g.nsm);
         if (e) return e;
       } else if (f32) {
-        k_ycols<float2><<<dim3(cdiv(KZ, g.Ccol), 9, g.nb), 256, sm, st>>>(F);
-      } else if (g.ds) {
-        k_ycols<dsc><<<dim3(cdiv(KZ, g.Ccol), 9, g.nb), 256, sm, st>>>(F);
+        k_ycols<float2><<<grid, 256, smem_ycols(g.Ccol, M), st>>>(F);
       } else {
-        k_ycols<double2><<<dim3(cdiv(KZ, g.Ccol), 9, g.nb), 256, sm, st>>>(F);
+        k_ycols<fxc><<<grid, 256, smem_ycols_fx(g.Ccol, M, 0), st>>>(F);
       }
       n = 2;
-      if (f32) {   // the mean column in double-single, over the FP32 pass's zeros
+      if (f32) {   // the mean column in fixed point, over the FP32 pass's zeros
         YJob Fm = F;
         Fm.K = 1; Fm.C = 1; Fm.pl = g.plPn;
         Fm.src = g.Zm; Fm.src_f32 = 0;
         Fm.src_mstride = 9LL * M; Fm.src_fstride = M;
         Fm.vm = 1; Fm.vj = 1;
-        k_ycols<dsc><<<dim3(1, 9, g.nb), 256, smem_ycols(1, M, 0), st>>>(Fm);
+        k_ycols<fxc><<<dim3(1, 9, g.nb), 256, smem_ycols_fx(1, M, 0), st>>>(Fm);
         ++n;
       }
       break;
@@ -1092,28 +1209,26 @@ static cudaError_t diag_join3(const DiagStreams& d) {
 static void diag_energy_y3(const GroupDev& g, cudaStream_t st) {
   const int KZ = g.KZ;
   const size_t NK = (size_t)g.N * KZ;
-  YJob J = yjob3(g, true, g.Me, g.CcolE, g.plPe, g.tw4E);
+  YJob J = yjob3(g, true, g.Me, g.CcolE, g.plPe, true);
   J.tw4f = g.tw4Ef;   // mixed groups transform in FP32 (the sums stay FP64)
-  J.tw4d = g.tw4Ed;   // double-single groups in double-single
+  J.tw4x = g.tw4Ex;
   J.src = g.X; J.dst = g.DY;
   J.src_mstride = 9 * NK; J.dst_mstride = 3LL * g.Me * KZ;
   J.src_fstride = NK; J.dst_fstride = (long long)g.Me * KZ;
   for (int i = 0; i < 3; ++i) { J.src_field[i] = i; J.dst_field[i] = i; J.deriv[i] = 0; }
-  if (g.f32) k_ycols<float2><<<dim3(cdiv(KZ, g.CcolE), 3, g.nb), 256, smem_ycols(g.CcolE, g.Me, 1), st>>>(J);
-  else if (g.ds) k_ycols<dsc><<<dim3(cdiv(KZ, g.CcolE), 3, g.nb), 256, smem_ycols(g.CcolE, g.Me, 0), st>>>(J);
-  else k_ycols<double2><<<dim3(cdiv(KZ, g.CcolE), 3, g.nb), 256, smem_ycols(g.CcolE, g.Me, 0), st>>>(J);
+  const dim3 grid(cdiv(KZ, g.CcolE), 3, g.nb);
+  if (g.f32) k_ycols<float2><<<grid, 256, smem_ycols(g.CcolE, g.Me), st>>>(J);
+  else k_ycols<fxc><<<grid, 256, smem_ycols_fx(g.CcolE, g.Me, 0), st>>>(J);
 }
 static void diag_trc_y3(const GroupDev& g, cudaStream_t st) {
   const int KZ = g.KZ;
   const size_t NK = (size_t)g.N * KZ;
-  YJob T = yjob3(g, true, g.N - 1, g.CcolU, g.plPu, nullptr);
+  YJob T = yjob3(g, true, g.N - 1, g.CcolU, g.plPu, false);
   T.src = g.X; T.dst = g.DT;
   T.src_mstride = 9 * NK; T.dst_mstride = (long long)NK;
   T.src_fstride = NK; T.dst_fstride = 0;
   T.src_field[0] = 3; T.src_field2[0] = 6; T.src_field3[0] = 8; T.dst_field[0] = 0; T.deriv[0] = 0;
-  if (g.ds || g.f32)   // double-single (FP64 in and out, FP64 sums downstream)
-    k_ycols<dsc, true><<<dim3(cdiv(KZ, g.CcolU), 1, g.nb), 256, smem_ycols(g.CcolU, g.Pu, 0), st>>>(T);
-  else k_ycols<double2, true><<<dim3(cdiv(KZ, g.CcolU), 1, g.nb), 256, smem_ycols(g.CcolU, g.Pu, 0), st>>>(T);
+  k_ycols<fxc, true><<<dim3(cdiv(KZ, g.CcolU), 1, g.nb), 256, smem_ycols_fx(g.CcolU, g.Pu, 0), st>>>(T);
 }
 
 cudaError_t launch_diag_transforms3(const GroupDev& g, cudaStream_t st) {
@@ -1131,13 +1246,11 @@ cudaError_t launch_diag_split3(const GroupDev& g, const DiagStreams& d, int* nl)
   // mid-plane: per-mode sums, then z and x syntheses of the 8 quantities
   k_diag_mid3<<<dim3(cdiv(KZ, kMidModesPerBlock3), g.nb), 256, 0, d.s[2]>>>(g);
   ZJob Zm = zjob(g, true, g.nz, 1, g.plNz);
-  Zm.src = g.DM; Zm.src_f32 = 0; Zm.dst = g.DMZ; Zm.dst_f32 = 0;
+  Zm.src = g.DM; Zm.dst = g.DMZ;
   Zm.src_mstride = 8LL * KZ; Zm.dst_mstride = 8LL * g.nz * K;
   Zm.src_fstride = KZ; Zm.dst_fstride = (long long)g.nz * K;
   for (int i = 0; i < 8; ++i) { Zm.src_field[i] = i; Zm.dst_field[i] = i; Zm.dz[i] = 0; }
-  if (g.ds || g.f32)
-    k_zcols<dsc, true><<<dim3(cdiv(K, Zm.C), 8, g.nb), 256, smem_zcols(Zm.C, g.nz, 0), d.s[2]>>>(Zm);
-  else k_zcols<double2, true><<<dim3(cdiv(K, Zm.C), 8, g.nb), 256, smem_zcols(Zm.C, g.nz, 0), d.s[2]>>>(Zm);
+  k_zcols_fx<true><<<dim3(cdiv(K, Zm.C), 8, g.nb), 256, smem_zcols(Zm.C, g.nz), d.s[2]>>>(Zm);
   XJob Xm{};
   Xm.srcC = g.DMZ; Xm.dstR = g.MV;
   Xm.src_mstride = 8LL * g.nz * K; Xm.dst_mstride = 8LL * g.nz * g.nx;
@@ -1148,21 +1261,19 @@ cudaError_t launch_diag_split3(const GroupDev& g, const DiagStreams& d, int* nl)
   // Tr c = c_xx + c_yy + c_zz on the unpadded grid: y (Gauss-Lobatto) -> z -> x
   diag_trc_y3(g, d.s[0]);
   ZJob Z = zjob(g, true, g.nz, g.N, g.plNz);
-  Z.src = g.DT; Z.src_f32 = 0; Z.dst = g.DZ; Z.dst_f32 = 0;
+  Z.src = g.DT; Z.dst = g.DZ;
   Z.src_mstride = (long long)NK; Z.dst_mstride = (long long)g.N * g.nz * K;
   Z.src_fstride = 0; Z.dst_fstride = 0;
   Z.src_field[0] = 0; Z.dst_field[0] = 0; Z.dz[0] = 0;
-  if (g.ds || g.f32)
-    k_zcols<dsc, true><<<dim3(cdiv(K, Z.C), g.N, g.nb), 256, smem_zcols(Z.C, g.nz, 0), d.s[0]>>>(Z);
-  else k_zcols<double2, true><<<dim3(cdiv(K, Z.C), g.N, g.nb), 256, smem_zcols(Z.C, g.nz, 0), d.s[0]>>>(Z);
+  k_zcols_fx<true><<<dim3(cdiv(K, Z.C), g.N, g.nb), 256, smem_zcols(Z.C, g.nz), d.s[0]>>>(Z);
   XJob X{};
   X.srcC = g.DZ; X.dstR = g.DV;
   X.src_mstride = (long long)g.N * g.nz * K; X.dst_mstride = (long long)g.N * g.nz * g.nx;
   X.src_fstride = 0; X.dst_fstride = 0;
   X.src_rstep = 1; X.dst_rstep = 1;
   X.nf = 1; X.K = K; X.n = g.nx; X.c2r = 1; X.status = g.status; X.pl = g.plNx;
-  X.pair_rows = 1; X.nrows = g.N * g.nz;
-  k_xrows<<<dim3(cdiv(g.N * g.nz, 2), g.nb), 256, smem_xrows(1, g.nx), d.s[0]>>>(X);
+  X.nrows = g.N * g.nz; X.pair_rows = xrows_pairs(g.nx, X.nrows * g.nb);
+  k_xrows<<<dim3(xrows_pair_blocks(X.pair_rows, X.nrows), g.nb), 256, smem_xrows(X.pair_rows, g.nx), d.s[0]>>>(X);
   if ((e = cudaGetLastError()) || (e = diag_join3(d))) return e;
   k_diag_part3<<<dim3(g.ntile, g.nb), 256, 0, d.s[0]>>>(g);
   k_diag_count3<<<dim3(g.ntile, g.nb), 256, 0, d.s[0]>>>(g);
@@ -1212,13 +1323,13 @@ cudaError_t launch_phys_to_state3(const GroupDev& g, int b, cudaStream_t st) {
   Z.src = g.DZ; Z.dst = g.stageS;     // stageS reused as [9][N][KZ]
   Z.src_fstride = rowsp * K; Z.dst_fstride = (long long)N * KZ;
   for (int i = 0; i < 9; ++i) { Z.src_field[i] = i; Z.dst_field[i] = i; Z.dz[i] = 0; }
-  k_zcols<double2, true><<<dim3(cdiv(K, Z.C), 9 * N, 1), 256, smem_zcols(Z.C, nz, 0), st>>>(Z);
-  YJob J = yjob3(g, false, N - 1, g.CcolU, g.plPu, nullptr);
+  k_zcols_fx<true><<<dim3(cdiv(K, Z.C), 9 * N, 1), 256, smem_zcols(Z.C, nz), st>>>(Z);
+  YJob J = yjob3(g, false, N - 1, g.CcolU, g.plPu, false);
   J.status = nullptr;
   J.src = g.stageS; J.dst = g.X + (size_t)b * 9 * NK;
   J.src_fstride = (long long)N * KZ; J.dst_fstride = NK;
   for (int i = 0; i < 9; ++i) { J.src_field[i] = i; J.dst_field[i] = i; J.deriv[i] = 0; }
-  k_ycols<double2, true><<<dim3(cdiv(KZ, g.CcolU), 9, 1), 256, smem_ycols(g.CcolU, g.Pu, 0), st>>>(J);
+  k_ycols<fxc, true><<<dim3(cdiv(KZ, g.CcolU), 9, 1), 256, smem_ycols_fx(g.CcolU, g.Pu, 0), st>>>(J);
   k_reset3<<<1, 32, 0, st>>>(g, b);
   return cudaGetLastError();
 }
@@ -1227,18 +1338,18 @@ cudaError_t launch_state_to_phys3(const GroupDev& g, int b, cudaStream_t st) {
   const int K = g.K, KZ = g.KZ, N = g.N, nz = g.nz, nx = g.nx;
   const size_t NK = (size_t)N * KZ;
   const long long rowsp = (long long)N * nz;
-  YJob J = yjob3(g, true, N - 1, g.CcolU, g.plPu, nullptr);
+  YJob J = yjob3(g, true, N - 1, g.CcolU, g.plPu, false);
   J.status = nullptr;
   J.src = g.X + (size_t)b * 9 * NK; J.dst = g.stageS;
   J.src_fstride = NK; J.dst_fstride = (long long)N * KZ;
   for (int i = 0; i < 9; ++i) { J.src_field[i] = i; J.dst_field[i] = i; J.deriv[i] = 0; }
-  k_ycols<double2, true><<<dim3(cdiv(KZ, g.CcolU), 9, 1), 256, smem_ycols(g.CcolU, g.Pu, 0), st>>>(J);
+  k_ycols<fxc, true><<<dim3(cdiv(KZ, g.CcolU), 9, 1), 256, smem_ycols_fx(g.CcolU, g.Pu, 0), st>>>(J);
   ZJob Z = zjob(g, true, nz, N, g.plNz);
   Z.status = nullptr;
   Z.src = g.stageS; Z.dst = g.DZ;
   Z.src_fstride = (long long)N * KZ; Z.dst_fstride = rowsp * K;
   for (int i = 0; i < 9; ++i) { Z.src_field[i] = i; Z.dst_field[i] = i; Z.dz[i] = 0; }
-  k_zcols<double2, true><<<dim3(cdiv(K, Z.C), 9 * N, 1), 256, smem_zcols(Z.C, nz, 0), st>>>(Z);
+  k_zcols_fx<true><<<dim3(cdiv(K, Z.C), 9 * N, 1), 256, smem_zcols(Z.C, nz), st>>>(Z);
   XJob X{};
   X.srcC = g.DZ; X.dstR = g.stage;
   X.src_fstride = rowsp * K; X.dst_fstride = rowsp * nx;

@@ -75,10 +75,9 @@ extern "C" int ptt_explicit_rhs_noalloc(const ptt_params* p, const double* d_spe
   if (((uintptr_t)d_spec & 15) || ((uintptr_t)d_out & 15) || d_spec == d_out) return PTT_EINVAL;
   ptt::GroupDev g{};
   ptt::MemberPrm prm{};
-  std::vector<double2> twP, twMx, tw4;
-  std::vector<double> tt[2];
-  std::vector<int> tk[2];
-  int s = ptt::shape_plan(*p, g, twP, twMx, tw4, prm, tt, tk);
+  std::vector<int4> tables;   // twiddles of the two plans, forward and inverse quarter tables
+  size_t toff[4];
+  int s = ptt::shape_plan(*p, g, tables, toff, prm);
   if (s) return s;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   {
@@ -106,14 +105,7 @@ extern "C" int ptt_explicit_rhs_noalloc(const ptt_params* p, const double* d_spe
   const size_t oRb = off; off = align256(off + 2 * NK * sizeof(double2));
   const size_t oYp = off; off = align256(off + 9 * rows * K * sizeof(double2));
   const size_t oZp = off; off = align256(off + 5 * rows * K * sizeof(double2));
-  const size_t oTP = off; off = align256(off + twP.size() * sizeof(double2));
-  const size_t oTM = off; off = align256(off + twMx.size() * sizeof(double2));
-  const size_t oT4 = off; off = align256(off + tw4.size() * sizeof(double2));
-  size_t oTT[2], oTK[2];
-  for (int i = 0; i < 2; ++i) {
-    oTT[i] = off; off = align256(off + tt[i].size() * sizeof(double));
-    oTK[i] = off; off = align256(off + tk[i].size() * sizeof(int));
-  }
+  const size_t oTw = off; off = align256(off + tables.size() * sizeof(int4));
   const size_t oPr = off; off = align256(off + sizeof(ptt::MemberPrm));
   const size_t oSt = off; off = align256(off + sizeof(int));
   const size_t oCn = off; off = align256(off + sizeof(long long));
@@ -135,15 +127,10 @@ extern "C" int ptt_explicit_rhs_noalloc(const ptt_params* p, const double* d_spe
   g.Rb = (double2*)(b + oRb);   // H_x, H_y
   g.Yp = (double2*)(b + oYp);
   g.Zp = (double2*)(b + oZp);
-  g.plP.tw = (const double2*)(b + oTP);
-  g.plMx.tw = (const double2*)(b + oTM);
-  ptt::FftPlan* pls[2] = {&g.plP, &g.plMx};
-  for (int i = 0; i < 2; ++i) {
-    pls[i]->tt = (const double*)(b + oTT[i]);
-    pls[i]->tk = (const int*)(b + oTK[i]);
-  }
-  g.tw4P = (const double2*)(b + oT4);                      // forward table, M entries
-  g.tw4Pi = (const double2*)(b + oT4) + tw4.size() / 2;    // inverse table, M entries
+  g.plP.twx = (const int4*)(b + oTw) + toff[0];
+  g.plMx.twx = (const int4*)(b + oTw) + toff[1];
+  g.tw4Px = (const int4*)(b + oTw) + toff[2];
+  g.tw4Pix = (const int4*)(b + oTw) + toff[3];
   g.prm = (ptt::MemberPrm*)(b + oPr);
   g.status = (int*)(b + oSt);
   g.count = (long long*)(b + oCn);
@@ -152,18 +139,8 @@ extern "C" int ptt_explicit_rhs_noalloc(const ptt_params* p, const double* d_spe
   // rewritten on every call (the array keeps the previous call's contents)
   e = cudaMemsetAsync(b + oSt, 0, sizeof(int), st);
   if (!e) e = cudaMemsetAsync(b + oCn, 0, sizeof(long long), st);
-  if (!e) e = cudaMemcpyAsync(b + oTP, twP.data(), twP.size() * sizeof(double2),
+  if (!e) e = cudaMemcpyAsync(b + oTw, tables.data(), tables.size() * sizeof(int4),
                               cudaMemcpyHostToDevice, st);
-  if (!e) e = cudaMemcpyAsync(b + oTM, twMx.data(), twMx.size() * sizeof(double2),
-                              cudaMemcpyHostToDevice, st);
-  if (!e) e = cudaMemcpyAsync(b + oT4, tw4.data(), tw4.size() * sizeof(double2),
-                              cudaMemcpyHostToDevice, st);
-  for (int i = 0; i < 2 && !e; ++i) {
-    e = cudaMemcpyAsync(b + oTT[i], tt[i].data(), tt[i].size() * sizeof(double),
-                        cudaMemcpyHostToDevice, st);
-    if (!e) e = cudaMemcpyAsync(b + oTK[i], tk[i].data(), tk[i].size() * sizeof(int),
-                                cudaMemcpyHostToDevice, st);
-  }
   if (!e) e = cudaMemcpyAsync(b + oPr, &prm, sizeof(prm), cudaMemcpyHostToDevice, st);
   if (!e) e = ptt::launch_transpose((const double2*)d_spec, g.X, 5, g.N, g.K, st);
   if (!e) e = ptt::launch_explicit(g, st);
