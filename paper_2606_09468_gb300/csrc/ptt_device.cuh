@@ -627,130 +627,167 @@ __device__ void warp_qt_solve(int N, int p, double alpha, const double2* R, doub
 // Lane-sequential forms for the per-mode spectral stage: one lane owns one
 // (Fourier mode, Chebyshev parity) pair and walks its ~N/2 coefficients in
 // order, so a warp advances 32 independent recurrences with every lane busy.
-// Columns are indexed by n (stride 1); a lane touches only n = p mod 2 on
-// input and, for the derivative, only n = 1 - p mod 2 on output.
+// Columns are indexed by n (stride 1).  Bound by the FP64 pipe (64 cycles per
+// warp instruction, as long as its latency: one warp keeps a sub-partition's
+// pipe full), so whatever can be formed on the way through a recurrence is
+// (the loads of the next row are issued before the current row's arithmetic),
+// and what needs no FP64 instruction has none.
 
-// Chebyshev derivative, parity half: from the inputs a_k, k = p mod 2, the
-// outputs b_{k-1} = (k == 1 ? 1 : 2) sum_{k' >= k, k' = k mod 2} k' a_{k'}
-// (b_{n-1} = b_{n+1} + 2 n a_n, b_0 halved); the lane whose output parity is
-// that of N - 1 also writes b_{N-1} = 0.  The two lanes of one column
-// together produce the whole derivative; `out` must not alias `a`.
-__device__ __forceinline__ void lane_cheb_deriv(const double2* __restrict__ a,
-                                                double2* __restrict__ out, int N, int p) {
-  const int top = ((N - 1 - p) & ~1) + p;   // largest k = p mod 2 below N
+// 0 <= k < 2^24 as a double, x / 2 where z holds: integer instructions.
+__device__ __forceinline__ double lane_i2d(int k) { return f64_from_f32((float)k); }
+__device__ __forceinline__ double lane_half(double x, bool z) {
+  const int h = __double2hiint(x);
+  const bool scale = z && (((unsigned)h >> 20) & 0x7FFu) - 2u < 2045u;   // normal, result normal
+  return __hiloint2double(scale ? h - 0x100000 : h, __double2loint(x));
+}
+__device__ __forceinline__ double2 lane_half2(double2 v, bool z) {
+  return make_double2(lane_half(v.x, z), lane_half(v.y, z));
+}
+
+// Explicit momentum term of one component, outputs n = p mod 2:
+//   out_n = nr_n + gam ((D cy)_n + i (kx cx_n + kz cz_n)),
+// (D cy)_n = sum over k = n + 1, n + 3, ... of 2 k cy_k, halved at n = 0.
+__device__ __forceinline__ void lane_div_h(int N, int p, const double2* __restrict__ cy,
+                                           const double2* __restrict__ cx, const double2* __restrict__ cz,
+                                           const double2* __restrict__ nr, double gam, double gkx, double gkz,
+                                           double2* __restrict__ out) {
+  const int nl = ((N - 1 - p) & ~1) + p;
   double2 acc = czero();
 #pragma unroll 4
-  for (int k = top; k >= 1; k -= 2) {
-    acc = cfma((double)k, a[k], acc);
-    out[k - 1] = cscl(acc, k == 1 ? 1.0 : 2.0);
+  for (int n = nl; n >= p; n -= 2) {
+    const int k = min(n + 1, N - 1);   // n = N - 1 has no term: times 0
+    acc = cfma(n + 1 < N ? lane_i2d(2 * k) : 0.0, cy[k], acc);
+    const double2 a = cx[n], c = cz[n], d = lane_half2(acc, n == 0);
+    double2 h = cfma(gam, d, nr[n]);
+    h.x = fma(-gkz, c.y, fma(-gkx, a.y, h.x));
+    h.y = fma(gkz, c.x, fma(gkx, a.x, h.y));
+    out[n] = h;
   }
-  if (((N - 1) & 1) != p) out[N - 1] = czero();
 }
 
-// Quasi-tridiagonal tau solve of one parity (system stated at k_spec):
-// backward elimination P_n = (r_n - u_n P_{n+2}) inv_n with the three-term
-// right-hand side r_n of the twice-integrated rows, accumulating the
-// boundary sum U = sum F_n P_n; the boundary row gives
-// a_p = (bcfac sum_{n = p} R_n - U) G; forward substitution
-// a_n = P_n + Q_n a_{n-2}.  Q, inv, F: the right-hand-side-independent
-// elimination factors of this (alpha, mode, parity), precomputed on the
-// host.  The solve runs on R and flips the result's sign when the system's
-// right-hand side is rsign R with rsign = -1.  `out` must not alias R (every
-// input is independent of the recurrence, so unrolled iterations keep
-// several loads in flight).
-__device__ __forceinline__ void lane_qt_solve(int N, int p, double alpha,
-                                              const double2* __restrict__ R,
-                                              double2* __restrict__ out,
-                                              const double* __restrict__ Q,
-                                              const double* __restrict__ inv,
-                                              const double* __restrict__ F, double G,
-                                              const double* __restrict__ w1,
-                                              const double* __restrict__ w2,
-                                              const double* __restrict__ w3, double bcfac,
-                                              double rsign) {
+// q_n = (D^2 v)_n - k2 v_n for n = p mod 2 (the inner derivative's entries of
+// the other parity stay in a register).
+__device__ __forceinline__ void lane_lap(int N, int p, const double2* __restrict__ v, double k2,
+                                         double2* __restrict__ out) {
   const int nl = ((N - 1 - p) & ~1) + p;
-  double2 Pn2 = czero(), U = czero(), rs = czero(), Rp2 = czero();
-  double2 R0 = R[nl];
+  double2 a1 = czero(), a2 = czero(), vp = czero();   // vp = v_{n+2}
 #pragma unroll 4
+  for (int n = nl; n >= p; n -= 2) {
+    a1 = cfma(lane_i2d(2 * (n + 2)), vp, a1);   // (D v)_{n+1}
+    a2 = cfma(lane_i2d(2 * (n + 1)), a1, a2);
+    vp = v[n];
+    out[n] = cfma(-k2, vp, lane_half2(a2, n == 0));
+  }
+}
+
+// One row of the histories of an evolved column: the current values x, nn and
+// the older slots (E: values, Nn: explicit terms).
+struct LaneHist {
+  const double2 *E0, *E1, *E2;
+  ptrdiff_t dn;    // from a slot of E to that of N
+  double ca[4];    // -sa_{j+1}/dt
+  int o;           // order - 1
+};
+struct LaneRow { double2 e[3], m[3]; };
+template <bool FULL>
+__device__ __forceinline__ LaneRow lane_hist_row(const LaneHist& h, int n) {
+  LaneRow r;
+  if (FULL || h.o >= 1) { r.e[0] = h.E0[n]; r.m[0] = h.E0[n + h.dn]; }
+  if (FULL || h.o >= 2) { r.e[1] = h.E1[n]; r.m[1] = h.E1[n + h.dn]; }
+  if (FULL) { r.e[2] = h.E2[n]; r.m[2] = h.E2[n + h.dn]; }
+  return r;
+}
+// R = sb_0 nn + sum_j (-sa_{j+1}/dt) x^{n-j} + sum_{j>=1} sb_j N^{n-j}; FULL:
+// order 4, else orders 1 to 3 of the first steps.
+template <bool FULL>
+__device__ __forceinline__ double2 lane_sbdf(const LaneHist& h, const LaneRow& r, double2 x, double2 nn) {
+  const double* cb = c_sb[FULL ? 3 : h.o];
+  double2 acc = cfma(cb[0], nn, cscl(x, h.ca[0]));
+  if (FULL || h.o >= 1) acc = cfma(cb[1], r.m[0], cfma(h.ca[1], r.e[0], acc));
+  if (FULL || h.o >= 2) acc = cfma(cb[2], r.m[1], cfma(h.ca[2], r.e[1], acc));
+  if (FULL) acc = cfma(cb[3], r.m[2], cfma(h.ca[3], r.e[2], acc));
+  return acc;
+}
+
+// Quasi-tridiagonal tau solve of one parity (system stated at k_spec), in two
+// passes.  lane_qt_back: the backward elimination
+//   P_n = inv_n (w2_n R_n - w1_n R_{n-2} - w3_n (R_{n+2} - alpha P_{n+2}))
+// (w1 twice its table at n = 2; no w2 term on the last row, no w3 term on the
+// last two) and the boundary sum U = sum F_n P_n, with rs = sum R_n where SUM;
+// R comes from ld(n) (a row's loads) and ev(row, n), called once for every n
+// in descending order.  lane_qt_fwd: a_p = (bcfac rs - U) G, then
+// a_n = P_n + Q_n a_{n-2}, in place or into out.  Q, inv, F: the
+// right-hand-side-independent elimination factors of this (alpha, mode,
+// parity), precomputed on the host.
+template <bool SUM, typename Ld, typename Ev>
+__device__ __forceinline__ double2 lane_qt_back(int N, int p, double alpha, Ld ld, Ev ev, double2* __restrict__ P,
+                                                const double* __restrict__ inv, const double* __restrict__ F,
+                                                const double* __restrict__ w, double2& rs) {
+  const int nl = ((N - 1 - p) & ~1) + p;
+  auto row = ld(nl);
+  double iv1 = inv[nl], f1 = F[nl];
+  double2 R0 = ev(row, nl), Rp = czero(), Pp = czero(), U = czero();
+  row = ld(max(nl - 2, p));
+  rs = SUM ? R0 : czero();
+#pragma unroll 1
   for (int n = nl; n >= p + 2; n -= 2) {
-    const double2 Rm2 = R[n - 2];
-    const double cc = (n == 2) ? 2.0 : 1.0;
-    double2 r = cscl(Rm2, -cc * w1[n]);
-    if (n <= N - 3) r = cfma(w2[n], R0, r);
-    double un = 0.0;
-    if (n <= N - 5) {
-      r = cfma(-w3[n], Rp2, r);
-      un = -alpha * w3[n];
-    }
-    const double2 P = cscl(cfma(-un, Pn2, r), inv[n]);
-    out[n] = P;
-    U = cfma(F[n], P, U);
-    rs = cadd(rs, R0);
-    Pn2 = P;
-    Rp2 = R0;
-    R0 = Rm2;
+    const double iv = iv1, f = f1;
+    const double w1t = w[n], w2t = w[N + n], w3t = w[2 * N + n];
+    const double2 Rm = ev(row, n - 2);
+    row = ld(max(n - 4, p));   // in flight during the elimination's own arithmetic
+    iv1 = inv[n - 2];
+    f1 = F[n - 2];
+    const double w1 = __hiloint2double(__double2hiint(w1t) + (n == 2 ? 0x100000 : 0), __double2loint(w1t));
+    const double w2 = (n <= N - 3) ? w2t : 0.0, w3 = (n <= N - 5) ? w3t : 0.0;
+    const double2 S = cfma(-alpha, Pp, Rp);
+    const double2 r = cfma(-w3, S, cfma(w2, R0, cscl(Rm, -w1)));
+    const double2 Pn = cscl(r, iv);
+    P[n] = Pn;
+    U = cfma(f, Pn, U);
+    if (SUM) rs = cadd(rs, Rm);
+    Pp = Pn;
+    Rp = R0;
+    R0 = Rm;
   }
-  rs = cadd(rs, R0);   // R_p
-  double2 a = cscl(csub(cscl(rs, bcfac), U), G);
+  return U;
+}
+// use(n, a_n) is called once for every n, in ascending order.
+template <typename Use>
+__device__ __forceinline__ void lane_qt_fwd(int N, int p, double2 a, double2 wall, const double2* P, double2* out,
+                                            const double* __restrict__ Q, Use use) {
+  constexpr int kU = 4;
+  const int nl = ((N - 1 - p) & ~1) + p;
   out[p] = a;
-#pragma unroll 4
-  for (int n = p + 2; n <= nl; n += 2) {
-    a = cfma(Q[n], a, out[n]);
-    out[n] = a;
+  use(p, a);
+  if (nl == p) return;
+  for (int n0 = p + 2; n0 < nl; n0 += 2 * kU) {
+    double2 v[kU];
+    double q[kU];
+#pragma unroll
+    for (int t = 0; t < kU; ++t) {
+      const int n = min(n0 + 2 * t, nl);
+      v[t] = P[n];
+      q[t] = Q[n];
+    }
+#pragma unroll
+    for (int t = 0; t < kU; ++t) {
+      const int n = n0 + 2 * t;
+      if (n < nl) {
+        a = cfma(q[t], a, v[t]);
+        out[n] = a;
+        use(n, a);
+      }
+    }
   }
-  if (nl > p && fabs(Q[nl]) > kTopFromWall) {   // top coefficient from the wall row
+  const double ql = Q[nl];
+  a = cfma(ql, a, P[nl]);
+  if (fabs(ql) > kTopFromWall) {   // top coefficient from the wall row
     double2 part = czero();
     for (int n = p; n < nl; n += 2) part = cadd(part, out[n]);
-    out[nl] = csub(cscl(rs, bcfac), part);
+    a = csub(wall, part);
   }
-  // solved for R; the right-hand side is rsign R
-  if (rsign < 0.0)
-    for (int n = p; n <= nl; n += 2) out[n] = cneg_bits(out[n]);
-}
-
-// SBDF sum of one evolved column, parity p, order index O (0..3: SBDF1-4):
-// writes the current values x, nn into the history slot (E, Nn) and
-// R = sb_0 nn + sum_j (-sa_{j+1}/dt) x^{n-j} + sum_{j>=1} sb_j N^{n-j}
-// over the O older slots Eo[j-1], No[j-1].
-template <int O>
-__device__ __forceinline__ void lane_sbdf(int N, int p, double idt,
-                                          const double2* __restrict__ x,
-                                          const double2* __restrict__ nn,
-                                          double2* __restrict__ E, double2* __restrict__ Nn,
-                                          const double2* __restrict__ Eo0,
-                                          const double2* __restrict__ Eo1,
-                                          const double2* __restrict__ Eo2,
-                                          const double2* __restrict__ No0,
-                                          const double2* __restrict__ No1,
-                                          const double2* __restrict__ No2,
-                                          double2* __restrict__ R) {
-  const double ca0 = -c_sa[O][1] * idt, cb0 = c_sb[O][0];
-  const double ca1 = (O >= 1) ? -c_sa[O][2] * idt : 0.0, cb1 = (O >= 1) ? c_sb[O][1] : 0.0;
-  const double ca2 = (O >= 2) ? -c_sa[O][3] * idt : 0.0, cb2 = (O >= 2) ? c_sb[O][2] : 0.0;
-  const double ca3 = (O >= 3) ? -c_sa[O][4] * idt : 0.0, cb3 = (O >= 3) ? c_sb[O][3] : 0.0;
-#pragma unroll 4
-  for (int n = p; n < N; n += 2) {
-    const double2 xv = x[n], nv = nn[n];
-    E[n] = xv;
-    Nn[n] = nv;
-    double2 acc = cfma(cb0, nv, cscl(xv, ca0));
-    if (O >= 1) acc = cfma(cb1, No0[n], cfma(ca1, Eo0[n], acc));
-    if (O >= 2) acc = cfma(cb2, No1[n], cfma(ca2, Eo1[n], acc));
-    if (O >= 3) acc = cfma(cb3, No2[n], cfma(ca3, Eo2[n], acc));
-    R[n] = acc;
-  }
-}
-
-__device__ __forceinline__ void lane_sbdf_any(int o, int N, int p, double idt, const double2* x,
-                                              const double2* nn, double2* E, double2* Nn,
-                                              const double2* const* Eo, const double2* const* No,
-                                              double2* R) {
-  switch (o) {
-    case 0: lane_sbdf<0>(N, p, idt, x, nn, E, Nn, Eo[0], Eo[1], Eo[2], No[0], No[1], No[2], R); break;
-    case 1: lane_sbdf<1>(N, p, idt, x, nn, E, Nn, Eo[0], Eo[1], Eo[2], No[0], No[1], No[2], R); break;
-    case 2: lane_sbdf<2>(N, p, idt, x, nn, E, Nn, Eo[0], Eo[1], Eo[2], No[0], No[1], No[2], R); break;
-    default: lane_sbdf<3>(N, p, idt, x, nn, E, Nn, Eo[0], Eo[1], Eo[2], No[0], No[1], No[2], R); break;
-  }
+  out[nl] = a;
+  use(nl, a);
 }
 
 // ---------------------------------------------- per-mode spectral stage

@@ -481,22 +481,159 @@ __global__ void __launch_bounds__(512) k_xfused3(GroupDev g) {
 // eta (k != 0) or W; then u = i (kx Dv - kz eta)/k^2, w = i (kz Dv + kx eta)/k^2.
 //
 // A block takes 16 modes; lane l of every warp owns mode l/2 of the block and
-// Chebyshev parity l%2, and each warp runs one component task of a phase, so
-// all recurrences run lane-sequentially with full warps.  Per-mode scratch
-// columns live in SS (workspace; L2-resident while the block runs):
+// Chebyshev parity l%2, and each of the eight warps runs one chain:
+//   V    q1 = (D^2 - k^2) v; then, in one descending pass, its forcing from H,
+//        the history and the SBDF sum and the phi elimination; the v system;
+//        the influence correction with D v
+//   Q2   q2, its forcing, SBDF sum and system (eta, W)
+//   C0-5 a conformation component's SBDF sum and system; three of them first
+//        form a component of H
+// About 300 FP64 instructions per coefficient pair and 64 cycles each make
+// the FP64 pipe the bound (0.2 ms at 128 x 97 x 64 were every SM equally
+// loaded); 256 blocks on 152 SMs put 2/1.7 of that on the busiest, and the
+// chains are paired per sub-partition (a warp's index mod 4) as evenly as
+// they go: V + C5, Q2 + C0, C1 + C2, C3 + C4.  Blocks turn the pairs by one
+// partition each, so that two of an SM do not load the same one.
+// Measured at 128 x 97 x 64: 0.61 -> 0.40 ms (one pass per recurrence, a
+// barrier between any two, 390 FP64 instructions); rows loaded one ahead while
+// the elimination's arithmetic runs (both rows at once spill at the 128
+// registers that two blocks per SM leave).
+// Per-mode scratch columns live in SS (workspace; L2-resident while the block
+// runs):
 enum {
-  S3_DCXY = 0, S3_DCYY, S3_DCYZ, S3_DV, S3_D2V,   // derivatives of the state
-  S3_HX, S3_HY, S3_HZ,                             // explicit momentum terms H
-  S3_Q1, S3_Q2,                                    // evolved q1, q2 (state)
-  S3_F1T, S3_F1, S3_F2,                            // forcings of q1, q2
-  S3_R,                                            // 8 SBDF sums (13..20)
-  S3_DVN = S3_R + 8,                               // D of the new v
-  S3_PHI, S3_ETA,                                  // solved phi, eta
-  kScr3                                            // 24 columns per mode
+  S3_HX = 0, S3_HY, S3_HZ,   // explicit momentum terms H
+  S3_P,                      // 6: the c components' eliminations
+  S3_PHI = S3_P + 6,         // phi
+  S3_ETA, S3_DVN,            // eta, D of the new v
+  kScr3
 };
 constexpr int kModesPerBlock = 16;
 
-__global__ void __launch_bounds__(256) k_spec3(GroupDev g, int mode) {
+// Named barriers: `n` threads of the block in all, those that only signal
+// (after their writes) and those that wait.
+__device__ __forceinline__ void bar_signal(int id, int n) {
+  __threadfence_block();
+  __syncwarp();
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_wait(int id, int n) {
+  __threadfence_block();
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
+// The lane's mode and its tables.
+struct Mode3 {
+  int N, p, md, o;
+  bool mean;
+  double kx, kz, k2;
+  size_t NK, col;
+};
+
+__device__ __forceinline__ LaneHist hist3(const GroupDev& g, const Mode3& m, int b, int slot, int q, double idt) {
+  LaneHist h;
+  h.o = m.o;
+  for (int j = 0; j < 4; ++j) h.ca[j] = -c_sa[m.o][j + 1] * idt;
+  auto at = [&](double2* base, int j) {
+    return base + ((((size_t)((slot - j) & 3)) * g.nb + b) * 8 + q) * m.NK + m.col;
+  };
+  h.E0 = at(g.Eh, 1); h.E1 = at(g.Eh, 2); h.E2 = at(g.Eh, 3);
+  h.dn = g.Nh - g.Eh;
+  return h;
+}
+
+// Elimination of a conformation component x with explicit term nn.
+template <bool FULL>
+__device__ __forceinline__ double2 chain3_c(const Mode3& m, const LaneHist& h, const double2* __restrict__ x,
+                                            const double2* __restrict__ nn, double2* __restrict__ E,
+                                            double2* __restrict__ Nn, double alpha, double2* __restrict__ P,
+                                            const double* inv, const double* F, const double* w, bool solve,
+                                            double2& rs) {
+  struct Row { LaneRow h; double2 x, nn; };
+  auto ld = [&](int n) {
+    Row r;
+    r.h = lane_hist_row<FULL>(h, n);
+    r.x = x[n];
+    r.nn = nn[n];
+    return r;
+  };
+  auto ev = [&](const Row& r, int n) {
+    E[n] = r.x;
+    Nn[n] = r.nn;
+    return lane_sbdf<FULL>(h, r.h, r.x, r.nn);
+  };
+  if (solve) return lane_qt_back<true>(m.N, m.p, alpha, ld, ev, P, inv, F, w, rs);
+  // no diffusion: P = R / alpha
+  const double ia = 1.0 / alpha;
+#pragma unroll 2
+  for (int n = m.p; n < m.N; n += 2) P[n] = cscl(ev(ld(n), n), ia);
+  return czero();
+}
+
+// Elimination of q1 (phi, or U of the mean mode): forcing
+// -D(i kx H_x + i kz H_z) - k^2 H_y (mean mode: H_x) on the way down.
+template <bool FULL>
+__device__ __forceinline__ double2 chain3_v(const Mode3& m, const LaneHist& h, const double2* __restrict__ Hx,
+                                            const double2* __restrict__ Hy, const double2* __restrict__ Hz,
+                                            const double2* __restrict__ E, double2* __restrict__ Nn, double alpha,
+                                            double2* __restrict__ P, const double* inv, const double* F,
+                                            const double* w) {
+  struct Row { LaneRow h; double2 x, hx, hz, hy; };
+  auto ld = [&](int n) {
+    Row r;
+    r.h = lane_hist_row<FULL>(h, n);
+    r.x = E[n];
+    const int k = m.mean ? n : min(n + 1, m.N - 1);
+    r.hx = Hx[k];
+    r.hz = Hz[k];
+    r.hy = Hy[n];
+    return r;
+  };
+  double2 acc = czero();
+  auto ev = [&](const Row& r, int n) {
+    const double2 s = cfma(m.kz, r.hz, cscl(r.hx, m.kx));
+    acc = cfma(n + 1 < m.N ? lane_i2d(2 * (n + 1)) : 0.0, s, acc);
+    const double2 d = lane_half2(acc, n == 0);
+    double2 f = make_double2(fma(-m.k2, r.hy.x, d.y), fma(-m.k2, r.hy.y, -d.x));
+    if (m.mean) f = r.hx;
+    Nn[n] = f;
+    return lane_sbdf<FULL>(h, r.h, r.x, f);
+  };
+  double2 rs;
+  return lane_qt_back<false>(m.N, m.p, alpha, ld, ev, P, inv, F, w, rs);
+}
+
+// Elimination of q2 = i kz u - i kx w with forcing i kz H_x - i kx H_z (mean
+// mode: w and H_z).
+template <bool FULL>
+__device__ __forceinline__ double2 chain3_q(const Mode3& m, const LaneHist& h, const double2* __restrict__ u,
+                                            const double2* __restrict__ w_, const double2* __restrict__ Hx,
+                                            const double2* __restrict__ Hz, double2* __restrict__ E,
+                                            double2* __restrict__ Nn, double alpha, double2* __restrict__ P,
+                                            const double* inv, const double* F, const double* w) {
+  struct Row { LaneRow h; double2 u, w, hx, hz; };
+  auto ld = [&](int n) {
+    Row r;
+    r.h = lane_hist_row<FULL>(h, n);
+    r.u = u[n];
+    r.w = w_[n];
+    r.hx = Hx[n];
+    r.hz = Hz[n];
+    return r;
+  };
+  auto ev = [&](const Row& r, int n) {
+    double2 x = mul_i(cfma(-m.kx, r.w, cscl(r.u, m.kz)));
+    double2 f = mul_i(cfma(-m.kx, r.hz, cscl(r.hx, m.kz)));
+    if (m.mean) { x = r.w; f = r.hz; }
+    E[n] = x;
+    Nn[n] = f;
+    return lane_sbdf<FULL>(h, r.h, x, f);
+  };
+  double2 rs;
+  return lane_qt_back<false>(m.N, m.p, alpha, ld, ev, P, inv, F, w, rs);
+}
+
+__global__ void __launch_bounds__(256, 2) k_spec3(const __grid_constant__ GroupDev g, int mode) {
   const int b = blockIdx.y;
   if (g.status[b]) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -509,21 +646,24 @@ __global__ void __launch_bounds__(256) k_spec3(GroupDev g, int mode) {
   const int mx = md / nz, mzi = md - mx * nz, hz = nz / 2;
   const bool nyq = (mzi == hz);
   const bool act = inb && !nyq;
-  const bool mean = (mx == 0 && mzi == 0);
   const MemberPrm pr = g.prm[b];
   const long long cnt = g.count[b];
   const int slot = (int)(cnt & 3);
   const int o = (cnt < 3) ? (int)cnt : 3;
   const int sz = (mzi < hz) ? mzi : mzi - nz;
-  const double kx = 2.0 * 3.14159265358979323846 * mx / pr.lx;
-  const double kz = 2.0 * 3.14159265358979323846 * sz / pr.lz;
-  const double k2 = kx * kx + kz * kz;
-  const size_t col = (size_t)md * N;
+  Mode3 m;
+  m.N = N; m.p = p; m.md = md; m.o = o;
+  m.mean = (mx == 0 && mzi == 0);
+  m.kx = 2.0 * 3.14159265358979323846 * mx / pr.lx;
+  m.kz = 2.0 * 3.14159265358979323846 * sz / pr.lz;
+  m.k2 = m.kx * m.kx + m.kz * m.kz;
+  m.NK = NK; m.col = (size_t)md * N;
+  const bool mean = m.mean;
+  const size_t col = m.col;
   double2* X = g.X + (size_t)b * 9 * NK + col;          // field f at X + f * NK
   const double2* NR = g.NR + (size_t)b * 9 * NK + col;
   double2* S = g.SS + (size_t)b * kScr3 * NK + col;     // scratch column a at S + a * NK
   auto SC = [&](int a) { return S + (size_t)a * NK; };
-  const double gam = pr.gam;
 
   // the dropped Nyquist slot stays zero
   if (warp == 0 && inb && nyq) {
@@ -540,176 +680,136 @@ __global__ void __launch_bounds__(256) k_spec3(GroupDev g, int mode) {
         for (int n = p; n < N; n += 2) R[f * NK + n] = czero();
     }
   }
-  // phase 1: derivatives D c_xy, D c_yy, D c_yz; D v, D^2 v
-  if (act) {
-    if (warp == 0) lane_cheb_deriv(X + 4 * NK, SC(S3_DCXY), N, p);
-    else if (warp == 1) lane_cheb_deriv(X + 6 * NK, SC(S3_DCYY), N, p);
-    else if (warp == 2) lane_cheb_deriv(X + 7 * NK, SC(S3_DCYZ), N, p);
-  }
-  if (warp == 3) {
-    const bool d = act && mode == 0 && !mean;
-    if (d) lane_cheb_deriv(X + NK, SC(S3_DV), N, p);
-    __syncwarp();
-    if (d) lane_cheb_deriv(SC(S3_DV), SC(S3_D2V), N, p);
-  }
-  __syncthreads();
-  // Element-wise phases split the lane's column over the eight warps: warp w
-  // takes elements [w c8, (w + 1) c8) of its lane's parity (n = p + 2 i), so
-  // every warp keeps loads in flight (one warp per column waited on each
-  // element in turn).
-  const int Lp = (N - p + 1) / 2;
-  const int c8 = (Lp + 7) / 8;
-  const int e0 = min(Lp, warp * c8), e1 = min(Lp, e0 + c8);
-  // phase 2: H (all three components), evolved q1, q2
-  if (act) {
-    const double2* __restrict__ Xc = X;
-    const double2* __restrict__ Sd = S;
-    double2* __restrict__ Sw = S;
-    const double fx = mean ? pr.forcing : 0.0;
-    for (int i = e0; i < e1; ++i) {
-      const int n = p + 2 * i;
-#pragma unroll
-      for (int t = 0; t < 3; ++t) {
-        // (div c)_i = i kx c_xi + D c_yi + i kz c_zi
-        const int cx = (t == 0) ? 3 : (t == 1) ? 4 : 5;     // c_xx, c_xy, c_xz
-        const int cz = (t == 0) ? 5 : (t == 1) ? 7 : 8;     // c_xz, c_yz, c_zz
-        const double2 dv = cadd(cscl(mul_i(Xc[(size_t)cx * NK + n]), kx),
-                                cadd(Sd[(size_t)(S3_DCXY + t) * NK + n],
-                                     cscl(mul_i(Xc[(size_t)cz * NK + n]), kz)));
-        double2 h = cfma(gam, dv, NR[(size_t)(6 + t) * NK + n]);
-        if (t == 0 && n == 0) h.x += fx;
-        Sw[(size_t)(S3_HX + t) * NK + n] = h;
-      }
-      if (mode == 0) {
-        Sw[(size_t)S3_Q1 * NK + n] = mean ? Xc[n] : cfma(-k2, Xc[NK + n], Sd[(size_t)S3_D2V * NK + n]);
-        Sw[(size_t)S3_Q2 * NK + n] =
-            mean ? Xc[2 * NK + n] : csub(cscl(mul_i(Xc[n]), kz), cscl(mul_i(Xc[2 * NK + n]), kx));
-      }
+  // the warp's chain: 0-5 a c component, 6 V, 7 Q2
+  const int part = (warp - (int)blockIdx.x - (int)blockIdx.x / 152) & 3;   // 152 SMs: block i + 152 joins block i
+  const int role = (warp < 4) ? (part == 0 ? 6 : part == 1 ? 7 : part == 2 ? 1 : 3)
+                              : (part == 0 ? 5 : part == 1 ? 0 : part == 2 ? 2 : 4);
+  // explicit momentum term t on component warp t + 1:
+  // (div c)_i = i kx c_xi + D c_yi + i kz c_zi
+  if (role >= 1 && role <= 3) {
+    const int t = role - 1;
+    const int cx = 3 + t;                               // c_xx, c_xy, c_xz
+    const int cy = (t == 0) ? 4 : 5 + t;                // c_xy, c_yy, c_yz
+    const int cz = (t == 0) ? 5 : 6 + t;                // c_xz, c_yz, c_zz
+    double2* H = (mode == 1) ? g.Rb + ((size_t)b * 4 + t) * NK + col : SC(S3_HX + t);
+    if (act) {
+      lane_div_h(N, p, X + cy * NK, X + cx * NK, X + cz * NK, NR + (size_t)(6 + t) * NK, pr.gam, pr.gam * m.kx,
+                 pr.gam * m.kz, H);
+      if (mean && t == 0 && p == 0) H[0].x += pr.forcing;
     }
   }
-  __syncthreads();
-  if (mode == 1) {   // explicit right-hand side only: H -> Rb
-    if (act && warp < 3) {
-      double2* R = g.Rb + (size_t)b * 4 * NK + col + (size_t)warp * NK;
-      const double2* H = SC(S3_HX + warp);
-      for (int n = p; n < N; n += 2) R[n] = H[n];
+  if (mode == 1) return;   // explicit right-hand side only: H in Rb
+  const double* w = g.wrow;
+  const double a0 = c_sa[o][0], idt = 1.0 / pr.dt;
+  const double* qt = g.qt + ((size_t)b * 4 + o) * 3 * 3 * NK + col;
+  auto T = [&](int sys, int k) { return qt + (size_t)(sys * 3 + k) * NK; };
+  auto G = [&](int sys) { return g.qtG[((((size_t)b * 4 + o) * 3 + sys) * 2 + p) * KZ + md]; };
+  auto cur = [&](double2* base, int q) { return base + (((size_t)slot * nb + b) * 8 + q) * NK + col; };
+  if (role < 6) {
+    if (role >= 1 && role <= 3) bar_signal(1, 160);   // H is there (the other end: V and Q2)
+    const double alpha = a0 / pr.dt + pr.kappa * m.k2;
+    const bool solve = pr.kappa != 0.0;
+    double2 U = czero(), rs = czero();
+    double2* P = SC(S3_P + role);
+    double2* x = X + (size_t)(3 + role) * NK;
+    if (act) {
+      const LaneHist h = hist3(g, m, b, slot, role, idt);
+      const double2* nn = NR + (size_t)role * NK;
+      U = (o == 3) ? chain3_c<true>(m, h, x, nn, cur(g.Eh, role), cur(g.Nh, role), alpha, P, T(0, 1), T(0, 2), w,
+                                    solve, rs)
+                   : chain3_c<false>(m, h, x, nn, cur(g.Eh, role), cur(g.Nh, role), alpha, P, T(0, 1), T(0, 2), w,
+                                     solve, rs);
     }
-    return;
-  }
-  // phase 3: forcings of q1 = -D(i kx H_x + i kz H_z) - k^2 H_y and of
-  // q2 = i kz H_x - i kx H_z (mean mode: H_x, H_z): the element-wise parts
-  // over all warps, the derivative on warp 0
-  {
-    const double2* __restrict__ Hx = SC(S3_HX);
-    const double2* __restrict__ Hy = SC(S3_HY);
-    const double2* __restrict__ Hz = SC(S3_HZ);
-    double2* __restrict__ t = SC(S3_F1T);
-    double2* __restrict__ f2 = SC(S3_F2);
-    if (act)
-      for (int i = e0; i < e1; ++i) {
-        const int n = p + 2 * i;
-        if (!mean) t[n] = cadd(cscl(mul_i(Hx[n]), kx), cscl(mul_i(Hz[n]), kz));
-        f2[n] = mean ? Hz[n] : csub(cscl(mul_i(Hx[n]), kz), cscl(mul_i(Hz[n]), kx));
-      }
-    __syncthreads();
-    if (warp == 0 && act && !mean) lane_cheb_deriv(SC(S3_F1T), SC(S3_F1), N, p);
-    __syncthreads();
-    double2* __restrict__ f = SC(S3_F1);
-    if (act)
-      for (int i = e0; i < e1; ++i) {
-        const int n = p + 2 * i;
-        f[n] = mean ? Hx[n] : csub(cscl(f[n], -1.0), cscl(Hy[n], k2));
-      }
-  }
-  __syncthreads();
-  // phase 4: history slot and SBDF sums, warp s for evolved quantity s
-  if (act) {
-    const int s2 = warp;
-    const double2* x = (s2 < 6) ? X + (size_t)(3 + s2) * NK : SC(S3_Q1 + (s2 - 6));
-    const double2* nn = (s2 < 6) ? NR + (size_t)s2 * NK : SC(S3_F1 + (s2 - 6));
-    double2* E = g.Eh + ((size_t)slot * nb + b) * 8 * NK + (size_t)s2 * NK + col;
-    double2* R = SC(S3_R + s2);
-    const double2* Eo[3];
-    for (int jj = 1; jj <= 3; ++jj) {
-      const size_t sl = (size_t)((slot - jj) & 3);
-      Eo[jj - 1] = g.Eh + (sl * nb + b) * 8 * NK + (size_t)s2 * NK + col;
-    }
-    // FP64 history in every form: in a mixed group the mean mode would need
-    // it in FP64 (its explicit terms carry the 2/Re forcing and the
-    // 10^4-sized stretching), and its lanes share warps with the other
-    // modes, so an FP32 history elsewhere would diverge the warps of the
-    // block holding the mean mode, which sets the launch's time (one wave
-    // at 128 x 97 x 64: measured 0.60 -> 0.66 ms)
-    double2* Nn = g.Nh + ((size_t)slot * nb + b) * 8 * NK + (size_t)s2 * NK + col;
-    const double2* No[3];
-    for (int jj = 1; jj <= 3; ++jj) {
-      const size_t sl = (size_t)((slot - jj) & 3);
-      No[jj - 1] = g.Nh + (sl * nb + b) * 8 * NK + (size_t)s2 * NK + col;
-    }
-    lane_sbdf_any(o, N, p, 1.0 / pr.dt, x, nn, E, Nn, Eo, No, R);
-  }
-  __syncthreads();
-  // phase 5: tau solves; warps 0-5 the c components, 6 q1, 7 q2
-  if (act) {
-    const double* w1 = g.wrow;
-    const double* w2 = g.wrow + N;
-    const double* w3 = g.wrow + 2 * N;
-    const double a0 = c_sa[o][0];
-    const double* qt = g.qt + ((size_t)b * 4 + o) * 3 * 3 * NK + col;
-    auto T = [&](int sys, int k) { return qt + (size_t)(sys * 3 + k) * NK; };
-    auto G = [&](int sys) { return g.qtG[((((size_t)b * 4 + o) * 3 + sys) * 2 + p) * KZ + md]; };
-    if (warp < 6) {
-      const double2* R = SC(S3_R + warp);
-      double2* out = X + (size_t)(3 + warp) * NK;
-      const double alpha = a0 / pr.dt + pr.kappa * k2;
-      if (pr.kappa == 0.0) {
-        const double ia = 1.0 / alpha;
-        for (int n = p; n < N; n += 2) out[n] = cscl(R[n], ia);
+    bar_wait(2, 192);   // H has read the old c (the six component warps)
+    if (act) {
+      if (solve) {
+        const double2 wall = cscl(rs, pr.dt / a0);
+        lane_qt_fwd(N, p, cscl(csub(wall, U), G(0)), wall, P, x, T(0, 0), [](int, double2) {});
       } else {
-        lane_qt_solve(N, p, alpha, R, out, T(0, 0), T(0, 1), T(0, 2), G(0), w1, w2, w3,
-                      pr.dt / a0, 1.0);
+#pragma unroll 4
+        for (int n = p; n < N; n += 2) x[n] = P[n];
       }
-    } else if (warp == 6) {
-      double2* R1 = SC(S3_R + 6);
+    }
+  } else if (role == 6) {
+    double2* E = cur(g.Eh, 6);
+    double2* v = X + NK;
+    if (act) {
       if (mean) {
-        lane_qt_solve(N, p, a0 / pr.dt, R1, X, T(1, 0), T(1, 1), T(1, 2), G(1), w1, w2, w3, 0.0, 1.0);
-        for (int n = p; n < N; n += 2) X[NK + n] = czero();
+#pragma unroll 4
+        for (int n = p; n < N; n += 2) E[n] = X[n];
       } else {
-        double2* v = X + NK;
-        double2* phi = SC(S3_PHI);
-        lane_qt_solve(N, p, a0 / pr.dt + pr.nu * k2, R1, phi, T(1, 0), T(1, 1), T(1, 2), G(1), w1,
-                      w2, w3, 0.0, 1.0);
-        lane_qt_solve(N, p, k2, phi, v, T(2, 0), T(2, 1), T(2, 2), G(2), w1, w2, w3, 0.0, -1.0);
-        double2 sacc = czero();
-        for (int n = p; n < N; n += 2) sacc = cfma((double)n * n, v[n], sacc);
-        const double* vh = g.vh + ((size_t)b * 4 + o) * NK + col;
-        const double2 coef = cscl(sacc, -g.vhS[(((size_t)b * 4 + o) * 2 + p) * KZ + md]);
-        for (int n = p; n < N; n += 2)
-          v[n] = make_double2(fma(coef.x, vh[n], v[n].x), fma(coef.y, vh[n], v[n].y));
+        lane_lap(N, p, v, m.k2, E);
       }
-    } else {
-      double2* R2 = SC(S3_R + 7);
-      const double alpha = mean ? a0 / pr.dt : a0 / pr.dt + pr.nu * k2;
-      double2* out = mean ? X + 2 * NK : SC(S3_ETA);   // W, or eta
-      lane_qt_solve(N, p, alpha, R2, out, T(1, 0), T(1, 1), T(1, 2), G(1), w1, w2, w3, 0.0, 1.0);
+    }
+    bar_wait(1, 160);
+    if (act) {
+      const LaneHist h = hist3(g, m, b, slot, 6, idt);
+      double2* phi = SC(S3_PHI);
+      const double alpha = mean ? a0 / pr.dt : a0 / pr.dt + pr.nu * m.k2;
+      const double2 U = (o == 3) ? chain3_v<true>(m, h, SC(S3_HX), SC(S3_HY), SC(S3_HZ), E, cur(g.Nh, 6), alpha, phi,
+                                                  T(1, 1), T(1, 2), w)
+                                 : chain3_v<false>(m, h, SC(S3_HX), SC(S3_HY), SC(S3_HZ), E, cur(g.Nh, 6), alpha, phi,
+                                                   T(1, 1), T(1, 2), w);
+      lane_qt_fwd(N, p, cscl(U, -G(1)), czero(), phi, mean ? X : phi, T(1, 0), [](int, double2) {});
+      if (mean) {
+        for (int n = p; n < N; n += 2) v[n] = czero();
+      } else {
+        // (D^2 - k^2) v = phi: the solve's right-hand side is -phi
+        double2 rs, sacc = czero();
+        const double2 U2 = lane_qt_back<false>(
+            N, p, m.k2, [&](int n) { return phi[n]; },
+            [&](double2 r, int) { return cneg_bits(r); }, v, T(2, 1), T(2, 2), w, rs);
+        lane_qt_fwd(N, p, cscl(U2, -G(2)), czero(), v, v, T(2, 0),
+                    [&](int n, double2 a) { sacc = cfma(lane_i2d(n * n), a, sacc); });
+        // influence correction and D v, top down
+        const double* __restrict__ vh = g.vh + ((size_t)b * 4 + o) * NK + col;
+        double2* __restrict__ dv = SC(S3_DVN);
+        double2* __restrict__ vr = v;
+        const double2 coef = cscl(sacc, -g.vhS[(((size_t)b * 4 + o) * 2 + p) * KZ + md]);
+        const int nl = ((N - 1 - p) & ~1) + p;
+        double2 acc = czero();
+        if (nl != N - 1) dv[N - 1] = czero();
+#pragma unroll 4
+        for (int n = nl; n >= p; n -= 2) {
+          const double f = vh[n];
+          const double2 a = vr[n];
+          const double2 vn = make_double2(fma(coef.x, f, a.x), fma(coef.y, f, a.y));
+          vr[n] = vn;
+          acc = cfma(lane_i2d(2 * n), vn, acc);
+          if (n > 0) dv[n - 1] = lane_half2(acc, n == 1);
+        }
+      }
+    }
+  } else {
+    bar_wait(1, 160);
+    if (act) {
+      const LaneHist h = hist3(g, m, b, slot, 7, idt);
+      double2* eta = SC(S3_ETA);
+      const double alpha = mean ? a0 / pr.dt : a0 / pr.dt + pr.nu * m.k2;
+      const double2 U = (o == 3) ? chain3_q<true>(m, h, X, X + 2 * NK, SC(S3_HX), SC(S3_HZ), cur(g.Eh, 7),
+                                                  cur(g.Nh, 7), alpha, eta, T(1, 1), T(1, 2), w)
+                                 : chain3_q<false>(m, h, X, X + 2 * NK, SC(S3_HX), SC(S3_HZ), cur(g.Eh, 7),
+                                                   cur(g.Nh, 7), alpha, eta, T(1, 1), T(1, 2), w);
+      lane_qt_fwd(N, p, cscl(U, -G(1)), czero(), eta, mean ? X + 2 * NK : eta, T(1, 0), [](int, double2) {});
     }
   }
   __syncthreads();
-  // phase 6: u, w from D v and eta (k != 0): the derivative on warp 0, the
-  // element-wise part over all warps
-  const bool dvw = act && !mean;
-  if (warp == 0 && dvw) lane_cheb_deriv(X + NK, SC(S3_DVN), N, p);
-  __syncthreads();
-  if (dvw) {
+  // u, w from D v and eta (k != 0), warp w on elements [w c8, (w + 1) c8) of
+  // its lane's parity
+  if (act && !mean) {
+    const int Lp = (N - p + 1) / 2, c8 = (Lp + 7) / 8;
+    const int e0 = min(Lp, warp * c8), e1 = min(Lp, e0 + c8);
     const double2* __restrict__ dv = SC(S3_DVN);
     const double2* __restrict__ et = SC(S3_ETA);
     double2* __restrict__ u = X;
-    double2* __restrict__ w = X + 2 * NK;
-    const double ik2 = 1.0 / k2;
+    double2* __restrict__ wv = X + 2 * NK;
+    const double ax = m.kx / m.k2, az = m.kz / m.k2;
+#pragma unroll 4
     for (int i = e0; i < e1; ++i) {
       const int n = p + 2 * i;
-      u[n] = cscl(mul_i(csub(cscl(dv[n], kx), cscl(et[n], kz))), ik2);
-      w[n] = cscl(mul_i(cadd(cscl(dv[n], kz), cscl(et[n], kx))), ik2);
+      const double2 d = dv[n], e = et[n];
+      u[n] = mul_i(cfma(-az, e, cscl(d, ax)));
+      wv[n] = mul_i(cfma(ax, e, cscl(d, az)));
     }
   }
 }
