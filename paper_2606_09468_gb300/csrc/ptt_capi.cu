@@ -835,6 +835,8 @@ void member_prm(const ptt_params& p, MemberPrm& q) {
   q.u_max = p.blowup_u_max > 0 ? p.blowup_u_max : 1e300;
   q.kx1 = 2.0 * kPi / q.lx;
   q.kz1 = 2.0 * kPi / q.lz;
+  q.idt = 1.0 / p.dt;
+  for (int o = 0; o < 4; ++o) { q.a0dt[o] = kSA0[o] / p.dt; q.dta0[o] = p.dt / kSA0[o]; }
   q.kx1f = (float)q.kx1;
   q.kz1f = (float)q.kz1;
   q.epsf = (float)q.eps;

@@ -436,6 +436,20 @@ __device__ __forceinline__ double2 warp_allsum2(double2 v) {
   return v;
 }
 
+// 0 <= k < 2^23 as a double, without the FP64 pipe and without branches.
+__device__ __forceinline__ double lane_i2d(int k) {
+  const unsigned b = __float_as_uint(__uint_as_float(0x4B000000u | (unsigned)k) - 8388608.f);
+  return __hiloint2double((int)((b >> 3) + (k ? 0x38000000u : 0u)), (int)(b << 29));
+}
+template <typename T> __device__ __forceinline__ T int_as(int k);
+template <> __device__ __forceinline__ double int_as<double>(int k) { return lane_i2d(k); }
+template <> __device__ __forceinline__ float int_as<float>(int k) { return (float)k; }
+// Mean over y of T_n (n even), 2/(1 - n^2): four times the tau rows' table
+// w2_n = 1/(2 (n^2 - 1)) with its sign turned (w holds w1, w2, w3 from n = 2).
+__device__ __forceinline__ double cheb_mean_weight(const double* w, int N, int n) {
+  return n == 0 ? 2.0 : -4.0 * w[N + n];
+}
+
 // Chebyshev derivative by one warp: out_n = (2/c_n) sum_{p > n, p + n odd} p a_p
 // (c_0 = 2), as two same-parity suffix sums T(k) = sum_{p >= k, p = k mod 2} p a_p
 // with out_{k-1} = (2/c_{k-1}) T(k).  `out` must not alias `a`.
@@ -451,7 +465,7 @@ __device__ void warp_cheb_deriv_par(const C2* a, C2* out, int N, int par) {
   C2 acc = zero2<C2>();
   for (int i = i1 - 1; i >= i0; --i) {
     const int k = par + 2 * i;
-    acc = cfma((T)(2 * k), a[k], acc);
+    acc = cfma(int_as<T>(2 * k), a[k], acc);
     if (k >= 1) out[k - 1] = acc;
   }
   C2 inc = acc;
@@ -487,7 +501,8 @@ __device__ __forceinline__ double2 cneg_bits(double2 v) {
 // a_i = P_i + Q_i a_{i-1} are affine recurrences, evaluated as warp scans of
 // affine maps; the boundary sums are warp reductions.  `out` may alias R.
 // CH >= the rows per lane, ceil((L - 1)/32) (register arrays of that size).
-template <int CH>
+// WALL: the wall row has a right-hand side (bcfac sum R), else it is 0.
+template <int CH, bool WALL>
 __device__ void warp_qt_solve(int N, int p, double alpha, const double2* R, double2* out,
                               const double* Q, const double* inv, const double* F, double G,
                               const double* w1, const double* w2, const double* w3,
@@ -507,23 +522,24 @@ __device__ void warp_qt_solve(int N, int p, double alpha, const double2* R, doub
       const int n = p + 2 * i;
       const double2 Rm2 = R[n - 2];
       const double2 R0 = R[n];
-      const double cc = (n == 2) ? 2.0 : 1.0;
-      double2 r = cscl(Rm2, -cc * w1[n]);
+      const double w1n = w1[n], iv = inv[n];   // w1 counts twice at n = 2
+      double2 r = cscl(Rm2, -__hiloint2double(__double2hiint(w1n) + (n == 2 ? 0x100000 : 0), __double2loint(w1n)));
       if (n <= N - 3) r = cfma(w2[n], R0, r);
       double un = 0.0;
       if (n <= N - 5) {
-        r = cfma(-w3[n], R[n + 2], r);
-        un = -alpha * w3[n];
+        const double w3n = w3[n];
+        r = cfma(-w3n, R[n + 2], r);
+        un = alpha * w3n;
       }
-      al[t] = cscl(r, inv[n]);
-      be[t] = -un * inv[n];
-      rs = cadd(rs, R0);
+      al[t] = cscl(r, iv);
+      be[t] = un * iv;
+      if (WALL) rs = cadd(rs, R0);
     } else {
       al[t] = czero();
       be[t] = 1.0;
     }
   }
-  if (lane == 0) rs = cadd(rs, R[p]);
+  if (WALL && lane == 0) rs = cadd(rs, R[p]);
   __syncwarp();
   // backward: chunk map P_{i0} = A + B P_{i1}
   double2 A = czero();
@@ -559,9 +575,8 @@ __device__ void warp_qt_solve(int N, int p, double alpha, const double2* R, doub
       U = cfma(F[n], P, U);
     }
   }
-  U = warp_allsum2(U);
-  rs = warp_allsum2(rs);
-  const double2 a0 = cscl(csub(cscl(rs, bcfac), U), G);
+  const double2 a0 = cscl(warp_allsum2(WALL ? make_double2(fma(bcfac, rs.x, -U.x), fma(bcfac, rs.y, -U.y))
+                                            : cneg_bits(U)), G);
   // forward: chunk map a_{i1-1} = C + D a_{i0-1}
   double2 Cc = czero();
   double Dd = 1.0;
@@ -592,7 +607,9 @@ __device__ void warp_qt_solve(int N, int p, double alpha, const double2* R, doub
   double ED = __shfl_up_sync(kFull, ID, 1);
   if (lane == 0) { EC = czero(); ED = 1.0; }
   double2 av = cfma(ED, a0, EC);
-  double2 part = (lane == 0) ? a0 : czero();  // sum of a_{p+2i}, i < L-1
+  const int nl = p + 2 * (L - 1);
+  const bool top = L > 1 && fabs(Q[nl]) > kTopFromWall;
+  double2 part = (lane == 0) ? a0 : czero();  // sum of a_{p+2i}, i < L-1, where top
   __syncwarp();
 #pragma unroll
   for (int t = 0; t < CH; ++t) {
@@ -600,7 +617,7 @@ __device__ void warp_qt_solve(int N, int p, double alpha, const double2* R, doub
     if (t < c && i < i1) {
       av = cfma(Qv[t], av, Pv[t]);
       out[p + 2 * i] = av;
-      if (i < L - 1) part = cadd(part, av);
+      if (top && i < L - 1) part = cadd(part, av);
     }
   }
   if (lane == 0) out[p] = a0;
@@ -610,10 +627,10 @@ __device__ void warp_qt_solve(int N, int p, double alpha, const double2* R, doub
   // substitution forms a_top = P + Q a_{top-2} with |Q| ~ alpha/(4 n^2 kappa)
   // and amplifies the rounding of a_{top-2}; the wall row of the same system
   // gives a_top = g - sum of the others with rounding of the sum only.
-  const int nl = p + 2 * (L - 1);
-  if (L > 1 && fabs(Q[nl]) > kTopFromWall) {
+  if (top) {
+    if (WALL) part = make_double2(fma(-bcfac, rs.x, part.x), fma(-bcfac, rs.y, part.y));
     part = warp_allsum2(part);
-    if (lane == 0) out[nl] = csub(cscl(rs, bcfac), part);
+    if (lane == 0) out[nl] = cneg_bits(part);
     __syncwarp();
   }
   // the solve above is of (alpha - beta D^2) a = R; the system's right-hand
@@ -633,8 +650,7 @@ __device__ void warp_qt_solve(int N, int p, double alpha, const double2* R, doub
 // (the loads of the next row are issued before the current row's arithmetic),
 // and what needs no FP64 instruction has none.
 
-// 0 <= k < 2^24 as a double, x / 2 where z holds: integer instructions.
-__device__ __forceinline__ double lane_i2d(int k) { return f64_from_f32((float)k); }
+// x / 2 where z holds, by integer instructions.
 __device__ __forceinline__ double lane_half(double x, bool z) {
   const int h = __double2hiint(x);
   const bool scale = z && (((unsigned)h >> 20) & 0x7FFu) - 2u < 2045u;   // normal, result normal

@@ -42,9 +42,11 @@ struct MemberPrm {
   double lx, lz, re, wi, beta, eps, kappa, dt;
   double inv_wi, gam, nu, forcing;  // 1/Wi, (1-beta)/(Re Wi), beta/Re, 2/Re
   double trc_max, u_max;
-  // 2 pi / Lx, 2 pi / Lz and their FP32 roundings, computed on the host: a
-  // division per thread would cost the FP32 kernels tens of FP64 operations
-  double kx1, kz1;
+  // 2 pi / Lx, 2 pi / Lz and their FP32 roundings, 1/dt and, per SBDF order,
+  // a_0/dt and dt/a_0, computed on the host: a division per thread costs a
+  // kernel tens of FP64 instructions of 64 cycles each (the ones of the 2D
+  // per-mode stage were a quarter of its FP64 work)
+  double kx1, kz1, idt, a0dt[4], dta0[4];
   float kx1f, kz1f;
   float epsf, inv_wif;              // FP32 roundings of eps, 1/Wi
 };

@@ -299,6 +299,13 @@ __global__ void __launch_bounds__(kFxThreads, 4) k_xfused_fx_multi(const GroupDe
 // unbounded; CH = 2 and 4 take three (80 registers, a few spilled words,
 // shared memory for three blocks up to ny = 257), CH = 8 two (its register
 // arrays would spill heavily at 80).
+// Bound by the FP64 pipe (68 % busy).  No division per warp (the host's
+// constants; 1/k by one warp), no small integer through a conversion, powers of
+// two by exponent, one tree per boundary sum: the 27-run sweep 0.92 -> 0.79 ms
+// per step, the 64-run ensemble 4.49 -> 2.77 ms (stage alone), 64 x 65 alone
+// 39 -> 33 us.  Recurrences of one instruction per row with a lane per real
+// recurrence halve the FP64 work again but were slower (1.01 ms, 40 us): one
+// warp's chain of rows is then all there is to wait for.
 template <int CH>
 __device__ __forceinline__ void spec_block(const GroupDev& g, int mode, Blk bk) {
   const int b = bk.y;
@@ -310,8 +317,8 @@ __device__ __forceinline__ void spec_block(const GroupDev& g, int mode, Blk bk) 
   const long long cnt = g.count[b];
   const int slot = (int)(cnt & 3);
   const int o = (cnt < 3) ? (int)cnt : 3;
-  const double km = 2.0 * 3.14159265358979323846 * m / pr.lx;
-  const double km2 = km * km;
+  const double km = pr.kx1 * m;
+  const double km2 = km * km, gk = pr.gam * km;
   extern __shared__ double2 sm[];
   double2* sc0 = sm;            // c_xx  -> new c_xx
   double2* sc1 = sm + N;        // c_xy  -> new c_xy
@@ -326,6 +333,8 @@ __device__ __forceinline__ void spec_block(const GroupDev& g, int mode, Blk bk) 
   const double2* X = g.X + (size_t)b * 5 * NK + (size_t)m * N;
   const double2* NR = g.NR + (size_t)b * 5 * NK + (size_t)m * N;
   const int tid = threadIdx.x, nt = blockDim.x;
+  __shared__ double s_ik;
+  if (tid == 224) s_ik = 1.0 / km;   // one division, by the last warp; used at the end
   for (int i = tid; i < N; i += nt) {
     sc0[i] = X[2 * NK + i];
     sc1[i] = X[3 * NK + i];
@@ -359,8 +368,10 @@ __device__ __forceinline__ void spec_block(const GroupDev& g, int mode, Blk bk) 
   }
   __syncthreads();
   for (int n = tid; n < N; n += nt) {
-    double2 hx = cadd(shx[n], cscl(cadd(cscl(mul_i(sc0[n]), km), sR[n]), pr.gam));
-    const double2 hy = cadd(shy[n], cscl(cadd(cscl(mul_i(sc1[n]), km), sR[N + n]), pr.gam));
+    const double2 c0 = sc0[n], c1 = sc1[n];
+    double2 hx = cfma(pr.gam, sR[n], shx[n]), hy = cfma(pr.gam, sR[N + n], shy[n]);
+    hx = make_double2(fma(-gk, c0.y, hx.x), fma(gk, c0.x, hx.y));
+    hy = make_double2(fma(-gk, c1.y, hy.x), fma(gk, c1.x, hy.y));
     if (m == 0 && n == 0) hx.x += pr.forcing;
     shx[n] = hx;
     shy[n] = hy;
@@ -378,14 +389,16 @@ __device__ __forceinline__ void spec_block(const GroupDev& g, int mode, Blk bk) 
   // forcing of q: m >= 1: -D(i k H_x) - k^2 H_y; m = 0: H_x
   if (m != 0 && tid < 64) warp_cheb_deriv_par(shx, sR, N, tid >> 5);
   __syncthreads();
-  for (int n = tid; n < N; n += nt)
-    snq[n] = (m == 0) ? shx[n] : csub(cscl(mul_i(sR[n]), -km), cscl(shy[n], km2));
+  for (int n = tid; n < N; n += nt) {
+    const double2 d = sR[n], h = shy[n];
+    snq[n] = (m == 0) ? shx[n] : make_double2(fma(km, d.y, -(km2 * h.x)), fma(-km, d.x, -(km2 * h.y)));
+  }
   __syncthreads();
   // history slot and SBDF sums
   if (g.f32 && m != 0) {   // mixed groups: the explicit-term history and its sum in FP32
     double2* E = g.Eh + ((size_t)slot * nb + b) * 4 * NK + (size_t)m * N;
     float2* Nf = reinterpret_cast<float2*>(g.Nh + ((size_t)slot * nb + b) * 4 * NK) + (size_t)m * N;
-    const double idt = 1.0 / pr.dt;
+    const double idt = pr.idt;
     for (int i = tid; i < N; i += nt) {
       const double2 x[4] = {sc0[i], sc1[i], sc2[i], sq[i]};
       const double2 nn[4] = {NR[i], NR[NK + i], NR[2 * NK + i], snq[i]};
@@ -421,7 +434,7 @@ __device__ __forceinline__ void spec_block(const GroupDev& g, int mode, Blk bk) 
     };
     double2* E = g.Eh + ((size_t)slot * nb + b) * 4 * NK + (size_t)m * N;
     double2* Nn = nd((size_t)slot);
-    const double idt = 1.0 / pr.dt;
+    const double idt = pr.idt;
     for (int i = tid; i < N; i += nt) {
       const double2 x[4] = {sc0[i], sc1[i], sc2[i], sq[i]};
       const double2 nn[4] = {NR[i], NR[NK + i], NR[2 * NK + i], snq[i]};
@@ -445,7 +458,7 @@ __device__ __forceinline__ void spec_block(const GroupDev& g, int mode, Blk bk) 
   const double* w1 = g.wrow;
   const double* w2 = g.wrow + N;
   const double* w3 = g.wrow + 2 * N;
-  const double a0 = c_sa[o][0];
+  const double a0dt = g.prm[b].a0dt[o];
   {  // eight (system, parity) tau solves, one warp each
     const int t = tid >> 5;
     const int sys = t >> 1, p = t & 1;
@@ -457,25 +470,23 @@ __device__ __forceinline__ void spec_block(const GroupDev& g, int mode, Blk bk) 
     if (sys < 3) {
       double2* out = sm + (size_t)sys * N;  // sc0, sc1, sc2
       const double2* R = sR + (size_t)sys * N;
-      const double alpha = a0 / pr.dt + pr.kappa * km2;
+      const double alpha = fma(pr.kappa, km2, a0dt);
       if (pr.kappa == 0.0) {
         const double ia = 1.0 / alpha;
         for (int n = p + 2 * lane; n < N; n += 64) out[n] = cscl(R[n], ia);
       } else {
-        warp_qt_solve<CH>(N, p, alpha, R, out, T0, T0 + N, T0 + 2 * N, G(0), w1, w2, w3, pr.dt / a0,
-                      1.0);
+        warp_qt_solve<CH, true>(N, p, alpha, R, out, T0, T0 + N, T0 + 2 * N, G(0), w1, w2, w3, g.prm[b].dta0[o], 1.0);
       }
     } else if (m == 0) {
-      warp_qt_solve<CH>(N, p, a0 / pr.dt, sR + 3 * N, shy, T1, T1 + N, T1 + 2 * N, G(1), w1, w2, w3,
-                    0.0, 1.0);
+      warp_qt_solve<CH, false>(N, p, a0dt, sR + 3 * N, shy, T1, T1 + N, T1 + 2 * N, G(1), w1, w2, w3, 0.0, 1.0);
       for (int n = p + 2 * lane; n < N; n += 64) sv[n] = czero();
     } else {
       double2* Rv = sR + 3 * N;
-      warp_qt_solve<CH>(N, p, a0 / pr.dt + pr.nu * km2, Rv, Rv, T1, T1 + N, T1 + 2 * N, G(1), w1, w2,
-                    w3, 0.0, 1.0);
-      warp_qt_solve<CH>(N, p, km2, Rv, sv, T2, T2 + N, T2 + 2 * N, G(2), w1, w2, w3, 0.0, -1.0);
+      warp_qt_solve<CH, false>(N, p, fma(pr.nu, km2, a0dt), Rv, Rv, T1, T1 + N, T1 + 2 * N, G(1), w1, w2, w3, 0.0,
+                               1.0);
+      warp_qt_solve<CH, false>(N, p, km2, Rv, sv, T2, T2 + N, T2 + 2 * N, G(2), w1, w2, w3, 0.0, -1.0);
       double2 sacc = czero();
-      for (int n = p + 2 * lane; n < N; n += 64) sacc = cfma((double)n * n, sv[n], sacc);
+      for (int n = p + 2 * lane; n < N; n += 64) sacc = cfma(lane_i2d(n * n), sv[n], sacc);
       sacc = warp_allsum2(sacc);
       const double* vh = tb + 9 * N;
       const double2 coef = cscl(sacc, -g.vhS[(((size_t)b * 4 + o) * 2 + p) * K + m]);
@@ -488,7 +499,7 @@ __device__ __forceinline__ void spec_block(const GroupDev& g, int mode, Blk bk) 
   if (m != 0) {
     if (tid < 64) warp_cheb_deriv_par(sv, sR, N, tid >> 5);
     __syncthreads();
-    const double ik = 1.0 / km;
+    const double ik = s_ik;
     for (int n = tid; n < N; n += nt) shy[n] = cscl(mul_i(sR[n]), ik);
     __syncthreads();
   }
@@ -736,11 +747,11 @@ __device__ __forceinline__ void diag_final_block(const GroupDev& g, Blk bk) {
   // <Tr c> = 1/2 int (c_xx + c_yy)_0 dy + 1, int T_n = 2/(1-n^2), n even
   double mt = 0.0;
   for (int n = threadIdx.x; n < N; n += blockDim.x)
-    if ((n & 1) == 0) mt += (X[2 * NK + n].x + X[4 * NK + n].x) * (2.0 / (1.0 - (double)n * n));
+    if ((n & 1) == 0) mt += (X[2 * NK + n].x + X[4 * NK + n].x) * cheb_mean_weight(g.wrow, N, n);
   mt = block_sum(mt, sh);
   // mid-plane lines from the per-mode sums: (Tr c, u') (v, du/dx) (dv/dx, du/dy)
   fxc* A = reinterpret_cast<fxc*>(smraw);          // 3 lines of nx
-  const double kfac = 2.0 * 3.14159265358979323846 / pr.lx;
+  const double kfac = pr.kx1;
   const double2* DM = g.DM + (size_t)b * 4 * K;
   if (threadIdx.x < 96) {   // a warp per line
     const int l = threadIdx.x >> 5;

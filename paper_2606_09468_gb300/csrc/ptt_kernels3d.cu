@@ -654,8 +654,8 @@ __global__ void __launch_bounds__(256, 2) k_spec3(const __grid_constant__ GroupD
   Mode3 m;
   m.N = N; m.p = p; m.md = md; m.o = o;
   m.mean = (mx == 0 && mzi == 0);
-  m.kx = 2.0 * 3.14159265358979323846 * mx / pr.lx;
-  m.kz = 2.0 * 3.14159265358979323846 * sz / pr.lz;
+  m.kx = pr.kx1 * mx;
+  m.kz = pr.kz1 * sz;
   m.k2 = m.kx * m.kx + m.kz * m.kz;
   m.NK = NK; m.col = (size_t)md * N;
   const bool mean = m.mean;
@@ -680,6 +680,7 @@ __global__ void __launch_bounds__(256, 2) k_spec3(const __grid_constant__ GroupD
         for (int n = p; n < N; n += 2) R[f * NK + n] = czero();
     }
   }
+  __shared__ double s_ik2[32];   // 1/k^2 of the lanes, by V
   // the warp's chain: 0-5 a c component, 6 V, 7 Q2
   const int part = (warp - (int)blockIdx.x - (int)blockIdx.x / 152) & 3;   // 152 SMs: block i + 152 joins block i
   const int role = (warp < 4) ? (part == 0 ? 6 : part == 1 ? 7 : part == 2 ? 1 : 3)
@@ -700,14 +701,14 @@ __global__ void __launch_bounds__(256, 2) k_spec3(const __grid_constant__ GroupD
   }
   if (mode == 1) return;   // explicit right-hand side only: H in Rb
   const double* w = g.wrow;
-  const double a0 = c_sa[o][0], idt = 1.0 / pr.dt;
+  const double a0dt = g.prm[b].a0dt[o], idt = pr.idt;
   const double* qt = g.qt + ((size_t)b * 4 + o) * 3 * 3 * NK + col;
   auto T = [&](int sys, int k) { return qt + (size_t)(sys * 3 + k) * NK; };
   auto G = [&](int sys) { return g.qtG[((((size_t)b * 4 + o) * 3 + sys) * 2 + p) * KZ + md]; };
   auto cur = [&](double2* base, int q) { return base + (((size_t)slot * nb + b) * 8 + q) * NK + col; };
   if (role < 6) {
     if (role >= 1 && role <= 3) bar_signal(1, 160);   // H is there (the other end: V and Q2)
-    const double alpha = a0 / pr.dt + pr.kappa * m.k2;
+    const double alpha = fma(pr.kappa, m.k2, a0dt);
     const bool solve = pr.kappa != 0.0;
     double2 U = czero(), rs = czero();
     double2* P = SC(S3_P + role);
@@ -723,7 +724,7 @@ __global__ void __launch_bounds__(256, 2) k_spec3(const __grid_constant__ GroupD
     bar_wait(2, 192);   // H has read the old c (the six component warps)
     if (act) {
       if (solve) {
-        const double2 wall = cscl(rs, pr.dt / a0);
+        const double2 wall = cscl(rs, g.prm[b].dta0[o]);
         lane_qt_fwd(N, p, cscl(csub(wall, U), G(0)), wall, P, x, T(0, 0), [](int, double2) {});
       } else {
 #pragma unroll 4
@@ -741,11 +742,12 @@ __global__ void __launch_bounds__(256, 2) k_spec3(const __grid_constant__ GroupD
         lane_lap(N, p, v, m.k2, E);
       }
     }
+    s_ik2[lane] = mean ? 0.0 : 1.0 / m.k2;
     bar_wait(1, 160);
     if (act) {
       const LaneHist h = hist3(g, m, b, slot, 6, idt);
       double2* phi = SC(S3_PHI);
-      const double alpha = mean ? a0 / pr.dt : a0 / pr.dt + pr.nu * m.k2;
+      const double alpha = mean ? a0dt : fma(pr.nu, m.k2, a0dt);
       const double2 U = (o == 3) ? chain3_v<true>(m, h, SC(S3_HX), SC(S3_HY), SC(S3_HZ), E, cur(g.Nh, 6), alpha, phi,
                                                   T(1, 1), T(1, 2), w)
                                  : chain3_v<false>(m, h, SC(S3_HX), SC(S3_HY), SC(S3_HZ), E, cur(g.Nh, 6), alpha, phi,
@@ -785,7 +787,7 @@ __global__ void __launch_bounds__(256, 2) k_spec3(const __grid_constant__ GroupD
     if (act) {
       const LaneHist h = hist3(g, m, b, slot, 7, idt);
       double2* eta = SC(S3_ETA);
-      const double alpha = mean ? a0 / pr.dt : a0 / pr.dt + pr.nu * m.k2;
+      const double alpha = mean ? a0dt : fma(pr.nu, m.k2, a0dt);
       const double2 U = (o == 3) ? chain3_q<true>(m, h, X, X + 2 * NK, SC(S3_HX), SC(S3_HZ), cur(g.Eh, 7),
                                                   cur(g.Nh, 7), alpha, eta, T(1, 1), T(1, 2), w)
                                  : chain3_q<false>(m, h, X, X + 2 * NK, SC(S3_HX), SC(S3_HZ), cur(g.Eh, 7),
@@ -803,7 +805,7 @@ __global__ void __launch_bounds__(256, 2) k_spec3(const __grid_constant__ GroupD
     const double2* __restrict__ et = SC(S3_ETA);
     double2* __restrict__ u = X;
     double2* __restrict__ wv = X + 2 * NK;
-    const double ax = m.kx / m.k2, az = m.kz / m.k2;
+    const double ax = m.kx * s_ik2[lane], az = m.kz * s_ik2[lane];
 #pragma unroll 4
     for (int i = e0; i < e1; ++i) {
       const int n = p + 2 * i;
@@ -1027,7 +1029,7 @@ __global__ void __launch_bounds__(256) k_diag_final3(GroupDev g) {
   double mt = 0.0;
   for (int n = threadIdx.x; n < N; n += blockDim.x)
     if ((n & 1) == 0)
-      mt += (X[3 * NK + n].x + X[6 * NK + n].x + X[8 * NK + n].x) * (2.0 / (1.0 - (double)n * n));
+      mt += (X[3 * NK + n].x + X[6 * NK + n].x + X[8 * NK + n].x) * cheb_mean_weight(g.wrow, N, n);
   mt = block_sum(mt, sh);
   double te = 0.0;
   KeyExt ext = keyext_empty();

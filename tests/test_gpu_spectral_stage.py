@@ -32,3 +32,25 @@ def test_steps_3d(nx, ny, nz, kappa):
     for f in range(9):
         scale = max(np.max(np.abs(r)) for r in (ref[:3] if f < 3 else ref[3:]))
         assert np.max(np.abs(got[f] - ref[f])) <= 6e-11 * scale, f
+
+
+@pytest.mark.parametrize("nx,ny,kappa", [(8, 9, 5e-5), (10, 10, 5e-5), (14, 13, 0.0), (22, 34, 5e-5),
+                                         (16, 513, 5e-5), (512, 9, 5e-5)])
+def test_steps_2d(nx, ny, kappa):
+    import paper_2606_09468_gb300 as P
+    from oracle.ptt2d import Channel2D, Params
+    P.load_library()
+    kw = dict(I.PAPER, dt=I.DT)
+    kw["kappa"] = kappa
+    ora = Channel2D(Params(nx=nx, ny=ny, **kw))
+    ora.init_state(5, 0.02)
+    ctx = P.Context([P.make_params(nx=nx, ny=ny, **kw)])
+    ctx.init_state(0, 5, 0.02)
+    for _ in range(6):
+        ora.step()
+    ctx.step(6)
+    assert ctx.synchronize() == P.PTT_OK
+    got, ref = I.abi_to_phys(ctx.get_state(0)), ora.get_physical()
+    for f in range(5):
+        scale = max(np.max(np.abs(r)) for r in (ref[:2] if f < 2 else ref[2:]))
+        assert np.max(np.abs(got[f] - ref[f])) <= 6e-11 * scale, f
