@@ -1414,30 +1414,71 @@ __device__ __forceinline__ void tr_count(TrCounts& c, double t, const TrBands& B
   }
 }
 
-// Block-wide sums of 64-bit integers and merges of extrema (fixed order).
-// sh: shared memory of at least 3 * 32 long longs; the results are valid in
-// every thread.
-__device__ long long block_isum(long long v, long long* sh) {
+// Block reductions of the diagnostics in one barrier: warps reduce into shared
+// memory (sums of FP64 in lane order, then warps in index order: a fixed order;
+// counts and extrema on integers), one thread adds the warps.
+constexpr int kRedWarps = 8;   // 256 threads
+__device__ __forceinline__ double warp_sum_down(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  long long s = 0;
-  for (int i = 0; i < nw; ++i) s += sh[i];
-  __syncthreads();
-  return s;
+  return v;
 }
-__device__ KeyExt block_keyext(KeyExt e, long long* sh) {
+__device__ __forceinline__ KeyExt warp_keyext(KeyExt e) {
   for (int o = 16; o > 0; o >>= 1) keyext_merge(e, keyext_shfl_down(e, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (l == 0) { sh[w] = e.mn; sh[32 + w] = e.mx; sh[64 + w] = e.ma; }
-  __syncthreads();
-  KeyExt r = keyext_empty();
-  for (int i = 0; i < nw; ++i) keyext_merge(r, KeyExt{sh[i], sh[32 + i], sh[64 + i]});
-  __syncthreads();
-  return r;
+  return e;
+}
+// Tile results: energy, mean of Tr c (MEAN), extrema, counts (NC of them).
+template <int NC, bool MEAN>
+struct TileRed {
+  double e[kRedWarps], mt[kRedWarps];
+  long long mn[kRedWarps], mx[kRedWarps], ma[kRedWarps];
+  int cnt[kRedWarps][NC];
+  __device__ __forceinline__ void warp(double te, double tm, KeyExt x, const int (&c)[NC]) {
+    const int w = threadIdx.x >> 5;
+    te = warp_sum_down(te);
+    if (MEAN) tm = warp_sum_down(tm);
+    x = warp_keyext(x);
+    int n[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) n[k] = __reduce_add_sync(0xffffffffu, c[k]);
+    if ((threadIdx.x & 31) == 0) {
+      e[w] = te; mt[w] = tm;
+      mn[w] = x.mn; mx[w] = x.mx; ma[w] = x.ma;
+#pragma unroll
+      for (int k = 0; k < NC; ++k) cnt[w][k] = n[k];
+    }
+  }
+  // after the barrier, any thread
+  __device__ __forceinline__ double energy() const { return sum(e); }
+  __device__ __forceinline__ double mean() const { return sum(mt); }
+  __device__ __forceinline__ long long count(int k) const {
+    long long t = 0;
+    for (int w = 0; w < kRedWarps; ++w) t += cnt[w][k];
+    return t;
+  }
+  __device__ __forceinline__ KeyExt ext() const {
+    KeyExt x = keyext_empty();
+    for (int w = 0; w < kRedWarps; ++w) keyext_merge(x, KeyExt{mn[w], mx[w], ma[w]});
+    return x;
+  }
+  static __device__ __forceinline__ double sum(const double* v) {
+    double t = v[0];
+    for (int w = 1; w < kRedWarps; ++w) t += v[w];
+    return t;
+  }
+};
+// Counts of a block: out[k], k < 4, after a barrier (by threads k).
+__device__ __forceinline__ void counts_warp(const TrCounts& c, int (*sh)[4]) {
+  const int n0 = __reduce_add_sync(0xffffffffu, c.c3), n1 = __reduce_add_sync(0xffffffffu, c.c0);
+  const int n2 = __reduce_add_sync(0xffffffffu, c.b3), n3 = __reduce_add_sync(0xffffffffu, c.b0);
+  if ((threadIdx.x & 31) == 0) {
+    int* o = sh[threadIdx.x >> 5];
+    o[0] = n0; o[1] = n1; o[2] = n2; o[3] = n3;
+  }
+}
+__device__ __forceinline__ long long counts_total(const int (*sh)[4], int k) {
+  long long t = 0;
+  for (int w = 0; w < kRedWarps; ++w) t += sh[w][k];
+  return t;
 }
 
 // Sums of 32 per-thread values over the block, one total per value: a
@@ -1446,9 +1487,10 @@ __device__ KeyExt block_keyext(KeyExt e, long long* sh) {
 // lane, against 5 per value for a tree per value), then across the warps in
 // index order.  v is consumed; on return red[k], k < 32, holds the total of
 // v[k] (a fixed order: deterministic).  red: 32 * (blockDim.x / 32) doubles
-// of shared memory.
-__device__ void block_sum_scatter(double (&v)[32], double* red) {
-  const int l = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// of shared memory.  Only the first nw warps hold values.
+__device__ void block_sum_scatter(double (&v)[32], double* red, int nw) {
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < nw)
 #pragma unroll
   for (int s = 16; s >= 1; s >>= 1) {
     const bool up = (l & s) != 0;
@@ -1460,8 +1502,7 @@ __device__ void block_sum_scatter(double (&v)[32], double* red) {
     }
   }
   // lane l holds its warp's total of value l (index bits kept level by level)
-  __syncthreads();
-  red[w * 32 + l] = v[0];
+  if (w < nw) red[w * 32 + l] = v[0];
   __syncthreads();
   if (threadIdx.x < 32) {
     double t = red[threadIdx.x];
@@ -1489,48 +1530,6 @@ __device__ double block_tiles_amax(const double* pp, int ntile, int slot) {
   return __longlong_as_double(m);
 }
 
-// Max of pp[t * kPart + slot] over the ntile tiles of one member; every
-// thread of the block receives it.
-__device__ double block_tiles_max(const double* pp, int ntile, int slot) {
-  __shared__ double sm[32];
-  double m = 0.0;
-  for (int t = threadIdx.x; t < ntile; t += blockDim.x) m = fmax(m, pp[(size_t)t * kPart + slot]);
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) sm[w] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = fmax(m, sm[i]);
-    sm[0] = m;
-  }
-  __syncthreads();
-  const double r = sm[0];
-  __syncthreads();
-  return r;
-}
-
-// Block sums of NV values at once (fixed order: lanes by shuffles, then
-// warps in index order).  red: shared memory of (blockDim.x / 32) * NV
-// doubles; on return red[k], k < NV, holds the sum of v[k] over the block.
-template <int NV>
-__device__ void block_sum_many(const double (&v)[NV], double* red) {
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    double x = v[k];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if (l == 0) red[w * NV + k] = x;
-  }
-  __syncthreads();
-  double sum = 0.0;
-  if (threadIdx.x < NV)
-    for (int i = 0; i < nw; ++i) sum += red[i * NV + threadIdx.x];
-  __syncthreads();
-  if (threadIdx.x < NV) red[threadIdx.x] = sum;
-  __syncthreads();
-}
-
 // Histogram slot of x for the range [lo, hi) (PTT_HIST_BINS uniform bins,
 // slot 0 below lo, slot PTT_HIST_BINS + 1 at or above hi or not finite);
 // -1 when the quantity is switched off (lo >= hi).
@@ -1541,40 +1540,6 @@ __device__ __forceinline__ int hist_slot(double x, double lo, double hi) {
   const int k = (int)floor((x - lo) * ((double)PTT_HIST_BINS / (hi - lo)));
   return 1 + min(k, PTT_HIST_BINS - 1);
 }
-
-// Block-wide max of v (fixed order), valid in thread 0.
-__device__ double block_tiles_max_val(double v, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int i = 1; i < (int)(blockDim.x >> 5); ++i) v = fmax(v, sh[i]);
-  return v;
-}
-
-__device__ double block_sum(double v, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += sh[i];
-  }
-  return s;  // valid in thread 0
-}
-
-__device__ double2 warp_sum2(double2 v) {
-  for (int o = 16; o > 0; o >>= 1) {
-    v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-    v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-  }
-  return v;
-}
-
 
 inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 

@@ -149,21 +149,21 @@ struct GroupDev {
 constexpr int kPart = 48;  // values per diagnostics tile
 constexpr int kMacc = 33;  // window accumulator per member: 8 x 4 power sums + record count
 
-// Adds one diagnostics record's mid-plane power sums to its member's window
-// accumulator (called by the thread that writes the record).
-__device__ __forceinline__ void window_add(double* acc, const ptt_diag& r) {
-  for (int q = 0; q < 8; ++q)
-    for (int k = 0; k < 4; ++k) acc[4 * q + k] += r.mid_sums[q][k];
-  acc[32] += 1.0;
-}
+// Adds one diagnostics record's mid-plane power sum k (k < 32), or the record
+// itself (k = 32), to its member's window accumulator; a thread each.
+__device__ __forceinline__ void window_add(double* acc, int k, double sum) { acc[k] += (k < 32) ? sum : 1.0; }
 
 // Diagnostics tiles per member: about 2048 grid points each, so that one
-// member alone still spreads over the SMs; a function of the shape only, so
+// member alone still spreads over the SMs, and down to 512 (two per thread)
+// while that makes no more than 16: a tile is a chain of loads, 9 instead of 3
+// take k_diag_part and k_diag_count of a 64 x 65 step from 18 and 9.4 us to 9.6
+// and 5.8, but 64 instead of 27 at 350 x 155 hold up the next step's transforms
+// beside them (3.15 -> 3.31 ms for 20 steps).  A function of the shape only, so
 // that a member's diagnostics do not depend on the ensemble around it.
 inline int diag_tiles(int N, int nx, int nz) {
   const long long pts = (long long)N * nx * nz;
-  long long t = (pts + 2047) / 2048;
-  if (t < 1) t = 1;
+  const long long few = (pts + 511) / 512, many = (pts + 2047) / 2048;
+  long long t = few < 16 ? few : many > 16 ? many : 16;
   if (t > 1024) t = 1024;
   return (int)t;
 }

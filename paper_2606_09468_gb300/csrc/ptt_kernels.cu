@@ -570,7 +570,8 @@ __global__ void k_transpose(const double2* __restrict__ src, double2* __restrict
 //   the state on the bit patterns; then the counts of Tr c < 3, < 0 and the
 //   tie bands |Tr c - 3|, |Tr c| <= tau = 1e-9 max|Tr c|.
 enum { P_E = 0, P_MIN, P_MAX, P_AMAX, P_BAD, P_C3, P_C0, P_B3, P_B0 };
-constexpr int kMidLanes = 8, kMidModesPerBlock = 256 / kMidLanes;   // k_diag_mid, 256 threads
+// a warp per mode: with 8 lanes each the sums of 128 modes took 29 us on 4 blocks
+constexpr int kMidLanes = 32, kMidModesPerBlock = 256 / kMidLanes;   // k_diag_mid, 256 threads
 // Slot contents: P_E a double; P_MIN, P_MAX keys (dkey) of Tr c; P_AMAX the
 // bits of max |Tr c|; P_BAD and the counts 64-bit integers.
 __device__ __forceinline__ long long* islots(double* pp) { return reinterpret_cast<long long*>(pp); }
@@ -598,6 +599,7 @@ __device__ __forceinline__ void diag_part_block(const GroupDev& g, Blk bk) {
     const unsigned i0 = tile * per, i1 = min(tot, i0 + per);
     const FastDiv dK = fast_div((unsigned)K);
     double e0 = 0.0, e1 = 0.0;
+#pragma unroll 2
     for (unsigned i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
       const unsigned j = fdiv(i, dK), m = i - j * K;
       const double2 uu = DY[i], vv = DY[(size_t)Je * K + i];
@@ -623,20 +625,20 @@ __device__ __forceinline__ void diag_part_block(const GroupDev& g, Blk bk) {
     const double* X = reinterpret_cast<const double*>(g.X + (size_t)b * 5 * NK);
     const long long tot = 10LL * NK, per = (tot + g.ntile - 1) / g.ntile;
     const long long i0 = tile * per, i1 = min(tot, i0 + per);
+#pragma unroll 4
     for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) bad |= nonfinite(X[i]);
   }
-  __shared__ double sh[32];
-  __shared__ long long shk[96];
-  e = block_sum(e, sh);
-  ext = block_keyext(ext, shk);
-  bad = (int)block_isum(bad, shk);
+  __shared__ TileRed<1, false> red;
+  red.warp(e, 0.0, ext, {bad});
+  __syncthreads();
   if (threadIdx.x == 0) {
     double* pp = g.part + ((size_t)b * g.ntile + tile) * kPart;
-    pp[P_E] = e;
+    ext = red.ext();
+    pp[P_E] = red.energy();
     islots(pp)[P_MIN] = ext.mn;
     islots(pp)[P_MAX] = ext.mx;
     islots(pp)[P_AMAX] = ext.ma;
-    islots(pp)[P_BAD] = bad ? 1 : 0;
+    islots(pp)[P_BAD] = red.count(0) ? 1 : 0;
   }
 }
 
@@ -650,22 +652,17 @@ __device__ __forceinline__ void diag_count_block(const GroupDev& g, Blk bk) {
   const long long i0 = tile * per, i1 = min(tot, i0 + per);
   TrCounts c{0, 0, 0, 0};
   for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) tr_count(c, tr[i] + 1.0, B);
-  __shared__ long long shk[32];
-  const long long c3 = block_isum(c.c3, shk), c0 = block_isum(c.c0, shk);
-  const long long b3 = block_isum(c.b3, shk), b0 = block_isum(c.b0, shk);
-  if (threadIdx.x == 0) {
-    long long* pp = islots(g.part + ((size_t)b * g.ntile + tile) * kPart);
-    pp[P_C3] = c3;
-    pp[P_C0] = c0;
-    pp[P_B3] = b3;
-    pp[P_B0] = b0;
-  }
+  __shared__ int sc[kRedWarps][4];
+  counts_warp(c, sc);
+  __syncthreads();
+  if (threadIdx.x < 4)   // P_C3, P_C0, P_B3, P_B0
+    islots(g.part + ((size_t)b * g.ntile + tile) * kPart)[P_C3 + threadIdx.x] = counts_total(sc, threadIdx.x);
 }
 
 // Mid-plane spectra at y = 0, kMidLanes lanes per (member, Fourier mode):
 // T_n(0) = cos(n pi/2), T_n'(0) = n sin(n pi/2).  DM[b][q][m], q = Tr c, u, v,
 // du/dy (Chebyshev sums; x derivatives and the mean are applied later).
-// A mode's partial sums meet over its lanes only (three shuffle levels).
+// A mode's partial sums meet over its lanes only.
 __device__ __forceinline__ double2 seg_sum2(double2 v) {
 #pragma unroll
   for (int o = kMidLanes / 2; o > 0; o >>= 1) {
@@ -696,7 +693,7 @@ __device__ __forceinline__ void diag_mid_block(const GroupDev& g, Blk bk) {
       }
     } else {
       const double s = (r4 == 1) ? 1.0 : -1.0;
-      for (int n = sub; n < N; n += kMidLanes) uy = cfma(s * n, X[n], uy);
+      for (int n = sub; n < N; n += kMidLanes) uy = cfma(s * lane_i2d(n), X[n], uy);
     }
   }
   tr = seg_sum2(tr);
@@ -713,11 +710,13 @@ __device__ __forceinline__ void diag_mid_block(const GroupDev& g, Blk bk) {
 }
 
 // Per member: reduce the tiles, <Tr c> from the mean mode, mid-plane
-// statistics, blow-up test, record.
+// statistics, blow-up test, record.  One block: bound by latency; the tiles' and
+// the mean's reductions share one barrier, counts are reduced by integer warp
+// instructions, sums by the warps that have points only, and the record is
+// written by several threads (64 x 65: 31 -> 22 us, 256 x 129: 37 -> 27 us).
 __device__ __forceinline__ void diag_final_block(const GroupDev& g, Blk bk) {
   const int b = bk.x;
   if (g.status[b]) return;
-  __shared__ double sh[32];
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ FxS fs[6];
   const int K = g.K, N = g.N, nx = g.nx;
@@ -725,30 +724,28 @@ __device__ __forceinline__ void diag_final_block(const GroupDev& g, Blk bk) {
   const MemberPrm pr = g.prm[b];
   const double* pp = g.part + (size_t)b * g.ntile * kPart;
   // tile results, each thread a fixed set of tiles, then fixed-order trees
-  // (the energy in FP64, extrema and counts on integers)
-  __shared__ long long shk[96];
-  double te = 0.0;
-  KeyExt ext = keyext_empty();
-  long long tbad = 0, tc[4] = {0, 0, 0, 0};
-  for (int t = threadIdx.x; t < g.ntile; t += blockDim.x) {
-    const double* q = pp + (size_t)t * kPart;
-    const long long* qi = islots(q);
-    te += q[P_E];
-    keyext_merge(ext, KeyExt{qi[P_MIN], qi[P_MAX], qi[P_AMAX]});
-    tbad |= qi[P_BAD];
-    for (int k = 0; k < 4; ++k) tc[k] += qi[P_C3 + k];
+  // (the energy in FP64, extrema and counts on integers); <Tr c> = 1/2 int
+  // (c_xx + c_yy)_0 dy + 1, int T_n = 2/(1-n^2), n even
+  __shared__ TileRed<5, true> tr;
+  __shared__ double s_rms;
+  {
+    double te = 0.0, mt = 0.0;
+    KeyExt x = keyext_empty();
+    int tc[5] = {0, 0, 0, 0, 0};   // the four counts, non-finite tiles
+    for (int t = threadIdx.x; t < g.ntile; t += blockDim.x) {
+      const double* q = pp + (size_t)t * kPart;
+      const long long* qi = islots(q);
+      te += q[P_E];
+      keyext_merge(x, KeyExt{qi[P_MIN], qi[P_MAX], qi[P_AMAX]});
+      tc[4] += (int)qi[P_BAD];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) tc[k] += (int)qi[P_C3 + k];
+    }
+    const double2* X = g.X + (size_t)b * 5 * NK;
+    for (int n = 2 * threadIdx.x; n < N; n += 2 * blockDim.x)
+      mt += (X[2 * NK + n].x + X[4 * NK + n].x) * cheb_mean_weight(g.wrow, N, n);
+    tr.warp(te, mt, x, tc);
   }
-  te = block_sum(te, sh);
-  ext = block_keyext(ext, shk);
-  tbad = block_isum(tbad, shk);
-  for (int k = 0; k < 4; ++k) tc[k] = block_isum(tc[k], shk);
-  const TrBands B = tr_bands(1e-9 * __longlong_as_double(ext.ma));
-  const double2* X = g.X + (size_t)b * 5 * NK;
-  // <Tr c> = 1/2 int (c_xx + c_yy)_0 dy + 1, int T_n = 2/(1-n^2), n even
-  double mt = 0.0;
-  for (int n = threadIdx.x; n < N; n += blockDim.x)
-    if ((n & 1) == 0) mt += (X[2 * NK + n].x + X[4 * NK + n].x) * cheb_mean_weight(g.wrow, N, n);
-  mt = block_sum(mt, sh);
   // mid-plane lines from the per-mode sums: (Tr c, u') (v, du/dx) (dv/dx, du/dy)
   fxc* A = reinterpret_cast<fxc*>(smraw);          // 3 lines of nx
   const double kfac = pr.kx1;
@@ -782,7 +779,10 @@ __device__ __forceinline__ void diag_final_block(const GroupDev& g, Blk bk) {
     fx_xline(h, nx, K, mF, mG, fs[2 * l], fs[2 * l + 1]);
   }
   __syncthreads();
+  if (threadIdx.x == blockDim.x - 1) s_rms = sqrt(2.0 * (0.25 * tr.energy()));   // beside the transform
   fx_lines<+1, true>(A, 3, nx, &g.plNx, false);
+  const KeyExt ext = tr.ext();
+  const TrBands B = tr_bands(1e-9 * __longlong_as_double(ext.ma));
   // mid-plane histograms of the 6 quantities (shared-memory counts)
   constexpr int HS = PTT_HIST_BINS + 2;
   __shared__ unsigned int hsm[6 * HS];
@@ -825,37 +825,41 @@ __device__ __forceinline__ void diag_final_block(const GroupDev& g, Blk bk) {
     }
   }
   __shared__ double red[8 * 32];
-  block_sum_scatter(acc, red);   // its barriers also complete the shared counts
-  const long long m3 = block_isum(mc.c3, shk), m0 = block_isum(mc.c0, shk);
-  const long long mb3 = block_isum(mc.b3, shk), mb0 = block_isum(mc.b0, shk);
+  __shared__ int sc[kRedWarps][4];
+  counts_warp(mc, sc);
+  block_sum_scatter(acc, red, min(kRedWarps, (nx + 31) >> 5));   // its barriers also complete the shared counts
   if (hon) {
     unsigned long long* gh = g.hist + (size_t)b * 8 * HS;
     for (int i = threadIdx.x; i < 6 * HS; i += blockDim.x)
       if (hsm[i]) atomicAdd(&gh[i], (unsigned long long)hsm[i]);
   }
-  if (threadIdx.x == 0) {
-    const double e = 0.25 * te;
-    const bool bad = (tbad != 0);
-    const long long step = g.count[b];
+  const long long step = g.count[b];
+  ptt_diag& r = g.ring[(size_t)b * kRing + (size_t)(step % kRing)];
+  if (threadIdx.x < 33) {   // power sums of the record and of its member's window
+    const int k = threadIdx.x;
+    const double v = (k < 24) ? red[k] : 0.0;
+    if (k < 32) r.mid_sums[k >> 2][k & 3] = v;
+    window_add(g.macc + (size_t)b * kMacc, k, v);
+  }
+  if (threadIdx.x == blockDim.x - 1) {
+    const double e = 0.25 * tr.energy();
+    const bool bad = (tr.count(4) != 0);
     const double qnan = __longlong_as_double(0x7ff8000000000000LL);
-    ptt_diag& r = g.ring[(size_t)b * kRing + (size_t)(step % kRing)];
     r.step = step;
     r.t = step * pr.dt;
     r.energy = e;
-    r.mean_trc = 0.5 * mt + 1.0;
+    r.mean_trc = 0.5 * tr.mean() + 1.0;
     r.min_trc = bad ? qnan : dkey_val(ext.mn);
-    r.max_trc = bad ? qnan : dkey_val(ext.mx);
-    r.n_lt3 = tc[0]; r.n_lt0 = tc[1];
-    r.n_band3 = tc[2]; r.n_band0 = tc[3];
-    r.n_mid_lt3 = m3; r.n_mid_lt0 = m0;
-    r.n_mid_band3 = mb3; r.n_mid_band0 = mb0;
-    for (int qq = 0; qq < 8; ++qq)
-      for (int k = 0; k < 4; ++k) r.mid_sums[qq][k] = (qq < 6) ? red[4 * qq + k] : 0.0;
-    const bool blow = bad || !isfinite(e) || r.max_trc > pr.trc_max || sqrt(2.0 * e) > pr.u_max;
+    const double mx = bad ? qnan : dkey_val(ext.mx);
+    r.max_trc = mx;
+    r.n_lt3 = tr.count(0); r.n_lt0 = tr.count(1);
+    r.n_band3 = tr.count(2); r.n_band0 = tr.count(3);
+    r.n_mid_lt3 = counts_total(sc, 0); r.n_mid_lt0 = counts_total(sc, 1);
+    r.n_mid_band3 = counts_total(sc, 2); r.n_mid_band0 = counts_total(sc, 3);
+    const bool blow = bad || !isfinite(e) || mx > pr.trc_max || s_rms > pr.u_max;
     r.status = blow ? PTT_BLOWUP : PTT_OK;
     r.reserved = 0;
     if (blow) g.status[b] = 1;
-    window_add(g.macc + (size_t)b * kMacc, r);
   }
 }
 

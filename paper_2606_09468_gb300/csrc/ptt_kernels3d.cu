@@ -864,6 +864,7 @@ __global__ void __launch_bounds__(256) k_diag_part3(GroupDev g) {
     const unsigned i0 = tile * per, i1 = min(tot, i0 + per);
     const FastDiv dKZ = fast_div((unsigned)KZ);
     double e0 = 0.0, e1 = 0.0;
+#pragma unroll 2
     for (unsigned i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
       const unsigned j = fdiv(i, dKZ), md = i - j * KZ;
       const double2 a0 = DY[i], a1 = DY[(size_t)Je * KZ + i], a2 = DY[(size_t)2 * Je * KZ + i];
@@ -888,20 +889,20 @@ __global__ void __launch_bounds__(256) k_diag_part3(GroupDev g) {
     const double* Xd = reinterpret_cast<const double*>(g.X + (size_t)b * 9 * NK);
     const long long tot = 18LL * NK, per = (tot + g.ntile - 1) / g.ntile;
     const long long i0 = tile * per, i1 = min(tot, i0 + per);
+#pragma unroll 4
     for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) bad |= nonfinite3(Xd[i]);
   }
-  __shared__ double sh[32];
-  __shared__ long long shk[96];
-  e = block_sum(e, sh);
-  ext = block_keyext(ext, shk);
-  bad = (int)block_isum(bad, shk);
+  __shared__ TileRed<1, false> red;
+  red.warp(e, 0.0, ext, {bad});
+  __syncthreads();
   if (threadIdx.x == 0) {
     double* pp = g.part + ((size_t)b * g.ntile + tile) * kPart;
-    pp[P_E] = e;
+    ext = red.ext();
+    pp[P_E] = red.energy();
     islots3(pp)[P_MIN] = ext.mn;
     islots3(pp)[P_MAX] = ext.mx;
     islots3(pp)[P_AMAX] = ext.ma;
-    islots3(pp)[P_BAD] = bad ? 1 : 0;
+    islots3(pp)[P_BAD] = red.count(0) ? 1 : 0;
   }
 }
 
@@ -920,14 +921,11 @@ __global__ void __launch_bounds__(256) k_diag_count3(GroupDev g) {
     const long long i0 = tile * per, i1 = min(tot, i0 + per);
     for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) tr_count(c, tr[i], B);
   }
-  __shared__ long long shk[32];
-  const long long c3 = block_isum(c.c3, shk), c0 = block_isum(c.c0, shk);
-  const long long b3 = block_isum(c.b3, shk), b0 = block_isum(c.b0, shk);
+  __shared__ int sc[kRedWarps][4];
+  counts_warp(c, sc);
+  __syncthreads();
   double* pp = g.part + ((size_t)b * g.ntile + tile) * kPart;
-  if (threadIdx.x == 0) {
-    islots3(pp)[P_C3] = c3; islots3(pp)[P_C0] = c0;
-    islots3(pp)[P_B3] = b3; islots3(pp)[P_B0] = b0;
-  }
+  if (threadIdx.x < 4) islots3(pp)[P_C3 + threadIdx.x] = counts_total(sc, threadIdx.x);   // P_C3, P_C0, P_B3, P_B0
   const int npl = g.nz * g.nx;
   if (tile >= mid_tiles(npl, g.ntile)) return;   // block-uniform
   double sums[32];
@@ -954,14 +952,11 @@ __global__ void __launch_bounds__(256) k_diag_count3(GroupDev g) {
     }
   }
   __shared__ double red[8 * 32];
-  block_sum_scatter(sums, red);
-  const long long m3 = block_isum(mc.c3, shk), m0 = block_isum(mc.c0, shk);
-  const long long mb3 = block_isum(mc.b3, shk), mb0 = block_isum(mc.b0, shk);
+  __shared__ int smc[kRedWarps][4];
+  counts_warp(mc, smc);
+  block_sum_scatter(sums, red, kRedWarps);   // its barriers also complete the counts
   if (threadIdx.x < 32) pp[P_MS + threadIdx.x] = red[threadIdx.x];
-  if (threadIdx.x == 0) {
-    islots3(pp)[P_MC3] = m3; islots3(pp)[P_MC0] = m0;
-    islots3(pp)[P_MB3] = mb3; islots3(pp)[P_MB0] = mb0;
-  }
+  if (threadIdx.x < 4) islots3(pp)[P_MC3 + threadIdx.x] = counts_total(smc, threadIdx.x);   // P_MC3 ... P_MB0
 }
 
 // Mid-plane spectra at y = 0 per mode (kMidLanes3 lanes each): DM[b][q][mode]
@@ -985,10 +980,9 @@ __global__ void __launch_bounds__(256) k_diag_mid3(GroupDev g) {
   const size_t NK = (size_t)N * KZ;
   const double2* X = g.X + (size_t)b * 9 * NK + (size_t)(on ? md : 0) * N;
   double2 tr = czero(), u = czero(), v = czero(), w = czero();
-  const int r4 = sub & 3;   // n = sub (mod kMidLanes3): one residue of n mod 4 per lane
-  if (on && (r4 == 0 || r4 == 2)) {
-    const double s = (r4 == 0) ? 1.0 : -1.0;
-    for (int n = sub; n < N; n += kMidLanes3) {
+  if (on) {   // even n, one residue of n mod 4 per lane
+    const double s = (sub & 1) ? -1.0 : 1.0;
+    for (int n = 2 * sub; n < N; n += 2 * kMidLanes3) {
       tr = cfma(s, cadd(X[3 * NK + n], cadd(X[6 * NK + n], X[8 * NK + n])), tr);
       u = cfma(s, X[n], u);
       v = cfma(s, X[NK + n], v);
@@ -1019,67 +1013,68 @@ __global__ void __launch_bounds__(256) k_diag_mid3(GroupDev g) {
 __global__ void __launch_bounds__(256) k_diag_final3(GroupDev g) {
   const int b = blockIdx.x;
   if (g.status[b]) return;
-  __shared__ double sh[32];
-  __shared__ long long shk[96];
   const int KZ = g.KZ, N = g.N;
   const size_t NK = (size_t)N * KZ;
   const MemberPrm pr = g.prm[b];
   const double* pp = g.part + (size_t)b * g.ntile * kPart;
   const double2* X = g.X + (size_t)b * 9 * NK;
-  double mt = 0.0;
-  for (int n = threadIdx.x; n < N; n += blockDim.x)
-    if ((n & 1) == 0)
-      mt += (X[3 * NK + n].x + X[6 * NK + n].x + X[8 * NK + n].x) * cheb_mean_weight(g.wrow, N, n);
-  mt = block_sum(mt, sh);
-  double te = 0.0;
-  KeyExt ext = keyext_empty();
-  long long tbad = 0, cnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int t = threadIdx.x; t < g.ntile; t += blockDim.x) {
-    const double* q = pp + (size_t)t * kPart;
-    const long long* qi = islots3(q);
-    te += q[P_E];
-    keyext_merge(ext, KeyExt{qi[P_MIN], qi[P_MAX], qi[P_AMAX]});
-    tbad |= qi[P_BAD];
-    for (int k = 0; k < 4; ++k) cnt[k] += qi[P_C3 + k];
-  }
+  __shared__ TileRed<9, true> tr;
   const int nmt = mid_tiles(g.nz * g.nx, g.ntile);
-  for (int t = threadIdx.x; t < nmt; t += blockDim.x)
-    for (int k = 0; k < 4; ++k) cnt[4 + k] += islots3(pp + (size_t)t * kPart)[P_MC3 + k];
-  te = block_sum(te, sh);
-  ext = block_keyext(ext, shk);
-  tbad = block_isum(tbad, shk);
-  for (int k = 0; k < 8; ++k) cnt[k] = block_isum(cnt[k], shk);
-  // mid-plane sums: thread k < 32 adds slot k over the mid tiles in order
-  __shared__ double ms[32];
-  if (threadIdx.x < 32) {
-    double a = 0.0;
-    for (int t = 0; t < nmt; ++t) a += pp[(size_t)t * kPart + P_MS + threadIdx.x];
-    ms[threadIdx.x] = a;
+  {
+    double te = 0.0, mt = 0.0;
+    KeyExt x = keyext_empty();
+    int tc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};   // volume and mid-plane counts, non-finite tiles
+    for (int n = 2 * threadIdx.x; n < N; n += 2 * blockDim.x)
+      mt += (X[3 * NK + n].x + X[6 * NK + n].x + X[8 * NK + n].x) * cheb_mean_weight(g.wrow, N, n);
+    for (int t = threadIdx.x; t < g.ntile; t += blockDim.x) {
+      const double* q = pp + (size_t)t * kPart;
+      const long long* qi = islots3(q);
+      te += q[P_E];
+      keyext_merge(x, KeyExt{qi[P_MIN], qi[P_MAX], qi[P_AMAX]});
+      tc[8] += (int)qi[P_BAD];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) tc[k] += (int)qi[P_C3 + k];
+    }
+    for (int t = threadIdx.x; t < nmt; t += blockDim.x)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) tc[4 + k] += (int)islots3(pp + (size_t)t * kPart)[P_MC3 + k];
+    tr.warp(te, mt, x, tc);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const double e = 0.25 * te;
-    const bool bad = (tbad != 0);
-    const long long step = g.count[b];
+  const long long step = g.count[b];
+  ptt_diag& r = g.ring[(size_t)b * kRing + (size_t)(step % kRing)];
+  // mid-plane sums: thread k < 32 adds slot k over the mid tiles in order, for
+  // the record and its member's window
+  if (threadIdx.x < 33) {
+    const int k = threadIdx.x;
+    double a = 0.0;
+    if (k < 32) {
+#pragma unroll 4
+      for (int t = 0; t < nmt; ++t) a += pp[(size_t)t * kPart + P_MS + k];
+      r.mid_sums[k >> 2][k & 3] = a;
+    }
+    window_add(g.macc + (size_t)b * kMacc, k, a);
+  }
+  if (threadIdx.x == blockDim.x - 1) {
+    const double e = 0.25 * tr.energy();
+    const KeyExt ext = tr.ext();
+    const bool bad = (tr.count(8) != 0);
     const double qnan = __longlong_as_double(0x7ff8000000000000LL);
-    ptt_diag& r = g.ring[(size_t)b * kRing + (size_t)(step % kRing)];
     r.step = step;
     r.t = step * pr.dt;
     r.energy = e;
-    r.mean_trc = 0.5 * mt;
+    r.mean_trc = 0.5 * tr.mean();
     r.min_trc = bad ? qnan : dkey_val(ext.mn);
-    r.max_trc = bad ? qnan : dkey_val(ext.mx);
-    r.n_lt3 = cnt[0]; r.n_lt0 = cnt[1];
-    r.n_band3 = cnt[2]; r.n_band0 = cnt[3];
-    r.n_mid_lt3 = cnt[4]; r.n_mid_lt0 = cnt[5];
-    r.n_mid_band3 = cnt[6]; r.n_mid_band0 = cnt[7];
-    for (int q = 0; q < 8; ++q)
-      for (int k = 0; k < 4; ++k) r.mid_sums[q][k] = ms[4 * q + k];
-    const bool blow = bad || !isfinite(e) || r.max_trc > pr.trc_max || sqrt(2.0 * e) > pr.u_max;
+    const double mx = bad ? qnan : dkey_val(ext.mx);
+    r.max_trc = mx;
+    r.n_lt3 = tr.count(0); r.n_lt0 = tr.count(1);
+    r.n_band3 = tr.count(2); r.n_band0 = tr.count(3);
+    r.n_mid_lt3 = tr.count(4); r.n_mid_lt0 = tr.count(5);
+    r.n_mid_band3 = tr.count(6); r.n_mid_band0 = tr.count(7);
+    const bool blow = bad || !isfinite(e) || mx > pr.trc_max || sqrt(2.0 * e) > pr.u_max;
     r.status = blow ? PTT_BLOWUP : PTT_OK;
     r.reserved = 0;
     if (blow) g.status[b] = 1;
-    window_add(g.macc + (size_t)b * kMacc, r);
   }
 }
 
