@@ -1166,9 +1166,17 @@ struct XJob {
   // c2r with nf = 1: pair_rows lines per block, line p of all synthesises rows
   // 2p and 2p + 1 (< nrows) as its real and imaginary parts (xrows_pairs)
   int pair_rows, nrows;
+  // 3D physical values of a caller: real row y zy_nz + z lies at z zy_ny + y
+  // (zy_nz = 0: rows in order)
+  int zy_nz, zy_ny;
   const int* status;
   FftPlan pl;
 };
+__device__ __forceinline__ int xrow_real(const XJob& J, int row) {
+  if (J.zy_nz == 0) return row;
+  const int y = row / J.zy_nz;
+  return (row - y * J.zy_nz) * J.zy_ny + y;
+}
 
 // Fixed-point lines of real fields, shared by the x transforms: two fields
 // per line of n points, field q of the block on scale fs[q] (line q >> 1).
@@ -1290,7 +1298,7 @@ __device__ __forceinline__ void xrows_block(const XJob& J, Blk bk) {
     }
     __syncthreads();
     fx_lines<+1, true>(A, nl, n, &J.pl, false);
-    double* dst = J.dstR + b * J.dst_mstride + (long long)r0 * J.dst_rstep * n;
+    double* dst = J.dstR + b * J.dst_mstride + (long long)xrow_real(J, r0) * J.dst_rstep * n;
     for (int i = tid; i < nl * n; i += nt) {
       const int l = (int)fdiv((unsigned)i, dn), x = i - l * n;
       const fxc h = A[i];
@@ -1299,7 +1307,7 @@ __device__ __forceinline__ void xrows_block(const XJob& J, Blk bk) {
     }
   } else {
     const int nl = (nf + 1) / 2;
-    const double* src = J.srcR + b * J.src_mstride + (long long)row * J.src_rstep * n;
+    const double* src = J.srcR + b * J.src_mstride + (long long)xrow_real(J, row) * J.src_rstep * n;
     for (int l = tid >> 5; l < nl; l += nw) {
       fxc* h = A + l * n;
       for (int x = lane; x < n; x += 32)

@@ -230,7 +230,9 @@ cudaError_t launch_diag3(const GroupDev& g, cudaStream_t st, int* nlaunch);
 cudaError_t launch_diag_split3(const GroupDev& g, const DiagStreams& d, int* nlaunch);
 cudaError_t launch_diag_transforms3(const GroupDev& g, cudaStream_t st);
 cudaError_t launch_explicit3(const GroupDev& g, cudaStream_t st);
-cudaError_t launch_phys_to_state3(const GroupDev& g, int b, cudaStream_t st);
+// Physical values in g.stage: a caller's order [field][z][y][x] (abi), or
+// [field][y][z][x].
+cudaError_t launch_phys_to_state3(const GroupDev& g, int b, bool abi, cudaStream_t st);
 cudaError_t launch_state_to_phys3(const GroupDev& g, int b, cudaStream_t st);
 cudaError_t launch_reset_member3(const GroupDev& g, int b, cudaStream_t st);
 // Shared memory of the 3D fused x pass (18 lines: two FP32 buffers, or one in

@@ -1405,12 +1405,13 @@ cudaError_t launch_reset_member3(const GroupDev& g, int b, cudaStream_t st) {
 
 // physical staging [9][ny][nz][nx] -> state of member b: x analysis per
 // (y, z) row, z analysis per (y, mx), y analysis (DCT-I) per mode.
-cudaError_t launch_phys_to_state3(const GroupDev& g, int b, cudaStream_t st) {
+cudaError_t launch_phys_to_state3(const GroupDev& g, int b, bool abi, cudaStream_t st) {
   const int K = g.K, KZ = g.KZ, N = g.N, nz = g.nz, nx = g.nx;
   const size_t NK = (size_t)N * KZ;
   const long long rowsp = (long long)N * nz;
   XJob X{};
   X.srcR = g.stage; X.dstC = g.DZ;   // DZ reused as [9][N][nz][K]
+  if (abi) { X.zy_nz = nz; X.zy_ny = N; }
   X.src_fstride = rowsp * nx; X.dst_fstride = rowsp * K;
   X.src_rstep = 1; X.dst_rstep = 1;
   X.nf = 9; X.K = K; X.n = nx; X.c2r = 0; X.status = nullptr; X.pl = g.plNx;
@@ -1449,6 +1450,7 @@ cudaError_t launch_state_to_phys3(const GroupDev& g, int b, cudaStream_t st) {
   k_zcols_fx<true><<<dim3(cdiv(K, Z.C), 9 * N, 1), 256, smem_zcols(Z.C, nz), st>>>(Z);
   XJob X{};
   X.srcC = g.DZ; X.dstR = g.stage;
+  X.zy_nz = nz; X.zy_ny = N;
   X.src_fstride = rowsp * K; X.dst_fstride = rowsp * nx;
   X.src_rstep = 1; X.dst_rstep = 1;
   X.nf = 9; X.K = K; X.n = nx; X.c2r = 1; X.status = nullptr; X.pl = g.plNx;
