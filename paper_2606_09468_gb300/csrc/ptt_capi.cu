@@ -554,8 +554,13 @@ void group_sizes(int nx, int ny, int nz, Group& g) {
   d.Ccol = cols(!d.f32, d.M, d.N);
   d.CcolE = cols(!d.f32, d.Me, 0);
   d.CcolU = cols(true, d.Pu, 0);
-  d.xthreads = 512;   // launch-shape defaults (ptt_autotune may change them)
-  d.zC = 8;
+  // launch-shape defaults (ptt_autotune may change them).  x-mode lines per
+  // block of the z passes: 16 (whole 128-byte or 256-byte runs of a row, and the
+  // set-up of a block over more lines) while they take 32 KB.  y and z inverse
+  // of a mixed step, 8 and 16 lines: Mz = 96 0.356 and 0.332 ms, Mz = 66 0.167
+  // and 0.154, Mz = 192 1.53 and 1.66; FP64, Mz = 96: 0.642 and 0.613.
+  d.zC = 16;
+  while (d.zC > 1 && (d.zC > d.K || d.zC * d.Mz > 2048)) d.zC >>= 1;
 }
 
 // Plans of a group (d.f32 set): an FP32 group's padded lengths (M, Mx, Mz)
@@ -569,7 +574,19 @@ void group_plans(Group& g) {
     g.hp[i] = g.fx[i] ? make_plan_fx(n[i], three[i]) : make_plan(n[i], three[i]);
   }
   g.hpn = make_plan_fx(g.d.M);
-  if (!g.d.f32) g.d.xthreads = 256;
+  // threads of the fused x pass.  FP32: the 1024 that 64 registers leave an SM,
+  // over the blocks that shared memory leaves it (fewer threads a block have
+  // fewer idle in the passes, fewer blocks less of a block's barriers hidden).
+  // 3D, 512 and this many: Mx = 192 (256 threads) 0.406 and 0.286 ms, Mx = 135
+  // (192) 0.218 and 0.140, Mx = 384 (512; with 256 2.04) 1.96; 2D, the 27 shapes
+  // together 0.326 and 0.297.
+  if (g.d.f32) {
+    const long long sm = g.d.nz > 1 ? smem_xfused3(g.d.Mx, 1) : smem_xfused(g.d.Mx, 1);
+    const long long blocks = std::max(1LL, 227 * 1024LL / (sm + 1024));
+    g.d.xthreads = (int)std::max(128LL, std::min(512LL, 1024 / blocks / 64 * 64));
+  } else {
+    g.d.xthreads = 256;
+  }
 }
 
 // Least threads per block of the plan's passes.
