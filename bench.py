@@ -85,7 +85,7 @@ def parse():
                          "3d_mixed_large, ensemble_mixed, ensemble_fp64, 2d_NXxNY[_mixed]: one "
                          "shape of the 2D sweep, three seeds; 'mixedtc' in place of 'mixed' "
                          "selects the tensor-core Chebyshev passes instead of the FP32 FFTs, a "
-                         "'_ds' suffix the double-single form (PTT_FP64_DS); "
+                         "'_ds' suffix the form PTT_FP64_DS (the kernels of FP64); "
                          "3d_NXxNYxNZ[_mixed]: one 3D shape; sweep[_mixed|_ds]: the 27-run 2D "
                          "sweep; paper_shapes: the A1-A6 timings) "
                          "and print its line, for profiling; or midplane_stats: mixed vs FP64 "
@@ -529,11 +529,11 @@ def other_workloads(args):
             name = "3d_%s_%dx%dx%d" % (tags[prec], *shape)
             out[name] = {"value": pts * 1e3 / ms, "unit": METRIC, "ms_per_step": ms, "steps": n,
                          "grid_points": pts, "status": status,
-                         "dtype": {P.PTT_FP64: "f64",
+                         "dtype": {P.PTT_FP64: "f64 (transforms in 64-bit fixed point)",
                                    P.PTT_MIXED: "f32 transforms+products / f64 state+solves",
                                    P.PTT_MIXED_TC: "f32 x/z transforms+products, tensor-core "
                                                    "Chebyshev contractions / f64 state+solves",
-                                   P.PTT_FP64_DS: "double-single transforms+products / f64 "
+                                   P.PTT_FP64_DS: "64-bit fixed-point transforms / f64 products, "
                                                   "state+solves"}[prec],
                          "workload": "3D sPTT channel %dx%dx%d (x, y, z), Lx=10, Lz=5, paper fluid, "
                                      "dt=1e-3, laminar + seeded perturbation 1e-3" % shape}
@@ -585,7 +585,7 @@ def other_workloads(args):
 
 def paper_shapes(args):
     """The paper's production shapes (Table 1) at its box and time step, a few
-    steps each, in mixed precision, FP64 and double-single, with the wall time
+    steps each, in mixed precision, FP64 and FP64_DS, with the wall time
     the paper's run length (T/Wi = 68, dt = 2.5e-3) would take at the measured
     rate on this one GPU.  The
     paper's own cost, on CPU cores of ARCHER2: A1 2e5 core-hours, A6 1.6e6
@@ -779,8 +779,8 @@ def run_ours(args):
                          "stated_error_vs_oracle": "tests/test_gpu_mma.py: explicit rhs <= 1e-6 "
                                                    "(measured 0.9-1.6e-7 in 2D, as the FFT form)"})
         fp64_ds = mixed_form(P.PTT_FP64_DS)
-        fp64_ds.update({"dtype": "double-single (pairs of f32, 48 bits) transforms+products / "
-                                 "f64 state+solves+diagnostics",
+        fp64_ds.update({"dtype": "64-bit fixed-point transforms (the kernels of PTT_FP64) / "
+                                 "f64 products+state+solves+diagnostics",
                         "stated_error_vs_oracle": "tests/test_gpu_ds.py: the FP64 bars, 1 step <= 1e-11, "
                                                   "100 steps <= 1e-9"})
 
