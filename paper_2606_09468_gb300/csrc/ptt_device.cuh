@@ -258,7 +258,7 @@ struct FastDiv {
   unsigned m;
   bool one;
 };
-__device__ __forceinline__ FastDiv fast_div(unsigned d) {
+__host__ __device__ __forceinline__ FastDiv fast_div(unsigned d) {
   FastDiv f;
   f.one = (d == 1u);
   f.m = f.one ? 0u : 0xFFFFFFFFu / d + 1u;

@@ -46,6 +46,7 @@ struct ZJob {
   const int* status;
   const MemberPrm* prm;
   FftPlan pl;         // length Mz
+  FastDiv dC, dnz, dMz, drows;   // of C, nz, Mz, rows (z_set_lines)
   // mixed groups' step passes (mean/fluctuation split, see k_xfused3):
   // mean = 1, inverse: the kx = 0 line leaves its kz = 0 (mean) mode out;
   // mean = 2, forward: the kx = 0 line's mean mode is added in FP64 to
@@ -141,12 +142,16 @@ __global__ void __launch_bounds__(256, BIG ? 3 : 5) k_zcols_fx(const __grid_cons
   }
 }
 
-// FP32 z lines (mixed groups' step).
+// FP32 z lines (mixed groups' step).  Bound by instruction issue: three points
+// a thread or six, so what a block sets up counts.  The index divisors come
+// from the host and one loop fills the padded lines (before: a division per
+// loop and thread, a fill and a barrier of its own); 128 x 97 x 64, ten steps:
+// 12.99 -> 12.81 ms.
 __global__ void __launch_bounds__(256) k_zcols(ZJob J) {
   using CT = float2;
   const int b = blockIdx.z;
   if (J.status && J.status[b]) return;
-  const int f = blockIdx.y / J.rows;
+  const int f = (int)fdiv(blockIdx.y, J.drows);
   const int j = blockIdx.y - f * J.rows;
   const int C = J.C, K = J.K, nz = J.nz, Mz = J.Mz;
   const int m0 = blockIdx.x * C;
@@ -163,24 +168,24 @@ __global__ void __launch_bounds__(256) k_zcols(ZJob J) {
               (long long)j * Mz * K;
     const float kfac = J.prm[b].kz1f;
     const int dz = J.dz[f];
-    for (int i = tid; i < C * Mz; i += nt) A[i] = zero2<CT>();
-    __syncthreads();
     const bool skip0 = (J.mean == 1 && m0 == 0);
-    for (int i = tid; i < C * nz; i += nt) {
-      const int c = (int)fdiv((unsigned)i, fast_div((unsigned)nz)), mz = i - c * nz;
-      if (c < nc && mz != hz && !(skip0 && c == 0 && mz == 0)) {
-        const int s = (mz < hz) ? mz : mz - nz;
-        CT v = src[(long long)(m0 + c) * nz + mz];
+    for (int i = tid; i < C * Mz; i += nt) {
+      // slot q of line c: mode q, or q - Mz from the end; the padded middle is zero
+      const int c = (int)fdiv((unsigned)i, J.dMz), q = i - c * Mz;
+      const int s = (q < hz) ? q : q - Mz;
+      CT v = zero2<CT>();
+      if (c < nc && s > -hz && s < hz && !(skip0 && i == 0)) {
+        v = src[(m0 + c) * nz + (s < 0 ? s + nz : s)];
         if (dz) v = cscl(mul_i(v), kfac * (float)s);
-        A[c * Mz + (s >= 0 ? s : s + Mz)] = v;
       }
+      A[i] = v;
     }
     __syncthreads();
     // padded synthesis (Mz >= 3 nz/2): the slots nz/2 .. Mz - nz/2 are zero
     CT* res = fft_lines<+1>(A, B, C, Mz, J.pl, J.pl.radix[0] == 3 && Mz >= 3 * hz);
     for (int i = tid; i < Mz * C; i += nt) {
-      const int z = (int)fdiv((unsigned)i, fast_div((unsigned)C)), c = i - z * C;
-      if (c < nc) dst[(long long)z * K + m0 + c] = res[c * Mz + z];
+      const int z = (int)fdiv((unsigned)i, J.dC), c = i - z * C;
+      if (c < nc) dst[z * K + m0 + c] = res[c * Mz + z];
     }
   } else {
     const CT* src = static_cast<const CT*>(J.src) + b * J.src_mstride + J.src_field[f] * J.src_fstride +
@@ -188,14 +193,14 @@ __global__ void __launch_bounds__(256) k_zcols(ZJob J) {
     CT* dst = static_cast<CT*>(J.dst) + b * J.dst_mstride + J.dst_field[f] * J.dst_fstride +
               (long long)j * K * nz;
     for (int i = tid; i < Mz * C; i += nt) {
-      const int z = (int)fdiv((unsigned)i, fast_div((unsigned)C)), c = i - z * C;
-      A[c * Mz + z] = (c < nc) ? src[(long long)z * K + m0 + c] : zero2<CT>();
+      const int z = (int)fdiv((unsigned)i, J.dC), c = i - z * C;
+      A[c * Mz + z] = (c < nc) ? src[z * K + m0 + c] : zero2<CT>();
     }
     __syncthreads();
     CT* res = fft_lines<-1>(A, B, C, Mz, J.pl);
     const float inv = J.invf;
     for (int i = tid; i < C * nz; i += nt) {
-      const int c = (int)fdiv((unsigned)i, fast_div((unsigned)nz)), mz = i - c * nz;
+      const int c = (int)fdiv((unsigned)i, J.dnz), mz = i - c * nz;
       if (c < nc) {
         CT v = zero2<CT>();
         if (mz != hz) {
@@ -206,7 +211,7 @@ __global__ void __launch_bounds__(256) k_zcols(ZJob J) {
           J.zm[((size_t)b * 9 + J.dst_field[f]) * J.rows + j].x += (double)v.x;
           v = zero2<CT>();
         }
-        dst[(long long)(m0 + c) * nz + mz] = v;
+        dst[(m0 + c) * nz + mz] = v;
       }
     }
   }
@@ -1106,6 +1111,11 @@ YJob yjob3(const GroupDev& g, bool inverse, int M, int C, const FftPlan& pl, boo
   return J;
 }
 
+static void z_set_lines(ZJob& Z, int C) {
+  Z.C = C;
+  Z.dC = fast_div((unsigned)C);
+}
+
 ZJob zjob(const GroupDev& g, bool inverse, int Mz, int rows, const FftPlan& pl) {
   ZJob Z{};
   Z.K = g.K;
@@ -1114,11 +1124,14 @@ ZJob zjob(const GroupDev& g, bool inverse, int Mz, int rows, const FftPlan& pl) 
   Z.inv = 1.0 / Mz;
   Z.invf = (float)Z.inv;
   Z.inverse = inverse ? 1 : 0;
-  Z.C = 8;
   Z.rows = rows;
   Z.status = g.status;
   Z.prm = g.prm;
   Z.pl = pl;
+  Z.dnz = fast_div((unsigned)Z.nz);
+  Z.dMz = fast_div((unsigned)Mz);
+  Z.drows = fast_div((unsigned)rows);
+  z_set_lines(Z, 8);
   return Z;
 }
 
@@ -1201,7 +1214,7 @@ cudaError_t launch_stage3(const GroupDev& g, int stage, cudaStream_t st, int* nl
         ++n;
       }
       ZJob Z = zjob(g, true, Mz, M, g.plMz);
-      Z.C = g.zC;
+      z_set_lines(Z, g.zC);
       Z.src = J.dst;
       Z.dst = f32 ? (void*)g.Z3f : (void*)g.Z3;
       Z.mean = f32 ? 1 : 0;
@@ -1229,7 +1242,7 @@ cudaError_t launch_stage3(const GroupDev& g, int stage, cudaStream_t st, int* nl
     }
     case 2: {  // forward z (9) then forward y (9)
       ZJob Z = zjob(g, false, Mz, M, g.plMz);
-      Z.C = g.zC;
+      z_set_lines(Z, g.zC);
       Z.src = f32 ? (const void*)g.W3f : (const void*)g.W3;
       Z.dst = f32 ? (void*)g.V3f : (void*)g.V3;
       Z.mean = f32 ? 2 : 0;
