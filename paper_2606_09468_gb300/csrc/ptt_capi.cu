@@ -58,78 +58,6 @@ void cis(long long k, long long n, double* c, double* s) {
   *s = sgn_s * ss;
 }
 
-struct HostPlan {
-  int n = 0;
-  std::vector<int> radix;
-};
-
-// FP32 plans (mixed groups: the padded lengths and the energy grid), radices
-// 2 to 5 and 8 (few passes: each is a shared-memory round trip, and the
-// transforms are bound by instruction issue).  three_first: the padded x and z
-// lengths (3K or more for K kept modes), whose inverse lines are zero in the
-// middle third [n/3, 2n/3): a first pass of radix 3 has one zero input; used
-// where n has no factor 5.
-HostPlan make_plan(int n, bool three_first = false) {
-  HostPlan p;
-  p.n = n;
-  int r = n;
-  if (three_first && n % 3 == 0 && n % 5 != 0) { p.radix.push_back(3); r /= 3; }
-  // radix 5 first: the first pass takes no twiddles
-  for (int f : {5, 8, 4, 2, 3})
-    while (r % f == 0) { p.radix.push_back(f); r /= f; }
-  return p;
-}
-
-// Threads of the y and z kernels, which run their passes' butterflies at once
-// per group of lines: a plan's n / radix stays within them (fx_mb).
-constexpr int kFxPassThreads = 256;
-
-// Fixed-point plans: the factorisation of least estimated time per point, from
-// the cycles per warp of a butterfly (additions 2, products with a constant
-// 17, twiddles 55 per complex value) and about 35 per point and pass for the
-// shared-memory round trip and the indexes.  Primes 7, 11 and 13 (unpadded
-// lengths) take one pass each.  The first pass is an odd radix where there is
-// one: its stores are a radix apart, and even strides collide in the
-// shared-memory banks; three_first as above (radix 3 or 6).
-HostPlan make_plan_fx(int n, bool three_first = false) {
-  HostPlan p;
-  p.n = n;
-  int r = n;
-  std::vector<int> odd;
-  for (int f : {13, 11, 7})
-    while (r % f == 0) { odd.push_back(f); r /= f; }
-  const int rad[6] = {8, 6, 5, 4, 3, 2};
-  const double cost[6] = {103, 107, 121, 84, 94, 66};
-  std::vector<int> best, cur;
-  double bc = 1e30;
-  auto search = [&](auto&& self, int m, int from, double c) -> void {
-    if (c >= bc) return;
-    if (m == 1) { bc = c; best = cur; return; }
-    for (int i = from; i < 6; ++i)
-      if (m % rad[i] == 0 && n / rad[i] <= kFxPassThreads * fx_mb(rad[i])) {
-        cur.push_back(rad[i]);
-        self(self, m / rad[i], i, c + cost[i]);
-        cur.pop_back();
-      }
-  };
-  search(search, r, 0, 0.0);
-  auto lead = [&](int f) {
-    auto it = std::find(best.begin(), best.end(), f);
-    if (it == best.end()) return false;
-    best.erase(it);
-    p.radix.push_back(f);
-    return true;
-  };
-  if (three_first) { if (!lead(3)) lead(6); }
-  else if (odd.empty() && !lead(5)) lead(3);
-  p.radix.insert(p.radix.end(), odd.begin(), odd.end());
-  // then by size: the later passes' stores are contiguous
-  for (int f : {5, 3, 6, 4, 2, 8})
-    for (int b : best)
-      if (b == f) p.radix.push_back(f);
-  return p;
-}
-
 // cos and sin of 2 pi k / n in 62 fractional bits.  The first octant's angle
 // 2 pi q / (4n), q <= n/2, from FP64 z_0 and one Newton step of z^(4n) = 1:
 // z = z_0 (1 - (z_0^(4n) - 1)/(4n)), the power by squarings on 62 fractional
@@ -565,7 +493,8 @@ void group_sizes(int nx, int ny, int nz, Group& g) {
 
 // Plans of a group (d.f32 set): an FP32 group's padded lengths (M, Mx, Mz)
 // and energy grid (Me) in FP32, everything else in fixed point.
-void group_plans(Group& g) {
+// PTT_EINVAL where a length has none.
+int group_plans(Group& g) {
   const int n[7] = {g.d.M, g.d.Mx, g.d.nx, g.d.Pu, g.d.Me, g.d.Mz, g.d.nz};
   const bool three[7] = {false, true, false, false, false, true, false};
   const bool padded[7] = {true, true, false, false, true, true, false};
@@ -574,6 +503,14 @@ void group_plans(Group& g) {
     g.hp[i] = g.fx[i] ? make_plan_fx(n[i], three[i]) : make_plan(n[i], three[i]);
   }
   g.hpn = make_plan_fx(g.d.M);
+  bool ok = plan_ok(g.hpn, true);
+  for (int i = 0; i < 7; ++i) ok = ok && plan_ok(g.hp[i], g.fx[i]);
+  if (!ok) {
+    char msg[96];
+    std::snprintf(msg, sizeof(msg), "no transform plan for nx=%d ny=%d nz=%d", g.nx, g.ny, g.nz);
+    set_last_error(msg);
+    return PTT_EINVAL;
+  }
   // threads of the fused x pass.  FP32: the 1024 that 64 registers leave an SM,
   // over the blocks that shared memory leaves it (fewer threads a block have
   // fewer idle in the passes, fewer blocks less of a block's barriers hidden).
@@ -587,6 +524,7 @@ void group_plans(Group& g) {
   } else {
     g.d.xthreads = 256;
   }
+  return PTT_OK;
 }
 
 // Least threads per block of the plan's passes.
@@ -708,9 +646,8 @@ void carve(std::vector<Group>& groups, Carver& cv) {
   }
 }
 
-std::vector<Group> make_groups(const ptt_params* pm, int nmem) {
+int make_groups(const ptt_params* pm, int nmem, std::vector<Group>& groups) {
   std::map<std::tuple<int, int, int, int>, int> idx;
-  std::vector<Group> groups;
   for (int i = 0; i < nmem; ++i) {
     auto key = std::make_tuple(pm[i].nx, pm[i].ny, pm[i].nz, pm[i].precision);
     auto it = idx.find(key);
@@ -723,14 +660,14 @@ std::vector<Group> make_groups(const ptt_params* pm, int nmem) {
       g.d.f32 = (pm[i].precision == PTT_MIXED || pm[i].precision == PTT_MIXED_TC) ? 1 : 0;
       group_sizes(g.nx, g.ny, g.nz, g);
       g.ds = (pm[i].precision == PTT_FP64_DS) ? 1 : 0;
-      group_plans(g);
+      if (const int s = group_plans(g)) return s;
       g.d.ymma = (pm[i].precision == PTT_MIXED_TC) ? 1 : 0;   // requested; carve() checks the shape
       groups.push_back(std::move(g));
       it = idx.find(key);
     }
     groups[it->second].members.push_back(i);
   }
-  return groups;
+  return PTT_OK;
 }
 
 // A context can take one launch per stage over all its groups when they
@@ -805,7 +742,7 @@ int shape_plan(const ptt_params& p, GroupDev& d, std::vector<int4>& tables, size
   g.ny = p.ny;
   g.nz = 1;
   group_sizes(p.nx, p.ny, 1, g);
-  group_plans(g);
+  if (const int sp = group_plans(g)) return sp;
   d = g.d;
   d.nb = 1;
   // columns per block as carve() caps them for one member
@@ -870,7 +807,8 @@ int ptt_workspace_size(const ptt_params* pm, int32_t nmem, size_t* bytes) {
     int s = check_params(pm[i]);
     if (s) return s;
   }
-  std::vector<Group> groups = make_groups(pm, nmem);
+  std::vector<Group> groups;
+  if (const int s = make_groups(pm, nmem, groups)) return s;
   for (Group& g : groups) {
     if (g.d.nz == 1 && (smem_xfused(g.d.Mx, g.d.f32) > 227 * 1024 || smem_spec(g.d.N) > 227 * 1024))
       return PTT_EINVAL;
@@ -989,7 +927,7 @@ int ptt_create(const ptt_params* pm, int32_t nmem, void* d_ws, size_t bytes, voi
   std::unique_ptr<ptt_ctx> c(new (std::nothrow) ptt_ctx());
   if (!c) return PTT_ENOMEM;
   c->prm.assign(pm, pm + nmem);
-  c->groups = make_groups(pm, nmem);
+  if ((s = make_groups(pm, nmem, c->groups))) return s;
   c->stream = (cudaStream_t)stream;
   CK(cudaGetDevice(&c->device));
   Carver cv;

@@ -271,7 +271,7 @@ template <int DIR> struct FxBfly<DIR, 13> : FxBflyOdd<DIR, 13> {};
 // ------------------------------------------------------------ passes
 // One Stockham pass of radix R over nl lines (line l at offset l * ls), in
 // place: the lines go in groups whose butterflies sit in registers, one per
-// thread (fx_mb(R) of radix 2); the block waits between a group's loads
+// thread (fx_mb(R) of radix 2 and 3); the block waits between a group's loads
 // and its stores.  One buffer instead of two: the 3D x pass at 192 points takes
 // 55 KB a block, so several blocks share an SM and one block's barriers and
 // FP64 products run under another's butterflies.  (More butterflies per

@@ -6,10 +6,10 @@
 #include <cuda_runtime.h>
 
 #include "ptt.h"
+#include "ptt_plan.h"
 
 namespace ptt {
 
-constexpr int kMaxStages = 8;    // passes of a plan (n <= 1080: at most 7)
 constexpr int kRing = 1024;       // diagnostics records kept per member
 constexpr int kNumHist = 4;       // SBDF4 history depth
 
@@ -32,8 +32,6 @@ struct FftPlan {
   int pnb[kMaxStages], pst[kMaxStages], pns[kMaxStages];
   unsigned pmb[kMaxStages], pms[kMaxStages];
 };
-// Butterflies of radix R held by a thread in a fixed-point pass.
-__host__ __device__ constexpr int fx_mb(int R) { return R == 2 ? 2 : 1; }
 // Fills the per-pass constants of pl from pl.n, pl.nst and pl.radix.
 void plan_pass_consts(FftPlan& pl);
 
