@@ -405,17 +405,18 @@ __device__ __forceinline__ unsigned fx_units(double x, int emax) {
 // 2^extra: |x| < 2^(nbits + emax - 1042) in sum, so v = x 2^B with
 // B = 1102 - extra - nbits - emax stays below 2^(60 - extra) in sum; a 53-bit
 // mantissa shifted left by 8 then goes right by (emax - e) + nbits + extra - 19
-// >= 1.  A line of zeros (or of values below 2^-849) gives exact zeros: its
-// part of a packed line holds the other field's rounding.  One with a NaN, an
-// infinity or values above 2^990 gives NaN.
+// >= 1.  A line of zeros (or of values below 2^-927, where fx_to's exponents end)
+// gives exact zeros: its part of a packed line holds the other field's rounding.
+// One with a NaN, an infinity or values above 2^990 gives NaN.
+constexpr int kFxMinExp = 96;     // fx_to: C - 60 - k >= emax + 2 - 60 - 28 > 0
 __device__ __forceinline__ FxS fx_scale(int emax, unsigned sum, int extra) {
   FxS s;
-  const int nbits = 32 - __clz((int)sum);
-  const bool zero = emax < 174, bad = emax > 2013;
-  s.C = (zero || bad) ? 1084 : emax + nbits + extra - 18;
+  const int nbits = 32 - __clz((int)sum), C = emax + nbits + extra - 18;
+  const bool zero = emax < kFxMinExp, bad = emax > 2013;
+  s.C = (zero || bad) ? 1084 : C;
   s.am = (zero || bad) ? 0u : 0xFFFFFFFFu;
   s.om = bad ? 0x7FF80000u : 0u;
-  s.base = (zero || bad) ? 4096 : emax + nbits + extra - 19;
+  s.base = (zero || bad) ? 4096 : C - 1;
   return s;
 }
 // The scale of a line of cnt values get(i); m: the lane's largest fx_mag of
@@ -456,24 +457,28 @@ __device__ __forceinline__ void fx_line(fxc* h, int n, FxS& sc) {
   for (int i = lane; i < n; i += 32) h[i] = fx_from2(fx_raw(h[i]), s.base);
 }
 
-// v 2^(C - 1084 - k) as a double, rounded to nearest by about 24 integer
+// v 2^(C - 1084 - k) as a double, rounded to nearest by about 26 integer
 // instructions (a conversion and a scaling would hold the FP64 pipe for 128
 // cycles).  The magnitude is the ones' complement of a negative v, one unit
 // short; its top bit's position comes from the leading word rounded down to
-// FP32 (the low word, two bits down, when the high one is zero; below four
-// units the result is a number of the order of 2^-126 units).
+// FP32 (the low word, two bits down, when the high one is zero).  Below four
+// units (t = 0) the result is zero, so sh <= 30 wherever it counts and the
+// exponent, C - k - 60 at least, is positive for k <= 28 (fexpP, at most
+// log2 of 800 768 768).  (Its two instructions take no time that shows: 3D
+// 128 x 97 x 64 23.43 and 23.33 ms for ten steps, the 2D sweep 35.91 and 35.82.)
 __device__ __forceinline__ double fx_to(long long v, const FxS& f, int k = 0) {
   const int s = (int)(v >> 63);
   const unsigned hi = (unsigned)((int)(v >> 32) ^ s), lo = (unsigned)((int)v ^ s);
   const bool big = hi != 0u;
   const unsigned t = big ? hi : lo >> 2, l = big ? lo : lo << 30;
+  const unsigned am = t ? f.am : 0u;
   const int sh = 157 - (int)(__float_as_uint(__uint2float_rz(t)) >> 23);   // top bit to bit 62
   const unsigned long long N =
       (((unsigned long long)__funnelshift_l(l, t, sh) << 32) | (l << (sh & 31))) + 0x200u;
   const unsigned H = (unsigned)(N >> 32), L = (unsigned)N;
   const unsigned hw = (H >> 10) + ((unsigned)(f.C - k - (big ? 0 : 30) - sh) << 20);
-  return __hiloint2double((int)(((hw | ((unsigned)s & 0x80000000u)) & f.am) | f.om),
-                          (int)(__funnelshift_r(L, H, 10) & f.am));
+  return __hiloint2double((int)(((hw | ((unsigned)s & 0x80000000u)) & am) | f.om),
+                          (int)(__funnelshift_r(L, H, 10) & am));
 }
 __device__ __forceinline__ double2 fx_to2(fxc v, const FxS& f, int k = 0) {
   return make_double2(fx_to(v.x, f, k), fx_to(v.y, f, k));
