@@ -11,6 +11,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "ptt_div.h"
 #include "ptt_fx.cuh"
 #include "ptt_internal.h"
 
@@ -246,25 +247,6 @@ template <int DIR> struct Bfly<DIR, 8> {
     }
   }
 };
-
-// Division by a runtime divisor d through a multiply-high (the method of
-// Granlund and Montgomery, "Division by invariant integers using
-// multiplication", PLDI 1994, in its round-up form): with
-// m = floor((2^32 - 1)/d) + 1 = ceil(2^32/d), floor(x/d) = (x m) >> 32 holds
-// exactly whenever x d < 2^32 (the rounding excess of m contributes less than
-// x/2^32 < 1/d), which covers every index of the transforms here
-// (x < 2^20, d < 2^12).  d = 1 is passed through.
-struct FastDiv {
-  unsigned m;
-  bool one;
-};
-__host__ __device__ __forceinline__ FastDiv fast_div(unsigned d) {
-  FastDiv f;
-  f.one = (d == 1u);
-  f.m = f.one ? 0u : 0xFFFFFFFFu / d + 1u;
-  return f;
-}
-__device__ __forceinline__ unsigned fdiv(unsigned x, FastDiv f) { return f.one ? x : __umulhi(x, f.m); }
 
 // Constants of pass s of a plan, read from the plan (host-computed): the
 // passes divide nothing at run time.

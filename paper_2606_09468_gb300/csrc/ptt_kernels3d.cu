@@ -871,7 +871,9 @@ __global__ void __launch_bounds__(256) k_diag_part3(GroupDev g) {
     double e0 = 0.0, e1 = 0.0;
 #pragma unroll 2
     for (unsigned i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-      const unsigned j = fdiv(i, dKZ), md = i - j * KZ;
+      // i KZ passes 2^32 (192 x 129 x 96: 2.3e10), where fdiv's last modes of some
+      // rows would land in the next row
+      const unsigned j = fdiv_any(i, dKZ, (unsigned)KZ), md = i - j * KZ;
       const double2 a0 = DY[i], a1 = DY[(size_t)Je * KZ + i], a2 = DY[(size_t)2 * Je * KZ + i];
       const double q = fma(a0.x, a0.x, fma(a0.y, a0.y, fma(a1.x, a1.x, fma(a1.y, a1.y,
                            fma(a2.x, a2.x, a2.y * a2.y)))));
