@@ -38,6 +38,15 @@
  *    wavenumber s = q for q < nz/2, q - nz for q > nz/2, k = 2 pi s / lz; the
  *    slot q = nz/2 of the z Nyquist mode is stored and always zero), (re, im).
  *    The m = 0 plane of a real field is Hermitian in q.
+ *  - Range of values: the fixed-point transforms (every transform of PTT_FP64
+ *    and PTT_FP64_DS, the state's and the diagnostics' of the mixed forms) take
+ *    each line of a field, a row of points or a column of coefficients, on a
+ *    scale of its own, 2^-60 of the sum of its moduli.  Within a line, results
+ *    below four such units are zero.  A line whose largest value is below
+ *    2^-927 (8.8e-280) is taken as zero.  One with a NaN, an infinity or a sum
+ *    of moduli of 2^1018 (2.8e306) or more is NaN throughout; in a step the
+ *    products of a line come before their division by the number of points, so
+ *    products from about 2^990 (1e298) on are NaN there.
  *  - Device memory: the caller allocates ONE device workspace of at least
  *    ptt_workspace_size() bytes (256-byte aligned) and owns it; the library
  *    never allocates or frees device memory.  Host pointers are caller-owned

@@ -407,12 +407,14 @@ __device__ __forceinline__ unsigned fx_units(double x, int emax) {
 // mantissa shifted left by 8 then goes right by (emax - e) + nbits + extra - 19
 // >= 1.  A line of zeros (or of values below 2^-927, where fx_to's exponents end)
 // gives exact zeros: its part of a packed line holds the other field's rounding.
-// One with a NaN, an infinity or values above 2^990 gives NaN.
+// One with a NaN or an infinity, or whose results could pass the largest double
+// (a sum of moduli of 2^1018 or more), gives NaN.
+constexpr int kFxMaxC = 2044;     // results below 2^62 units: exponent fields up to C + 2
 constexpr int kFxMinExp = 96;     // fx_to: C - 60 - k >= emax + 2 - 60 - 28 > 0
 __device__ __forceinline__ FxS fx_scale(int emax, unsigned sum, int extra) {
   FxS s;
   const int nbits = 32 - __clz((int)sum), C = emax + nbits + extra - 18;
-  const bool zero = emax < kFxMinExp, bad = emax > 2013;
+  const bool zero = emax < kFxMinExp, bad = emax == 2047 || C > kFxMaxC;
   s.C = (zero || bad) ? 1084 : C;
   s.am = (zero || bad) ? 0u : 0xFFFFFFFFu;
   s.om = bad ? 0x7FF80000u : 0u;
